@@ -128,6 +128,7 @@ void make_devparams(const pic_params* p, long long n, DevParams* d) {
     d->h2shh_f = (float)(d->h2 * d->sh);
     d->hshh_f = (float)(d->h * d->sh);
     d->h6_f = (float)d->h6;
+    d->q_half_f = (float)d->q_half;
     d->spt = p->steps_per_turn;
     const double Dfl = std::floor(d->D);
     d->Di = (int)Dfl;
@@ -292,8 +293,7 @@ int read_status(pic_handle* h) {
 
 // Resets the per-launch synchronisation words of the cooperative window.
 cudaError_t reset_coop(pic_handle* h) {
-    const size_t Np1 = (size_t)h->dp.n_cells + 1;
-    cudaError_t e = cudaMemsetAsync(h->B.Qring, 0, sizeof(unsigned long long) * 3 * 2 * Np1 * pic::kQPad, h->st);
+    cudaError_t e = cudaMemsetAsync(h->B.Qring, 0, sizeof(unsigned long long) * pic::kQSlots * pic::q_slot_words(h->dp.n_cells), h->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->B.notdone, 0, sizeof(int) * 4, h->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->B.bar, 0, sizeof(unsigned int) * 64, h->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->B.K_out, 0, sizeof(long long), h->st);
@@ -456,7 +456,7 @@ int init32(pic_handle* h, const double* r0, const double* v0, int ptr_kind) {
         if (p->periods_once) ALLOC(h->Tin32_alt, N);
     }
     if (poisson) {
-        ALLOC(h->B.Qring, 3 * 2 * Np1 * pic::kQPad);
+        ALLOC(h->B.Qring, pic::kQSlots * pic::q_slot_words(p->n_cells));
         ALLOC(h->Qf, Np1);
         ALLOC(h->nout_f, 1);
         ALLOC(h->Ef, Np1);
@@ -644,7 +644,7 @@ int pic_init(const pic_params* p, int64_t n, const double* r0, const double* v0,
             ALLOC(B.cx, N);
         }
         ALLOC(B.cj, N);
-        ALLOC(B.Qring, 3 * 2 * Np1 * pic::kQPad);
+        ALLOC(B.Qring, pic::kQSlots * pic::q_slot_words(p->n_cells));
         ALLOC(h->Qf, Np1);
         ALLOC(h->nout_f, 1);
         ALLOC(h->Ef, Np1);
@@ -1338,11 +1338,14 @@ cudaError_t batch_upload(pic_batch* b) {
         int cp = b->copies;
         if (h->prm.field_model == PIC_FIELD_POISSON && d.n_blocks > 0) {
             const long long per_block = (h->n + d.n_blocks - 1) / d.n_blocks;
-            while (cp < 4 && pic::window32_batch_smem(h->prm.n_cells, 2 * cp) <= b->smem &&
+            while (cp < 4 && pic::window32_batch_smem(h->prm.n_cells, 2 * cp, b->block, true) <= b->smem &&
                    per_block >= 2048ll * 2 * cp)
                 cp *= 2;
         }
         d.P.hist_copies = cp;
+        d.P.q_cb = pic::q_count_bits(h->n, h->dp.W, d.n_blocks,
+                                     pic::field_in_regs(h->prm.n_cells, b->block) &&
+                                         pic::window32_batch_smem(h->prm.n_cells, cp, b->block, true) <= b->smem);
         d.B = h->B32;
         d.Tin = h->prm.periods_once ? h->Tin32 : nullptr;
         d.T_known = h->prm.periods_once ? 1 : 0;
@@ -1440,8 +1443,9 @@ int batch_configure(pic_batch* b, int block, int bps_want, double power, int cop
                     const BeamTimes* meas = nullptr) {
     if (block < 128 || block > 1024 || (block & 31)) return PIC_ERR_INVALID_ARG;
     if (copies != 1 && copies != 2 && copies != 4) return PIC_ERR_INVALID_ARG;
-    const size_t smem = pic::window32_batch_smem(b->max_cells, copies);
+    size_t smem = pic::window32_batch_smem(b->max_cells, copies, block, false);
     if (smem > 227 * 1024) return PIC_ERR_UNSUPPORTED;
+    const size_t smem_kept = pic::window32_batch_smem(b->max_cells, copies, block, true);
     if (smem > 0) {
         // the larger of the new and the current size, so that the current
         // configuration stays launchable if this one is refused below
@@ -1453,6 +1457,14 @@ int batch_configure(pic_batch* b, int block, int bps_want, double power, int cop
     if (e != cudaSuccess) return map_cuda(e);
     if (bps < 1) return PIC_ERR_UNSUPPORTED;
     if (bps_want > 0 && bps_want < bps) bps = bps_want;
+    // room for the largest mesh's counted charge words where it costs no block
+    if (smem_kept > smem && smem_kept <= pic::kWindowSmemMax) {
+        int bps_kept = 0;
+        e = pic::window32_batch_attr(smem_kept > b->smem ? smem_kept : b->smem);
+        if (e == cudaSuccess) e = pic::window32_batch_occupancy(block, smem_kept, &bps_kept);
+        if (e != cudaSuccess) return map_cuda(e);
+        if (bps_kept >= bps) smem = smem_kept;
+    }
     const long long G = (long long)bps * b->sm_count;
     if (G < b->n) return PIC_ERR_UNSUPPORTED;
     std::vector<double> w(b->n);

@@ -53,8 +53,10 @@ struct DevParams {
     int bar_extra;                     // testing only: arrivals a barrier waits for beyond the grid
     int parity_odd;                    // 1: E = rE(r)/|r| (odd in r, 0 on the axis); 0: E = rE(r)/r
     int hist_copies;                   // copies of each block's charge histogram (window kernel)
+    int q_cb;                          // count bits of the charge words; 0: the cycles end in a grid barrier
     // FP32 form (precision 1): the same quantities rounded once to binary32
     float r_min_f, inv_hr_f, ncells_f, Wf;
+    float q_half_f;
     float h2shh_f, hshh_f, h6_f;       // (h/2) sin(h/(2 eps)), h sin(h/(2 eps)), h/6
     int spt;                           // fine steps per turn of the E = 0 rotation
     int Di;                            // dt/h = Di + Df with Df in [0, 1)
@@ -607,6 +609,12 @@ __device__ __forceinline__ long long global_ns() {
 __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
     unsigned int v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
 

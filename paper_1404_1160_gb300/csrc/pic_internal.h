@@ -56,20 +56,55 @@ struct WinBufs {
     double2* cx;                // RK4: stage positions carried across a cycle
     double* cxr;                // Lawson: (Phi_h y)_R
     double2* traj;              // (Kmax+1) rows of n samples (R, V)
-    unsigned long long* Qring;  // 3 cycles x 2 fields x (n_cells+1), one node per kQPad words
-    int* notdone;               // 3 cycles; [3] trajectory band missed (this launch); [4] band replays
+    unsigned long long* Qring;  // kQSlots cycles of charge words (q_slot_words each)
+    int* notdone;               // [3] trajectory band missed (this launch); [4] band replays
     unsigned int* bar;          // grid barrier: [0] arrivals, [32] released generation
     int* status;                // DEV_* of the launch
     long long* K_out;           // fine steps of the window
 };
 
-// Global charge of a node sits alone on a 128-byte line so the atomics of
-// all blocks spread over many L2 slices.
-constexpr int kQPad = 16;
+// Global charge words of one field cycle ("slot"): two fields of n_cells + 1
+// nodes and one control word.  Four consecutive nodes share a 32-byte sector
+// and every sector has a 128-byte line of its own: the adds and loads of
+// neighbouring lanes travel as one sector request, and the sectors spread
+// over the L2 slices.
+constexpr int kQSlots = 3;
+__host__ __device__ constexpr size_t q_node(int j) { return ((size_t)(j >> 2) << 4) + (size_t)(j & 3); }
+__host__ __device__ constexpr size_t q_field_words(int n_cells) { return ((size_t)(n_cells >> 2) + 1) << 4; }
+__host__ __device__ constexpr size_t q_slot_words(int n_cells) { return 2 * q_field_words(n_cells) + 16; }
+// Whether a block of `block` threads builds the field from the nodes in
+// registers (at most 4 nodes per thread, 31 of every 32 threads, half a
+// block per field) or stages them in shared memory.
+__host__ __device__ constexpr bool field_in_regs(int n_cells, int block) {
+    return (block & 63) == 0 && block <= 1024 && n_cells + 1 <= 4 * 31 * (block >> 6);
+}
+// Count bits of the counted charge words (window_common.cuh) for n particles
+// of W units on n_blocks blocks: the blocks' arrivals below, the node charge
+// (at most n W) above.  0 when both do not fit one 64-bit word, or the launch
+// has no shared memory for the kept words (`kept`); the cycles then end in a
+// grid barrier.
+inline int q_count_bits(long long n, long long W, long long n_blocks, bool kept) {
+    if (!kept) return 0;
+    int cb = 1;
+    while ((1ll << cb) <= n_blocks) ++cb;
+    int qb = 0;
+    while (qb < 63 && (double)n * (double)W >= (double)(1ull << qb)) ++qb;
+    return qb + cb <= 64 ? cb : 0;
+}
 
 enum WindowMode { MODE_PERIODS = 0, MODE_ETD = 1, MODE_FINE = 2 };
 
+// Shared memory (int64 words) behind the field tables of a window: the last
+// complete charge words of both slots (counted form, register build only),
+// or the staged build's scan output.
+__host__ __device__ constexpr size_t cycle_words(int n_cells, int block, bool kept) {
+    return field_in_regs(n_cells, block) ? (kept ? 2 * (2 * ((size_t)n_cells + 1) + 1) : 0) : 2 * ((size_t)n_cells + 1);
+}
+// Dynamic shared memory a window kernel may take beside its static variables.
+constexpr size_t kWindowSmemMax = 227 * 1024 - 1024;
+
 struct WindowLaunch {
+    bool kept = false;        // shared memory for the counted charge words
     int coop_grid = 0, coop_block = 0;
     int hist = 0;             // 0: 32-bit split histograms, 1: 64-bit
     int stage = 0;            // 1: cp.async staging of each warp's next chunk
@@ -127,7 +162,7 @@ struct BeamDesc32 {
     int T_known;
     unsigned long long* t_ns;  // [2]: first start and last end (global timer, ns) of the beam's blocks
 };
-size_t window32_batch_smem(int max_cells, int copies);
+size_t window32_batch_smem(int max_cells, int copies, int block, bool kept);
 cudaError_t window32_batch_attr(size_t smem);
 cudaError_t window32_batch_occupancy(int block, size_t smem, int* blocks_per_sm);
 cudaError_t launch_window32_batch(const BeamDesc32* beams, int n_beams, int grid, int block, size_t smem,

@@ -198,14 +198,13 @@ __global__ void k_moments(DevParams P, WinBufs B, double* part_d, long long* par
 
 // ------------------------------------------------------------- launchers
 
-// Shared memory of the window kernel with `copies` histogram copies (at
-// least two copies' worth: the histogram region doubles as the int64 scan
-// input) and, with staging, two Stage buffers per warp.
-static size_t coop_smem_bytes(int n_cells, int copies, int block, int stage, int slot_words) {
+// Shared memory of the window kernel with `copies` histogram copies and,
+// with staging, two Stage buffers per warp.
+static size_t coop_smem_bytes(int n_cells, int copies, int block, int stage, int slot_words, bool kept = false) {
     const size_t Np1 = (size_t)n_cells + 1;
-    const size_t hc = (size_t)(copies > 2 ? copies : 2);
+    const size_t hc = (size_t)hist_copies_reserved(n_cells, copies, block);
     return (stage ? (size_t)(block / 32) * kStageBytesPerWarp : 0) + 2 * Np1 * sizeof(double2) +
-           hc * 2 * (size_t)slot_words * Np1 * sizeof(unsigned int) + 2 * Np1 * sizeof(long long) +
+           hc * 2 * (size_t)slot_words * Np1 * sizeof(unsigned int) + cycle_words(n_cells, block, kept) * sizeof(long long) +
            Np1 * sizeof(double);
 }
 
@@ -239,7 +238,9 @@ cudaError_t window_prepare(DevParams& P, int block, int blocks_per_sm, int sm_co
     int copies = kHistCopiesMax;
     while (copies > 1 && coop_smem_bytes(P.n_cells, copies, block, L->stage, slot) > limit) copies >>= 1;
     P.hist_copies = copies;
-    L->coop_smem = coop_smem_bytes(P.n_cells, copies, block, L->stage, slot);
+    L->kept = field_in_regs(P.n_cells, block) &&
+              coop_smem_bytes(P.n_cells, copies, block, L->stage, slot, true) <= kWindowSmemMax;
+    L->coop_smem = coop_smem_bytes(P.n_cells, copies, block, L->stage, slot, L->kept);
     int bps = 1 << 30;
     for (int hh = 0; hh < 3; ++hh) {
         void* fn = coop_fn(P.solver, hh, P.xs_fma, L->stage);
@@ -273,6 +274,7 @@ cudaError_t launch_window_coop(const DevParams& P, const WinBufs& B, const Windo
                                const double* Tin) {
     void* fn = coop_fn(P.solver, L.hist, P.xs_fma, L.stage);
     DevParams Pc = P;
+    Pc.q_cb = q_count_bits(P.n, P.W, (long long)L.coop_grid + P.bar_extra, L.kept);
     WinBufs Bc = B;
     void* args[] = {&Pc, &Bc, &mode, &T_known, &n_fine, &Tin};
     cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(L.coop_grid), dim3(L.coop_block), args, L.coop_smem, st);

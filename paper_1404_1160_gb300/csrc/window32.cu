@@ -149,24 +149,6 @@ __device__ __forceinline__ unsigned long long hist32_node(const unsigned int* h,
     return C * (unsigned long long)W - Sj + Sm;
 }
 
-// Adds this block's two histograms to the cycle's global charge; block 0
-// clears the charge of the cycle after.
-__device__ __forceinline__ void flush32(const DevParams& P, const WinBufs32& B, const unsigned int* hist, int cyc,
-                                        int lb) {
-    const int Np1 = P.n_cells + 1;
-    unsigned long long* Qg = B.Qring + (size_t)(cyc % 3) * 2 * Np1 * kQPad;
-    for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
-        const int f = idx >= Np1, j = idx - f * Np1;
-        const unsigned long long v =
-            hist32_node(hist + f * kHist32Words * Np1, Np1, j, P.W, P.hist_copies, 2 * kHist32Words * Np1);
-        if (v) atomicAdd(Qg + (size_t)idx * kQPad, v);
-    }
-    if (lb == 0) {
-        unsigned long long* Qn = B.Qring + (size_t)((cyc + 1) % 3) * 2 * Np1 * kQPad;
-        for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) Qn[(size_t)idx * kQPad] = 0ull;
-    }
-}
-
 // Field tables of one cycle from its global charge: exact int64 trapezoid
 // sums S_j = g_j - g_c, then in binary32 E_j = float(S_j) cq_j with the
 // per-node constant cq_j = q_unit / (2 r_j) (negated left of the axis for
@@ -177,48 +159,78 @@ __device__ __forceinline__ void flush32(const DevParams& P, const WinBufs32& B, 
 // particle by about h dE per stage).  All on the FP32 pipes: on this GPU the
 // FP64 conversion of every node in every block was most of the build.  q is
 // the int64 scan input (2 Np1), g the scan output, reused for E.
-// stop_src (may be null): the not-done count of the cycle, read together with
-// the charge; *s_stop = (count == 0) after the call.
-__device__ void build_fields32(const DevParams& P, const unsigned long long* Qg, long long* q, long long* g,
-                               float2* tab, const float* cq, float* edges, long long* s_warp, long long* s_c,
-                               const int* stop_src = nullptr, int* s_stop = nullptr) {
-    const int Nc = P.n_cells, Np1 = Nc + 1, c = P.c;
-    const float qh = (float)P.q_half;
-    if (stop_src && threadIdx.x == 0) *s_stop = (__ldcg(stop_src) == 0);
-    auto field_at = [&](int j, long long S, long long qj) -> float { return __ll2float_rn(j == c ? qj : S) * cq[j]; };
-    auto emit = [&](int f, int j, float e, float en, long long S) {
-        tab[f * Np1 + j] = make_float2(e, j < Nc ? en - e : 0.0f);
-        // odd reading: the lower edge value carries the sign flip (rE / |R|)
-        if (j == 0) edges[2 * f] = P.parity_odd ? -(__ll2float_rn(S) * qh) : __ll2float_rn(S) * qh;
-        if (j == Nc) edges[2 * f + 1] = __ll2float_rn(S) * qh;
-    };
-    if (field_build_regs_with(P, Qg, s_warp, field_at, emit)) {
-        __syncthreads();
-        return;
-    }
-    // staged build (meshes too large for the register form)
-    for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) q[idx] = (long long)__ldcg(Qg + (size_t)idx * kQPad);
+// `control`: the cycle carries the not-done count; s_stop = (count == 0).
+// One call ends a sweep: the block's histograms into the cycle's words, the
+// table of stage pair 1 (pair = 0) or 2 from the words of all blocks, and the
+// histograms and the sweep's counters cleared for the next sweep.  false: a
+// wait ran out of time.
+static __device__ __forceinline__ void clear_hist32(unsigned int* hist, int words) {
+    // 16-byte stores: the region starts aligned and holds a multiple of four words
+    for (int i = threadIdx.x; i < words / 4; i += blockDim.x) ((uint4*)hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+static __device__ __forceinline__ bool field_cycle32(int cyc, int pair, bool control) {
     __syncthreads();
-    block_exscan_pairs2(q, g, Nc, s_warp);
+    const int Nc = s_cyc.n_cells, Np1 = Nc + 1, c = s_cyc.c, copies = s_cyc.copies;
+    const int hw = kHist32Words * Np1;
+    unsigned int* hist = (unsigned int*)(smem_raw + s_cyc.hist);
+    float2* tab = (float2*)(smem_raw + (pair ? s_cyc.tabB : s_cyc.tabA));
+    float* edges = edges32(pair);
+    const float* cq = (const float*)(smem_raw + s_cyc.node_c);
+    unsigned long long* prev;
+    const unsigned long long* Q = cycle_exchange(cyc, control, &prev, [&](int f, int j) {
+        return hist32_node(hist + f * hw, Np1, j, s_cyc.W, copies, 2 * hw);
+    });
+    if (!Q) return false;
+    auto clear = [&]() {
+        clear_hist32(hist, copies * 2 * hw);
+        if (threadIdx.x == 0) {
+            s_cnt = 0;
+            s_next = 0;
+        }
+    };
+    auto field_at = [&](int j, long long S, long long qj) -> float { return __ll2float_rn(j == c ? qj : S) * cq[j]; };
+    auto edge = [&](int f, int j, long long S) {
+        // odd reading: the lower edge value carries the sign flip (rE / |R|)
+        const float rE = __ll2float_rn(S) * s_cyc.q_half_f;
+        if (j == 0) edges[2 * f] = s_cyc.parity_odd ? -rE : rE;
+        if (j == Nc) edges[2 * f + 1] = rE;
+    };
+    if (field_in_regs(Nc, blockDim.x)) {
+        auto emit = [&](int f, int j, float e, float en, long long S) {
+            tab[f * Np1 + j] = make_float2(e, j < Nc ? en - e : 0.0f);
+            if (j == 0 || j == Nc) edge(f, j, S);
+        };
+        if (!field_build_regs(Q, prev, control, field_at, emit, clear)) return false;
+        __syncthreads();
+        return true;
+    }
+    // staged build (meshes too large for the register form); the grid
+    // barrier has put every thread past its flush, so q may take the histograms
+    long long* q = (long long*)hist;
+    long long* g = (long long*)(smem_raw + s_cyc.g);
+    stage_charge(Q, q, control);
+    __syncthreads();
+    block_exscan_pairs2(q, g, Nc, s_tot);
     if (threadIdx.x < 2) {
-        s_c[threadIdx.x] = g[threadIdx.x * Np1 + c];
-        s_c[2 + threadIdx.x] = q[threadIdx.x * Np1 + c];
+        s_tot[threadIdx.x] = g[threadIdx.x * Np1 + c];
+        s_tot[2 + threadIdx.x] = q[threadIdx.x * Np1 + c];
     }
     __syncthreads();
     float* e = (float*)g;  // E_idx in the slot of g[idx] (float 2 idx), which only this thread reads
     for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
         const int f = idx >= Np1, j = idx - f * Np1;
-        const long long S = g[idx] - s_c[f];
-        if (j == 0) edges[2 * f] = P.parity_odd ? -(__ll2float_rn(S) * qh) : __ll2float_rn(S) * qh;
-        if (j == Nc) edges[2 * f + 1] = __ll2float_rn(S) * qh;
-        e[2 * idx] = field_at(j, S, s_c[2 + f]);
+        const long long S = g[idx] - s_tot[f];
+        if (j == 0 || j == Nc) edge(f, j, S);
+        e[2 * idx] = field_at(j, S, s_tot[2 + f]);
     }
     __syncthreads();
+    clear();
     for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
         const int j = idx >= Np1 ? idx - Np1 : idx;
         tab[idx] = make_float2(e[2 * idx], j < Nc ? e[2 * idx + 2] - e[2 * idx] : 0.0f);
     }
     __syncthreads();
+    return true;
 }
 
 // ------------------------------------------------------------ tracking
@@ -351,36 +363,39 @@ __device__ __forceinline__ unsigned int grp_tr(const Grp32& G, int q) {
 }
 
 // Shared memory of the FP32 window kernel (bytes).
-static size_t coop32_smem_bytes(int n_cells, int copies) {
+static size_t coop32_smem_bytes(int n_cells, int copies, int block, bool kept) {
     const size_t Np1 = (size_t)n_cells + 1;
     return (size_t)copies * 2 * kHist32Words * Np1 * sizeof(unsigned int)  // histograms; also the int64 scan input
-           + 2 * Np1 * sizeof(long long)                  // scan output, then E in FP64
-           + Np1 * sizeof(double)                         // 1/r_j
-           + 4 * Np1 * sizeof(float2);                    // tables of pair 1 and pair 2
+           + 4 * Np1 * sizeof(float2)                     // tables of pair 1 and pair 2
+           + cycle_words(n_cells, block, kept) * sizeof(long long)  // kept charge words, or scan output, then E
+           + Np1 * sizeof(float);                         // field constants
 }
 
 // The window of one beam on blocks lb = 0..nb-1 of its own (the whole grid
 // for a single beam, or a beam's share of a batch).
 __device__ __forceinline__ void window32_coop_body(const DevParams& P, const WinBufs32& B, int mode, int T_known,
-                                                   long long n_fine, const CTime* __restrict__ Tin, int lb, int nb,
-                                                   unsigned char* smem_raw) {
+                                                   long long n_fine, const CTime* __restrict__ Tin, int lb, int nb) {
     const int Nc = P.n_cells, Np1 = Nc + 1;
     const int hw = kHist32Words * Np1;
     const int copies = P.hist_copies;
     unsigned int* hist = (unsigned int*)smem_raw;  // copies x 2 fields x hw words
-    long long* g = (long long*)(hist + copies * 2 * hw);  // 2 Np1
-    float* cq = (float*)(g + 2 * Np1);              // Np1 (in a slot of Np1 doubles)
-    float2* tabA = (float2*)((double*)(g + 2 * Np1) + Np1);  // 2 Np1: fields of R1, R3
+    float2* tabA = (float2*)(hist + copies * 2 * hw);  // 2 Np1: fields of R1, R3
     float2* tabB = tabA + 2 * Np1;                  // 2 Np1: fields of R2, R4
-    __shared__ float s_edA[4], s_edB[4];
-    __shared__ long long s_warp[64], s_c[4];
-    __shared__ int s_ok, s_cnt, s_stop, s_next;
-
+    // scan output of the staged build (2 Np1), or the last complete charge
+    // words of the two slots where the field is built in registers
+    long long* g = (long long*)(tabB + 2 * Np1);
+    unsigned long long* prev = (unsigned long long*)g;  // 2 x (2 Np1 + 1)
+    float* cq = (float*)(g + cycle_words(Nc, blockDim.x, P.q_cb > 0));  // Np1
+    if (P.q_cb)
+        for (int i = threadIdx.x; i < 2 * (2 * Np1 + 1); i += blockDim.x) prev[i] = 0ull;
+    clear_hist32(hist, copies * 2 * hw);
+    auto off = [&](const void* p) { return (int)((const unsigned char*)p - smem_raw); };
+    cycle_setup(P, B.Qring, B.bar, B.status, nb, lb, off(hist), off(tabA), off(tabB), off(g), off(cq));
     for (int j = threadIdx.x; j < Np1; j += blockDim.x)
         cq[j] = (j == P.c) ? (P.parity_odd ? 0.0f : (float)(P.q_unit * P.inv_hr))
                            : (float)(((P.parity_odd && j < P.c) ? -P.q_half : P.q_half) / (P.r_min + (double)j * P.hr));
 
-    const bool detect_only = mode == MODE_PERIODS, fine_only = mode == MODE_FINE;
+    const bool detect_only = mode == MODE_PERIODS, fine_only = mode == MODE_FINE, track = !fine_only;
     const long long n = P.n, ld = B.ld;
     const int lane = threadIdx.x & 31;
     // Work unit: a group of 128 consecutive storage slots, lane l holding
@@ -403,11 +418,15 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
         if (fine_only) return (k & 1) ? B.traj : B.y;
         return k == 0 ? B.y : B.traj + (size_t)(k - 1) * ld;
     };
-    const long long tid = (long long)lb * blockDim.x + threadIdx.x;
-    const long long nthreads = (long long)nb * blockDim.x;
+    // Every slot is read and written by its own block only (set-up, sweeps and
+    // landing alike): blocks exchange nothing but the charge words.
+    const int my_slots = (int)my_groups * kGroup;
+    auto slot_of = [&](int s) -> long long { return ((long long)lb + (long long)(s / kGroup) * nb) * kGroup + s % kGroup; };
 
     if (!fine_only) {
-        for (long long i = tid; i < n; i += nthreads) {
+        for (int s = threadIdx.x; s < my_slots; s += blockDim.x) {
+            const long long i = slot_of(s);
+            if (i >= n) break;
             if (T_known) {
                 int flags = 0;
                 const Decomp32 d = resolve32(P, Tin[i], true, flags);
@@ -421,7 +440,6 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
         }
     }
 
-    unsigned int gen = 0;
     int cyc = 0;
     int K = 0;
     // lane l deposits into copy l mod copies: the lanes of a warp hold
@@ -429,17 +447,17 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
     unsigned int* histA = hist + (lane & (copies - 1)) * 2 * hw;
     unsigned int* histB = histA + hw;
 
-    for (int k = 0;; ++k) {
-        // ---- sweep A(k): finish step k-1 (write row k), sample k, deposit stage pair 1 of step k
-        for (int idx = threadIdx.x; idx < copies * 2 * hw; idx += blockDim.x) hist[idx] = 0u;
-        if (threadIdx.x == 0) {
-            s_cnt = 0;
-            s_next = 0;
-        }
-        __syncthreads();
-        const bool last_fine = fine_only && k == n_fine;
+    __syncthreads();
+
+    // half-steps: sweep A(k), cycle, sweep B(k), cycle (one copy of the cycle's code)
+    for (int hs = 0;; ++hs) {
+        const int k = hs >> 1;
         const float2 rb = P.rot[rot_index(P, 2ll * k)];      // Phi(t_k)
         const float2 rp = P.rot[rot_index(P, 2ll * k + 1)];  // Phi(t_k + h/2)
+        Grp32 cur;
+        if (!(hs & 1)) {
+        // ---- sweep A(k): finish step k-1 (write row k), sample k, deposit stage pair 1 of step k
+        const bool last_fine = fine_only && k == n_fine;
         float2 ra = rb, rm = rp, rk2 = rb;
         if (k > 0) {
             ra = P.rot[rot_index(P, 2ll * k - 2)];  // Phi(t_{k-1})
@@ -449,9 +467,7 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
         const float2* src = row(k > 0 ? k - 1 : 0);
         float2* dst = last_fine ? B.y : row(k);
         const float2* src2 = k > 1 ? row(k - 2) : nullptr;
-        const bool track = !fine_only;
         unsigned int cnt = 0;
-        Grp32 cur;
         for (long long gi = grab(); gi >= 0; gi = grab()) {
             const long long base = gi * kGroup + lane * kG;
             load_grp(src, B.tr, B.ce, base, track, k > 0, cur);
@@ -466,7 +482,7 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
                     const float e1 = grp_e(cur, 2 * q), e3 = grp_e(cur, 2 * q + 1);
                     float e2, e4;
                     locate_gather2(P, lawson32_R2(P, R3, e1), lawson32_R4(P, rb, zR, zV, e3), tabB, tabB + Np1,
-                                   s_edB, e2, e4);
+                                   edges32(1), e2, e4);
                     const float Vold = rot_V(ra, zR, zV);
                     lawson32_update(P, ra, rm, rb, e1, e2, e3, e4, zR, zV);
                     if (track && valid) {
@@ -501,23 +517,8 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
             cnt = __reduce_add_sync(0xffffffffu, cnt);
             if (lane == 0 && cnt) atomicAdd(&s_cnt, (int)cnt);
         }
-        __syncthreads();
-        flush32(P, B, hist, cyc, lb);
-        if (lb == 0 && threadIdx.x == 0) B.notdone[(k + 1) % 3] = 0;
-        if (threadIdx.x == 0 && s_cnt) atomicAdd(&B.notdone[k % 3], s_cnt);
-        if (!grid_sync(P, B.bar, gen, B.status, &s_ok, (unsigned int)nb)) return;
-        build_fields32(P, B.Qring + (size_t)(cyc % 3) * 2 * Np1 * kQPad, (long long*)hist, g, tabA, cq, s_edA,
-                       s_warp, s_c, track ? &B.notdone[k % 3] : nullptr, &s_stop);
-        if (track && s_stop) {
-            K = k;
-            break;
-        }
-        ++cyc;
-
+        } else {
         // ---- sweep B(k): gather pair 1 of step k, deposit stage pair 2
-        for (int idx = threadIdx.x; idx < copies * 2 * hw; idx += blockDim.x) hist[idx] = 0u;
-        if (threadIdx.x == 0) s_next = 0;
-        __syncthreads();
         const float2 rq = P.rot[rot_index(P, 2ll * k + 2)];  // Phi(t_k + h)
         const float2* srcB = row(k);
         for (long long gi = grab(); gi >= 0; gi = grab()) {
@@ -530,7 +531,7 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
                 const float zR = grp_get(cur, 2 * q), zV = grp_get(cur, 2 * q + 1);
                 const float R3 = rot_R(rp, zR, zV);
                 float e1, e3;
-                locate_gather2(P, rot_R(rb, zR, zV), R3, tabA, tabA + Np1, s_edA, e1, e3);
+                locate_gather2(P, rot_R(rb, zR, zV), R3, tabA, tabA + Np1, edges32(0), e1, e3);
                 eo[2 * q] = e1;
                 eo[2 * q + 1] = e3;
                 locate_deposit2(P, lawson32_R2(P, R3, e1), lawson32_R4(P, rq, zR, zV, e3), histA, histB, Np1, valid);
@@ -540,19 +541,22 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
             o[1] = make_float4(eo[4], eo[5], eo[6], eo[7]);
         }
         rev = !rev;
-        __syncthreads();
-        flush32(P, B, hist, cyc, lb);
-        if (!grid_sync(P, B.bar, gen, B.status, &s_ok, (unsigned int)nb)) return;
-        build_fields32(P, B.Qring + (size_t)(cyc % 3) * 2 * Np1 * kQPad, (long long*)hist, g, tabB, cq, s_edB,
-                       s_warp, s_c);
-        ++cyc;
+        }
+        const bool control = !(hs & 1) && track;
+        if (!field_cycle32(cyc++, hs & 1, control)) return;
+        if (control && s_stop) {
+            K = k;
+            break;
+        }
     }
 
     if (lb == 0 && threadIdx.x == 0 && !fine_only) *B.K_out = K;
     if (mode != MODE_ETD) return;
 
     // ---- landing (step 3) and extrapolation (step 4); row k holds z_k
-    for (long long i = tid; i < n; i += nthreads) {
+    for (int s = threadIdx.x; s < my_slots; s += blockDim.x) {
+        const long long i = slot_of(s);
+        if (i >= n) break;
         const CTime o = B.o[i], T = B.T[i];
         const int N = B.N[i];
         float yv[2][2];
@@ -583,8 +587,7 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
 
 __global__ void __launch_bounds__(kW32Threads, 1) k_window32_coop(DevParams P, WinBufs32 B, int mode, int T_known,
                                                                   long long n_fine, const CTime* __restrict__ Tin) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    window32_coop_body(P, B, mode, T_known, n_fine, Tin, blockIdx.x, gridDim.x, smem_raw);
+    window32_coop_body(P, B, mode, T_known, n_fine, Tin, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------- per-particle window (analytic E)
@@ -819,7 +822,6 @@ __global__ void __launch_bounds__(256) k_window32_local(DevParams P, WinBufs32 B
 // and runs that beam's window on the beam's own blocks (its barriers count
 // only them).  Beams never wait for each other.
 __global__ void __launch_bounds__(kW32Threads, 1) k_window32_batch(const BeamDesc32* __restrict__ beams, int n_beams) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ BeamDesc32 D;
     __shared__ int s_beam;
     if (threadIdx.x == 0) {
@@ -840,7 +842,7 @@ __global__ void __launch_bounds__(kW32Threads, 1) k_window32_batch(const BeamDes
     __syncthreads();
     const int lb = (int)blockIdx.x - D.first_block;
     if (threadIdx.x == 0) atomicMin(&D.t_ns[0], (unsigned long long)global_ns());
-    if (D.coop) window32_coop_body(D.P, D.B, MODE_ETD, D.T_known, 0, D.Tin, lb, D.n_blocks, smem_raw);
+    if (D.coop) window32_coop_body(D.P, D.B, MODE_ETD, D.T_known, 0, D.Tin, lb, D.n_blocks);
     else if (D.P.field == 1) window32_local_body<1>(D.P, D.B, MODE_ETD, D.T_known, 1, D.Tin, lb, D.n_blocks);
     else window32_local_body<2>(D.P, D.B, MODE_ETD, D.T_known, 1, D.Tin, lb, D.n_blocks);
     __syncthreads();  // the block's last thread is done before its end time
@@ -852,10 +854,9 @@ __global__ void k_batch_reset(const BeamDesc32* __restrict__ beams, int n_beams)
     if (b >= n_beams) return;
     const BeamDesc32& D = beams[b];
     if (D.coop) {
-        const size_t q = (size_t)3 * 2 * (D.P.n_cells + 1) * kQPad;
+        const size_t q = (size_t)kQSlots * q_slot_words(D.P.n_cells);
         for (size_t i = threadIdx.x; i < q; i += blockDim.x) D.B.Qring[i] = 0ull;
         for (int i = threadIdx.x; i < 64; i += blockDim.x) D.B.bar[i] = 0u;
-        if (threadIdx.x < 3) D.B.notdone[threadIdx.x] = 0;
     }
     if (threadIdx.x == 0) {
         *D.B.K_out = 0;
@@ -870,7 +871,9 @@ __global__ void k_batch_status(const BeamDesc32* __restrict__ beams, int n_beams
         out[b] = *beams[b].B.status;
 }
 
-size_t window32_batch_smem(int max_cells, int copies) { return max_cells > 0 ? coop32_smem_bytes(max_cells, copies) : 0; }
+size_t window32_batch_smem(int max_cells, int copies, int block, bool kept) {
+    return max_cells > 0 ? coop32_smem_bytes(max_cells, copies, block, kept) : 0;
+}
 
 cudaError_t window32_batch_attr(size_t smem) {
     return cudaFuncSetAttribute(k_window32_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -970,10 +973,11 @@ cudaError_t window32_prepare(DevParams& P, int block, int blocks_per_sm, int sm_
     // deposits enough positions per cycle for same-cell conflicts to matter
     int copies = kHist32CopiesMax;
     const long long per_block_est = P.n / (sm_count > 0 ? sm_count : 1);
-    while (copies > 1 && (coop32_smem_bytes(P.n_cells, copies) > 200 * 1024 || per_block_est < 64ll * copies * 32))
+    while (copies > 1 && (coop32_smem_bytes(P.n_cells, copies, block, false) > 200 * 1024 || per_block_est < 64ll * copies * 32))
         copies >>= 1;
     P.hist_copies = copies;
-    L->coop_smem = coop32_smem_bytes(P.n_cells, copies);
+    L->kept = field_in_regs(P.n_cells, block) && coop32_smem_bytes(P.n_cells, copies, block, true) <= kWindowSmemMax;
+    L->coop_smem = coop32_smem_bytes(P.n_cells, copies, block, L->kept);
     L->hist = 0;
     L->stage = 0;
     if (L->coop_smem > 227 * 1024) return cudaErrorNotSupported;
@@ -1005,6 +1009,7 @@ cudaError_t launch_window32_coop(const DevParams& P, const WinBufs32& B, const W
                                  int T_known, long long n_fine, cudaStream_t st, long long* launches,
                                  const CTime* Tin) {
     DevParams Pc = P;
+    Pc.q_cb = q_count_bits(P.n, P.W, (long long)L.coop_grid + P.bar_extra, L.kept);
     WinBufs32 Bc = B;
     void* args[] = {&Pc, &Bc, &mode, &T_known, &n_fine, &Tin};
     cudaError_t e = cudaLaunchCooperativeKernel((void*)k_window32_coop, dim3(L.coop_grid), dim3(L.coop_block), args,

@@ -18,10 +18,10 @@
 // (2,4).  One fine step is therefore two field cycles:
 //   sweep: gather previous pair, advance, deposit the next pair into a
 //          shared-memory int64 histogram per block;
-//   flush the histograms with global int64 atomics; grid barrier;
+//   add the histograms to the cycle's global charge words and wait until
+//   every block has (window_common.cuh);
 //   every block scans the mesh charge (block-wide int64 scan) into its own
 //   shared-memory field table.
-// Histogram sets rotate over three buffers so one barrier per cycle suffices.
 #pragma once
 
 #include "pic_internal.h"
@@ -47,6 +47,12 @@ struct Hist {
 };
 // 32-bit words per node that the shared-memory layout reserves
 __host__ __device__ constexpr int hist_slot_words(int hist) { return hist == 2 ? 4 : 3; }
+
+// histogram copies that the layout reserves: the staged field build uses the
+// region as its int64 scan input, which takes two copies' words
+__host__ __device__ constexpr int hist_copies_reserved(int n_cells, int copies, int block) {
+    return copies < 2 && !field_in_regs(n_cells, block) ? 2 : copies;
+}
 
 template <int HIST>
 __device__ __forceinline__ void deposit_cell(unsigned int* h, int Np1, const Cell& c, long long W) {
@@ -113,61 +119,77 @@ __device__ __forceinline__ unsigned long long hist_node(const unsigned int* h, i
 // Field tables of one cycle (two fields) from the cycle's global charge:
 // trapezoid integral from r = 0 (S_j = g_j - g_c), E_j = S_j q_unit/2 * (1/r_j),
 // E_c = Q_c q_unit / h_r, then (E_j, (E_{j+1}-E_j)/W) per cell.
-// stop_src (may be null): the not-done count of the cycle, read together with
-// the charge; *s_stop = (count == 0) after the call.
-static __device__ void build_fields(const DevParams& P, const unsigned long long* Qg, long long* q, long long* g,
-                             double2* tab, const double* inv_r, double* edges, long long* s_warp,
-                             const int* stop_src = nullptr, int* s_stop = nullptr) {
-    const int Nc = P.n_cells, Np1 = Nc + 1, c = P.c;
-    if (stop_src && threadIdx.x == 0) *s_stop = (__ldcg(stop_src) == 0);
-    auto emit = [&](int f, int j, double e, double en, long long S) {
-        double sl = 0.0;
-        if (j < Nc) {
-            const double d = en - e;
-            // d / W: exponent shift when the result stays normal (exact), else multiply
-            const int ex = (int)((__double_as_longlong(d) >> 52) & 0x7ff);
-            sl = (ex > P.log2W + 1 && ex < 0x7ff) ? scale_pow2(d, -P.log2W) : d * P.invW;
+// `control`: the cycle carries the not-done count; s_stop = (count == 0).
+// One call ends a sweep: the block's histograms into the cycle's words, the
+// table from the words of all blocks, and the histograms and the sweep's
+// counters cleared for the next sweep.  false: a wait ran out of time.
+template <int HIST>
+static __device__ __forceinline__ bool field_cycle(int cyc, bool control) {
+    __syncthreads();
+    const int Nc = s_cyc.n_cells, Np1 = Nc + 1, c = s_cyc.c, copies = s_cyc.copies;
+    const int words = Hist<HIST>::kWordsPerNode * Np1;
+    unsigned int* hist = (unsigned int*)(smem_raw + s_cyc.hist);
+    double2* tab = (double2*)(smem_raw + s_cyc.tabA);
+    const double* inv_r = (const double*)(smem_raw + s_cyc.node_c);
+    unsigned long long* prev;
+    const unsigned long long* Q = cycle_exchange(cyc, control, &prev, [&](int f, int j) {
+        return hist_node<HIST>(hist + f * words, Np1, j, s_cyc.W, 2 * words, copies);
+    });
+    if (!Q) return false;
+    auto clear = [&]() {
+        for (int i = threadIdx.x; i < copies * 2 * words; i += blockDim.x) hist[i] = 0u;
+        if (threadIdx.x == 0) {
+            s_cnt = 0;
+            s_next = 0;
         }
-        tab[f * Np1 + j] = make_double2(e, sl);
+    };
+    auto field_at = [&](int j, long long S, long long qj) -> double {
+        if (j == c) return s_cyc.parity_odd ? 0.0 : (i64_to_double(qj) * s_cyc.q_unit) * s_cyc.inv_hr;
+        const double e = (i64_to_double(S) * s_cyc.q_half) * inv_r[j];
+        return (s_cyc.parity_odd && j < c) ? -e : e;  // odd reading: rE / |r|
+    };
+    auto slope = [&](double d) -> double {
+        // d / W: exponent shift when the result stays normal (exact), else multiply
+        const int ex = (int)((__double_as_longlong(d) >> 52) & 0x7ff);
+        return (ex > s_cyc.log2W + 1 && ex < 0x7ff) ? scale_pow2(d, -s_cyc.log2W) : d * s_cyc.invW;
+    };
+    auto edge = [&](int f, int j, long long S) {
         // the off-mesh gather divides the edge rE by R: the odd reading
         // (rE / |R|) carries the sign flip in the lower edge value
-        if (j == 0) edges[2 * f] = P.parity_odd ? -(i64_to_double(S) * P.q_half) : i64_to_double(S) * P.q_half;
-        if (j == Nc) edges[2 * f + 1] = i64_to_double(S) * P.q_half;
+        const double rE = i64_to_double(S) * s_cyc.q_half;
+        if (j == 0) s_cyc.edges[2 * f] = s_cyc.parity_odd ? -rE : rE;
+        if (j == Nc) s_cyc.edges[2 * f + 1] = rE;
     };
-    if (field_build_regs(P, Qg, inv_r, s_warp, emit)) {
+    if (field_in_regs(Nc, blockDim.x)) {
+        auto emit = [&](int f, int j, double e, double en, long long S) {
+            tab[f * Np1 + j] = make_double2(e, j < Nc ? slope(en - e) : 0.0);
+            if (j == 0 || j == Nc) edge(f, j, S);
+        };
+        if (!field_build_regs(Q, prev, control, field_at, emit, clear)) return false;
         __syncthreads();
-        return;
+        return true;
     }
-    // staged build (meshes too large for the register form)
-    for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) q[idx] = (long long)__ldcg(Qg + (size_t)idx * kQPad);
+    // staged build (meshes too large for the register form); the grid
+    // barrier has put every thread past its flush, so q may take the histograms
+    long long* q = (long long*)hist;
+    long long* g = (long long*)(smem_raw + s_cyc.g);
+    stage_charge(Q, q, control);
     __syncthreads();
-    block_exscan_pairs2(q, g, Nc, s_warp);
+    block_exscan_pairs2(q, g, Nc, s_tot);
     for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
         const int f = idx >= Np1, j = idx - f * Np1;
         const long long S = g[idx] - g[f * Np1 + c];
-        // int64 -> double exactly as (double)S, on the integer pipe
-        const double Sd = i64_to_double(S);
-        double e;
-        if (j == c) e = P.parity_odd ? 0.0 : (i64_to_double(q[f * Np1 + c]) * P.q_unit) * P.inv_hr;
-        else e = (Sd * P.q_half) * inv_r[j];
-        if (P.parity_odd && j < c) e = -e;
-        tab[idx].x = e;
-        if (j == 0) edges[2 * f] = P.parity_odd ? -(Sd * P.q_half) : Sd * P.q_half;
-        if (j == Nc) edges[2 * f + 1] = Sd * P.q_half;
+        tab[idx].x = field_at(j, S, q[f * Np1 + c]);
+        if (j == 0 || j == Nc) edge(f, j, S);
     }
     __syncthreads();
+    clear();
     for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
         const int f = idx >= Np1, j = idx - f * Np1;
-        double sl = 0.0;
-        if (j < Nc) {
-            const double d = tab[idx + 1].x - tab[idx].x;
-            // d / W: exponent shift when the result stays normal (exact), else multiply
-            const int ex = (int)((__double_as_longlong(d) >> 52) & 0x7ff);
-            sl = (ex > P.log2W + 1 && ex < 0x7ff) ? scale_pow2(d, -P.log2W) : d * P.invW;
-        }
-        tab[idx].y = sl;
+        tab[idx].y = j < Nc ? slope(tab[idx + 1].x - tab[idx].x) : 0.0;
     }
     __syncthreads();
+    return true;
 }
 
 // Period tracking of one particle at sample k (k >= 1), V_{k-1} = Vold,
@@ -238,24 +260,6 @@ __device__ __forceinline__ bool band_holds(int x, int k, int band_m) {
 
 // ------------------------------------------------ cooperative Poisson window
 
-// Flushes this block's two histograms into the cycle's global charge and
-// (block 0) clears the charge buffer of the next cycle.
-template <int HIST>
-__device__ __forceinline__ void flush_hist(const DevParams& P, const WinBufs& B, const unsigned int* hist, int cyc) {
-    const int Np1 = P.n_cells + 1;
-    const int words = Hist<HIST>::kWordsPerNode * Np1;
-    unsigned long long* Qg = B.Qring + (size_t)(cyc % 3) * 2 * Np1 * kQPad;
-    for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
-        const int f = idx >= Np1, j = idx - f * Np1;
-        const unsigned long long v = hist_node<HIST>(hist + f * words, Np1, j, P.W, 2 * words, P.hist_copies);
-        if (v) atomicAdd(Qg + (size_t)idx * kQPad, v);
-    }
-    if (blockIdx.x == 0) {
-        unsigned long long* Qn = B.Qring + (size_t)((cyc + 1) % 3) * 2 * Np1 * kQPad;
-        for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) Qn[(size_t)idx * kQPad] = 0ull;
-    }
-}
-
 // One chunk (32 particles) of window state in shared memory; lane l owns
 // entry l of every array, so no warp synchronisation is needed.
 struct Stage {
@@ -320,24 +324,27 @@ __device__ __forceinline__ ChunkIn read_stage(const Stage* s, int lane) {
 template <int SOLVER, int HIST, int POW2, int STAGE>
 __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, WinBufs B, int mode, int T_known,
                                                                 long long n_fine, const double* __restrict__ Tin) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
     const int Nc = P.n_cells, Np1 = Nc + 1;
     const int words = Hist<HIST>::kWordsPerNode * Np1;   // 32-bit words per field histogram
     const int copies = P.hist_copies;
     Stage* stage = (Stage*)smem_raw;                      // STAGE: 2 per warp
     double2* tab = (double2*)(smem_raw + (STAGE ? (blockDim.x >> 5) * kStageBytesPerWarp : 0));  // 2 Np1
-    unsigned int* hist = (unsigned int*)(tab + 2 * Np1);  // copies x 2 fields x words (also the scan input)
-    long long* g = (long long*)(hist + (copies > 2 ? copies : 2) * 2 * hist_slot_words(HIST) * Np1);  // 2 Np1
-    double* inv_r = (double*)(g + 2 * Np1);               // Np1
-    __shared__ double s_edges[4];
-    __shared__ long long s_warp[64];
-    __shared__ int s_ok, s_cnt, s_stop, s_next;
-
+    unsigned int* hist = (unsigned int*)(tab + 2 * Np1);  // copies x 2 fields x words (staged build: also the scan input)
+    long long* g = (long long*)(hist + hist_copies_reserved(Nc, copies, blockDim.x) * 2 * hist_slot_words(HIST) * Np1);  // 2 Np1
+    double* inv_r = (double*)(g + cycle_words(Nc, blockDim.x, P.q_cb > 0));  // Np1
+    // the region of g holds the last complete charge words of the two slots
+    // instead where the field is built in registers
+    unsigned long long* prev = (unsigned long long*)g;  // 2 x (2 Np1 + 1)
+    if (P.q_cb)
+        for (int i = threadIdx.x; i < 2 * (2 * Np1 + 1); i += blockDim.x) prev[i] = 0ull;
+    for (int i = threadIdx.x; i < copies * 2 * words; i += blockDim.x) hist[i] = 0u;
+    auto off = [&](const void* p) { return (int)((const unsigned char*)p - smem_raw); };
+    cycle_setup(P, B.Qring, B.bar, B.status, gridDim.x, blockIdx.x, off(hist), off(tab), 0, off(g), off(inv_r));
     for (int j = threadIdx.x; j < Np1; j += blockDim.x)
         inv_r[j] = (j == P.c) ? 0.0 : 1.0 / (P.r_min + (double)j * P.hr);
 
     const bool detect_only = mode == MODE_PERIODS, fine_only = mode == MODE_FINE;
-    const long long n = P.n;
+    const unsigned int n = (unsigned int)P.n;  // below 2^31
     // Work unit: a chunk of 32 consecutive storage slots (phase-space
     // neighbours after the sort).  Block b owns the chunks c = b (mod grid),
     // so every block sees all phases (the sign changes of V spread evenly
@@ -345,25 +352,23 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     // the block, warps take the block's chunks dynamically from a shared
     // counter, so they finish a sweep together.
     const int lane = threadIdx.x & 31;
-    const long long n_chunks = (n + 31) / 32;
+    const unsigned int n_chunks = (n + 31) / 32;
     // lane l deposits into copy l mod copies (the lanes of a warp hold
     // phase-space neighbours, which mostly share a cell)
     unsigned int* const my_hist = hist + ((threadIdx.x & 31) % copies) * 2 * words;
     Stage* const my_stage = stage + 2 * (threadIdx.x >> 5);
-    const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
-    const long long g_warp = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-    const long long stride = n_warps * 32;  // static mapping (init and landing)
-    const long long i0 = g_warp * 32 + lane;
+    const unsigned int g_warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const unsigned int stride = gridDim.x * (blockDim.x & ~31u);  // static mapping (init and landing)
+    const unsigned int i0 = g_warp * 32 + lane;
     // next chunk of this block for this warp (warp-uniform)
-    auto grab = [&]() -> long long {
-        int m = 0;
+    auto grab = [&]() -> unsigned int {
+        unsigned int m = 0;
         if (lane == 0) m = atomicAdd(&s_next, 1);
         m = __shfl_sync(0xffffffffu, m, 0);
-        return (long long)blockIdx.x + (long long)m * gridDim.x;
+        return blockIdx.x + m * gridDim.x;
     };
     const double ie = P.inv_eps, mie = P.mie;
     const long long W = P.W;
-    unsigned int gen = 0;
     int cyc = 0;
     int K = 0;
     __shared__ int s_miss;
@@ -374,7 +379,7 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     for (int attempt = 0;; ++attempt) {
     const bool band = band_ok && attempt == 0;
     if (!fine_only) {
-        for (long long i = i0; i < n; i += stride) {
+        for (unsigned int i = i0; i < n; i += stride) {
             if (T_known) {
                 Track s;
                 s.flags = 0;
@@ -390,27 +395,25 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
         }
     }
 
-    for (int k = 0;; ++k) {
+    __syncthreads();
+    // half-steps: sweep A(k), cycle, sweep B(k), cycle (one copy of the cycle's code)
+    for (int hs = 0;; ++hs) {
+        const int k = hs >> 1;
+        if (!(hs & 1)) {
         // ---- sweep A(k): finish step k-1, sample k, deposit stage pair 1 of step k
-        for (int idx = threadIdx.x; idx < copies * 2 * words; idx += blockDim.x) hist[idx] = 0u;
-        if (threadIdx.x == 0) {
-            s_cnt = 0;
-            s_next = 0;
-        }
-        __syncthreads();
         const bool last_fine = fine_only && k == n_fine;
         const bool k0 = k == 0;
         unsigned int cnt = 0;
         int cur = 0;
-        long long c = grab();
+        unsigned int c = grab();
         if (STAGE) {
             if (c < n_chunks && c * 32 + lane < n) prefetch_chunk<SOLVER>(B, c * 32 + lane, true, fine_only, k0, my_stage, lane);
             cp_async_commit();
         }
         // warp-uniform trip count: lanes past the end run with an empty cell
         for (; c < n_chunks; cur ^= 1) {
-            const long long cn = grab();
-            const long long i = c * 32 + lane;
+            const unsigned int cn = grab();
+            const unsigned int i = c * 32 + lane;
             const bool valid = i < n;
             ChunkIn in;
             if (STAGE) {
@@ -425,8 +428,8 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
             double R = valid ? in.y.x : 0.0, V = valid ? in.y.y : 0.0;
             if (!valid) {
             } else if (k > 0) {
-                const double ea = mesh_gather(tab, s_edges[0], s_edges[1], in.cj.x, in.ca.x);
-                const double eb = mesh_gather(tab + Np1, s_edges[2], s_edges[3], in.cj.y, in.ca.y);
+                const double ea = mesh_gather(tab, s_cyc.edges[0], s_cyc.edges[1], in.cj.x, in.ca.x);
+                const double eb = mesh_gather(tab + Np1, s_cyc.edges[2], s_cyc.edges[3], in.cj.y, in.ca.y);
                 double Rn, Vn;
                 if (SOLVER == 1) {
                     // ce = (e1, e3), ea = e2, eb = e4, cx.x = (Phi_h y)_R
@@ -491,32 +494,17 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
             cnt = __reduce_add_sync(0xffffffffu, cnt);
             if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(&s_cnt, (int)cnt);
         }
-        __syncthreads();
-        flush_hist<HIST>(P, B, hist, cyc);
-        if (blockIdx.x == 0 && threadIdx.x == 0) B.notdone[(k + 1) % 3] = 0;
-        if (threadIdx.x == 0 && s_cnt) atomicAdd(&B.notdone[k % 3], s_cnt);
-        if (!grid_sync(P, B.bar, gen, B.status, &s_ok, gridDim.x)) return;
-        build_fields(P, B.Qring + (size_t)(cyc % 3) * 2 * Np1 * kQPad, (long long*)hist, g, tab, inv_r, s_edges, s_warp,
-                     fine_only ? nullptr : &B.notdone[k % 3], &s_stop);
-        if (!fine_only && s_stop) {
-            K = k;
-            break;
-        }
-        ++cyc;
-
+        } else {
         // ---- sweep B(k): gather pair 1, deposit stage pair 2
-        for (int idx = threadIdx.x; idx < copies * 2 * words; idx += blockDim.x) hist[idx] = 0u;
-        if (threadIdx.x == 0) s_next = 0;
-        __syncthreads();
-        cur = 0;
-        c = grab();
+        int cur = 0;
+        unsigned int c = grab();
         if (STAGE) {
             if (c < n_chunks && c * 32 + lane < n) prefetch_chunk<SOLVER>(B, c * 32 + lane, false, fine_only, false, my_stage, lane);
             cp_async_commit();
         }
         for (; c < n_chunks; cur ^= 1) {
-            const long long cn = grab();
-            const long long i = c * 32 + lane;
+            const unsigned int cn = grab();
+            const unsigned int i = c * 32 + lane;
             const bool valid = i < n;
             ChunkIn in;
             if (STAGE) {
@@ -535,8 +523,8 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
                 in.cj = make_short2(-3, -3);
             }
             const double R = in.y.x, V = in.y.y;
-            const double ea = mesh_gather(tab, s_edges[0], s_edges[1], in.cj.x, in.ca.x);
-            const double eb = mesh_gather(tab + Np1, s_edges[2], s_edges[3], in.cj.y, in.ca.y);
+            const double ea = mesh_gather(tab, s_cyc.edges[0], s_cyc.edges[1], in.cj.x, in.ca.x);
+            const double eb = mesh_gather(tab + Np1, s_cyc.edges[2], s_cyc.edges[3], in.cj.y, in.ca.y);
             double Pa, Pb;
             if (SOLVER == 1) {
                 // ea = e1 at y, eb = e3 at Phi_h/2 y
@@ -568,17 +556,19 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
             }
         }
         if (STAGE) cp_async_wait<0>();
-        __syncthreads();
-        flush_hist<HIST>(P, B, hist, cyc);
-        if (!grid_sync(P, B.bar, gen, B.status, &s_ok, gridDim.x)) return;
-        build_fields(P, B.Qring + (size_t)(cyc % 3) * 2 * Np1 * kQPad, (long long*)hist, g, tab, inv_r, s_edges, s_warp);
-        ++cyc;
+        }
+        const bool control = !(hs & 1) && !fine_only;
+        if (!field_cycle<HIST>(cyc++, control)) return;
+        if (control && s_stop) {
+            K = k;
+            break;
+        }
     }
 
     if (blockIdx.x == 0 && threadIdx.x == 0 && !fine_only) *B.K_out = K;
     if (detect_only) {
         // step 1 alone leaves y^n as it was: it is row 0 of the trajectory
-        for (long long i = i0; i < n; i += stride) B.y[i] = B.traj[i];
+        for (unsigned int i = i0; i < n; i += stride) B.y[i] = B.traj[i];
         return;
     }
     if (mode != MODE_ETD) return;
@@ -586,7 +576,7 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     // ---- landing (step 3) and extrapolation (step 4); with the band, a
     // particle whose landing rows were not all stored marks a miss
     bool miss = false;
-    for (long long i = i0; i < n; i += stride) {
+    for (unsigned int i = i0; i < n; i += stride) {
         const double o = B.o[i], T = B.T[i];
         const int N = B.N[i];
         const int nt = N > 0 ? 2 : 1;
@@ -618,20 +608,17 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     }
     if (!band) return;
     if (__syncthreads_or(miss) && threadIdx.x == 0) atomicOr(&B.notdone[3], 1);
-    if (!grid_sync(P, B.bar, gen, B.status, &s_ok, gridDim.x)) return;
+    if (!grid_sync()) return;
     if (threadIdx.x == 0) s_miss = ld_acquire_s32(&B.notdone[3]);
     __syncthreads();
     if (!s_miss) return;
-    // replay from y^n (row 0) with every row, for every particle; the charge
-    // buffer of the next cycle is the clear one
-    for (long long i = i0; i < n; i += stride) B.y[i] = B.traj[i];
+    // replay from y^n (row 0) with every row, for every particle
+    for (unsigned int i = i0; i < n; i += stride) B.y[i] = B.traj[i];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        B.notdone[0] = B.notdone[1] = B.notdone[2] = 0;
         atomicAdd(&B.notdone[4], 1);
     }
-    ++cyc;
     K = 0;
-    if (!grid_sync(P, B.bar, gen, B.status, &s_ok, gridDim.x)) return;
+    if (!grid_sync()) return;
     }
 }
 

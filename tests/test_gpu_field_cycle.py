@@ -1,0 +1,80 @@
+"""The field cycle of the window kernels at the edges of its forms.
+
+The charge words of a cycle count their own arrivals where n W leaves room,
+else the cycle ends in a grid barrier; the field is built from 1 to 4 nodes
+per thread in registers or from shared memory.  The charge is an exact
+integer either way, so every form gives the same bits: FP64 windows equal the
+oracle's, FP32 windows do not depend on the block size (128 threads take the
+barrier and the shared-memory build on these meshes).
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1404_1160_gb300 import inputs
+from paper_1404_1160_gb300 import pic
+from tests.gpu_common import bit_equal, cfg_of
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+# nodes = 31 (block / 64) per node of a thread: 1024 threads cover 496, 992, 1488, 1984
+EDGE_CELLS = [494, 496, 990, 992, 1486, 1488, 1982, 1984]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1404_1160_gb300 import build
+
+    build.build()
+    torch.cuda.set_device(0)
+
+
+def etd(p, R0, V0, steps=1):
+    h = pic.pic_init(p, R0, V0)
+    pic.pic_step(h, steps)
+    R, V = pic.pic_get_particles(h)
+    Q = pic.pic_get_field(h, p.n_cells)[0]
+    pic.pic_destroy(h)
+    return R, V, Q
+
+
+@pytest.mark.parametrize("n_cells", EDGE_CELLS)
+def test_fp64_register_build_edges(n_cells):
+    p = pic.pic_default_params(n_cells=n_cells, steps_per_turn=20, max_window_steps=60)
+    R0, V0 = inputs.gaussian_beam(1500, seed=n_cells, r_cut=None)
+    R, V, Q = etd(p, R0, V0)
+    ref = oracle.etd_step(cfg_of(p), R0, V0)
+    assert bit_equal(R, ref.R) and bit_equal(V, ref.V)
+    assert np.array_equal(Q, oracle.deposit(cfg_of(p), ref.R)[0])
+
+
+@pytest.mark.parametrize("n_cells", EDGE_CELLS)
+def test_fp32_register_build_edges(n_cells):
+    R0, V0 = inputs.gaussian_beam(1500, seed=n_cells, r_cut=None)
+    kw = dict(precision=1, n_cells=n_cells, steps_per_turn=20, max_window_steps=60)
+    a = etd(pic.pic_default_params(**kw), R0, V0, 2)
+    b = etd(pic.pic_default_params(block_size=128, **kw), R0, V0, 2)
+    assert all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("n,log2W", [(60_000, 40), (70_000, 40), (140_000, 40), (300, 32), (1, 32), (33, 40)])
+def test_count_bits_of_the_charge_words(n, log2W):
+    # n W on both sides of what the words hold beside the count (64 bits in all)
+    p = pic.pic_default_params(weight_fixed=1 << log2W, steps_per_turn=20, max_window_steps=60)
+    R0, V0 = inputs.gaussian_beam(n, seed=n, r_cut=4.0)
+    R, V, Q = etd(p, R0, V0)
+    ref = oracle.etd_step(cfg_of(p), R0, V0)
+    assert bit_equal(R, ref.R) and bit_equal(V, ref.V)
+    assert np.array_equal(Q, oracle.deposit(cfg_of(p), ref.R)[0])
+
+
+def test_all_particles_on_one_node():
+    # the whole charge n W in one word of every cycle (R = V = 0 stays on the axis)
+    n = 200_000
+    p = pic.pic_default_params(steps_per_turn=20, max_window_steps=60, field_parity=pic.PIC_PARITY_ODD)
+    R, V, Q = etd(p, np.zeros(n), np.zeros(n), 2)
+    assert not R.any() and not V.any()
+    assert Q[p.n_cells // 2] == n * p.weight_fixed and Q.sum() == n * p.weight_fixed
