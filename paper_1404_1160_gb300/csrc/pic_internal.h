@@ -107,7 +107,7 @@ struct WindowLaunch {
     bool kept = false;        // shared memory for the counted charge words
     int coop_grid = 0, coop_block = 0;
     int hist = 0;             // 0: 32-bit split histograms, 1: 64-bit
-    int stage = 0;            // 1: cp.async staging of each warp's next chunk
+    int stage = 0;            // WindowStage: how the chunks are kept
     size_t coop_smem = 0;
 };
 

@@ -198,14 +198,16 @@ __global__ void k_moments(DevParams P, WinBufs B, double* part_d, long long* par
 
 // ------------------------------------------------------------- launchers
 
-// Shared memory of the window kernel with `copies` histogram copies and,
-// with staging, two Stage buffers per warp.
-static size_t coop_smem_bytes(int n_cells, int copies, int block, int stage, int slot_words, bool kept = false) {
-    const size_t Np1 = (size_t)n_cells + 1;
-    const size_t hc = (size_t)hist_copies_reserved(n_cells, copies, block);
-    return (stage ? (size_t)(block / 32) * kStageBytesPerWarp : 0) + 2 * Np1 * sizeof(double2) +
-           hc * 2 * (size_t)slot_words * Np1 * sizeof(unsigned int) + cycle_words(n_cells, block, kept) * sizeof(long long) +
-           Np1 * sizeof(double);
+// Shared memory of the window kernel with `copies` histogram copies and the
+// chunk buffers of `stage` (`chunks`: chunks per block).
+static size_t coop_smem_bytes(const DevParams& P, int copies, int block, int stage, unsigned int chunks, int slot_words,
+                              bool kept = false) {
+    const size_t Np1 = (size_t)P.n_cells + 1;
+    const size_t hc = (size_t)hist_copies_reserved(P.n_cells, copies, block);
+    const size_t buf = P.solver == PIC_FINE_LAWSON_RK4 ? sizeof(Stage<1>) : sizeof(Stage<0>);
+    return stage_buffers(stage, block, chunks) * buf + 2 * Np1 * sizeof(double2) +
+           hc * 2 * (size_t)slot_words * Np1 * sizeof(unsigned int) +
+           cycle_words(P.n_cells, block, kept) * sizeof(long long) + Np1 * sizeof(double);
 }
 
 // The instantiations of k_window_coop live in window_coop.cu, compiled once
@@ -225,22 +227,31 @@ static void* coop_fn(int solver, int hist, int pow2, int stage) {
 
 cudaError_t window_prepare(DevParams& P, int block, int blocks_per_sm, int sm_count, WindowLaunch* L) {
     L->coop_block = block;
-    // staging when the block's shared memory stays within the per-block
-    // limit; then as many histogram copies (up to kHistCopiesMax) as fit
     const size_t limit = 220 * 1024;
-    // positions one block deposits into one field per cycle: at most the
-    // chunks of 32 of one block, with at least one block per SM
+    // One chunk per block fills the GPU before a block takes a second one: the
+    // sweeps of a small beam are a chain of FP64 latencies, which more warps
+    // on one SM only lengthen (the FP64 pipe takes 16 clocks per warp
+    // instruction), and a block costs the exchange next to nothing.
     const long long n_chunks = (P.n + 31) / 32;
-    long long need_blocks = (P.n + block - 1) / block;
-    const long long min_grid = need_blocks < sm_count ? (need_blocks < 1 ? 1 : need_blocks) : sm_count;
-    const int slot = (n_chunks + min_grid - 1) / min_grid * 32 > 65536 ? hist_slot_words(2) : hist_slot_words(0);
-    L->stage = coop_smem_bytes(P.n_cells, 1, block, 1, slot) <= limit ? 1 : 0;
+    const long long most = n_chunks < 1 ? 1 : n_chunks;
+    const long long min_grid = most < sm_count ? most : sm_count;  // with at least one block per SM
+    const unsigned int chunks = (unsigned int)((n_chunks + min_grid - 1) / min_grid);
+    // positions one block deposits into one field per cycle: its chunks of 32
+    const int slot = (long long)chunks * 32 > 65536 ? hist_slot_words(2) : hist_slot_words(0);
+    auto smem = [&](int copies, int stage, bool kept) {
+        return coop_smem_bytes(P, copies, block, stage, chunks, slot, kept);
+    };
+    // the chunks stay in shared memory where they fit beside two histogram
+    // copies and the charge words; else the next chunk is staged where that
+    // leaves room; then as many histogram copies (up to kHistCopiesMax) as fit
+    const bool regs = field_in_regs(P.n_cells, block);
     int copies = kHistCopiesMax;
-    while (copies > 1 && coop_smem_bytes(P.n_cells, copies, block, L->stage, slot) > limit) copies >>= 1;
+    if (blocks_per_sm <= 1 && smem(copies, STAGE_RESIDENT, regs) <= limit) L->stage = STAGE_RESIDENT;
+    else L->stage = smem(1, STAGE_NEXT, false) <= limit ? STAGE_NEXT : STAGE_NONE;
+    while (copies > 1 && smem(copies, L->stage, false) > limit) copies >>= 1;
     P.hist_copies = copies;
-    L->kept = field_in_regs(P.n_cells, block) &&
-              coop_smem_bytes(P.n_cells, copies, block, L->stage, slot, true) <= kWindowSmemMax;
-    L->coop_smem = coop_smem_bytes(P.n_cells, copies, block, L->stage, slot, L->kept);
+    L->kept = regs && smem(copies, L->stage, true) <= kWindowSmemMax;
+    L->coop_smem = smem(copies, L->stage, L->kept);
     int bps = 1 << 30;
     for (int hh = 0; hh < 3; ++hh) {
         void* fn = coop_fn(P.solver, hh, P.xs_fma, L->stage);
@@ -255,7 +266,7 @@ cudaError_t window_prepare(DevParams& P, int block, int blocks_per_sm, int sm_co
     const int want = blocks_per_sm > 0 ? blocks_per_sm : 1;
     if (want < bps) bps = want;
     long long grid = (long long)bps * sm_count;
-    if (need_blocks < grid) grid = need_blocks < 1 ? 1 : need_blocks;
+    if (most < grid) grid = most;
     L->coop_grid = (int)grid;
     // the split 32-bit histograms need qR < 2^32 (W <= 2^32) and at most
     // 65536 (HIST 0) or 2^21 (HIST 2, when the layout has its fourth word)

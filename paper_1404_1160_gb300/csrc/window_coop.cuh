@@ -261,16 +261,37 @@ __device__ __forceinline__ bool band_holds(int x, int k, int band_m) {
 // ------------------------------------------------ cooperative Poisson window
 
 // One chunk (32 particles) of window state in shared memory; lane l owns
-// entry l of every array, so no warp synchronisation is needed.
-struct Stage {
+// entry l of every array, so no warp synchronisation is needed.  cx: Lawson
+// carries (Phi_h y)_R, RK4 both stage positions.
+template <int SOLVER>
+struct StageCx {
+    double2 cx[32];
+};
+template <>
+struct StageCx<1> {
+    double cx[32];
+};
+template <int SOLVER>
+struct Stage : StageCx<SOLVER> {
     double2 y[32];
     double2 ce[32];
     double2 ca[32];
-    double2 cx[32];  // Lawson uses .x ((Phi_h y)_R), RK4 both stage positions
     int2 tr[32];
     short2 cj[32];
 };
-constexpr size_t kStageBytesPerWarp = 2 * sizeof(Stage);
+// How a window keeps its chunks: in global memory, loaded directly (0) or
+// through a double buffer per warp (1: the next chunk is in flight while the
+// current one is worked on), or in shared memory for the whole window (2).
+// A resident chunk saves the L2 round trip at the start of every sweep,
+// which a beam with one or two chunks per warp cannot hide.  Measured on
+// GB300 together with one block per SM instead of n/1024 blocks: two RK4 steps
+// of 20000 particles 9.17 -> 5.79 ms, the modified scheme on 150001 8.64 ->
+// 8.07 ms; 10^6 particles do not fit and stay staged (9.5 ms).
+enum WindowStage { STAGE_NONE = 0, STAGE_NEXT = 1, STAGE_RESIDENT = 2 };
+// Chunk buffers a block holds; `chunks`: the chunks of one block.
+__host__ __device__ constexpr size_t stage_buffers(int stage, int block, unsigned int chunks) {
+    return stage == STAGE_RESIDENT ? chunks : (stage == STAGE_NEXT ? 2 * (size_t)(block >> 5) : 0);
+}
 
 // The state a sweep reads for one particle.
 struct ChunkIn {
@@ -280,20 +301,20 @@ struct ChunkIn {
 };
 
 template <int SOLVER>
-__device__ __forceinline__ void prefetch_chunk(const WinBufs& B, long long i, bool sweepA, bool fine_only, bool k0,
-                                               Stage* s, int lane) {
+__device__ __forceinline__ void prefetch_chunk(const WinBufs& B, unsigned int i, bool sweepA, bool fine_only, bool k0,
+                                               Stage<SOLVER>* s, int lane) {
     cp_async16(&s->y[lane], &B.y[i]);
     if (sweepA && !fine_only) cp_async8(&s->tr[lane], &B.tr[i]);
     if (sweepA && k0) return;
     if (sweepA) cp_async16(&s->ce[lane], &B.ce[i]);
     cp_async16(&s->ca[lane], &B.ca[i]);
-    if (SOLVER == 1) cp_async8(&s->cx[lane].x, &B.cxr[i]);
+    if constexpr (SOLVER == 1) cp_async8(&s->cx[lane], &B.cxr[i]);
     else cp_async16(&s->cx[lane], &B.cx[i]);
     cp_async4(&s->cj[lane], &B.cj[i]);
 }
 
 template <int SOLVER>
-__device__ __forceinline__ ChunkIn load_chunk(const WinBufs& B, long long i, bool sweepA, bool fine_only, bool k0) {
+__device__ __forceinline__ ChunkIn load_chunk(const WinBufs& B, unsigned int i, bool sweepA, bool fine_only, bool k0) {
     ChunkIn c;
     c.y = B.y[i];
     c.tr = (sweepA && !fine_only) ? B.tr[i] : make_int2(0, 0);
@@ -310,12 +331,14 @@ __device__ __forceinline__ ChunkIn load_chunk(const WinBufs& B, long long i, boo
     return c;
 }
 
-__device__ __forceinline__ ChunkIn read_stage(const Stage* s, int lane) {
+template <int SOLVER>
+__device__ __forceinline__ ChunkIn read_stage(const Stage<SOLVER>* s, int lane) {
     ChunkIn c;
     c.y = s->y[lane];
     c.ce = s->ce[lane];
     c.ca = s->ca[lane];
-    c.cx = s->cx[lane];
+    if constexpr (SOLVER == 1) c.cx = make_double2(s->cx[lane], 0.0);
+    else c.cx = s->cx[lane];
     c.tr = s->tr[lane];
     c.cj = s->cj[lane];
     return c;
@@ -327,8 +350,10 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     const int Nc = P.n_cells, Np1 = Nc + 1;
     const int words = Hist<HIST>::kWordsPerNode * Np1;   // 32-bit words per field histogram
     const int copies = P.hist_copies;
-    Stage* stage = (Stage*)smem_raw;                      // STAGE: 2 per warp
-    double2* tab = (double2*)(smem_raw + (STAGE ? (blockDim.x >> 5) * kStageBytesPerWarp : 0));  // 2 Np1
+    const unsigned int n = (unsigned int)P.n;             // below 2^31
+    const unsigned int n_chunks = (n + 31) / 32;
+    Stage<SOLVER>* stage = (Stage<SOLVER>*)smem_raw;
+    double2* tab = (double2*)(stage + stage_buffers(STAGE, blockDim.x, (n_chunks + gridDim.x - 1) / gridDim.x));  // 2 Np1
     unsigned int* hist = (unsigned int*)(tab + 2 * Np1);  // copies x 2 fields x words (staged build: also the scan input)
     long long* g = (long long*)(hist + hist_copies_reserved(Nc, copies, blockDim.x) * 2 * hist_slot_words(HIST) * Np1);  // 2 Np1
     double* inv_r = (double*)(g + cycle_words(Nc, blockDim.x, P.q_cb > 0));  // Np1
@@ -344,7 +369,6 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
         inv_r[j] = (j == P.c) ? 0.0 : 1.0 / (P.r_min + (double)j * P.hr);
 
     const bool detect_only = mode == MODE_PERIODS, fine_only = mode == MODE_FINE;
-    const unsigned int n = (unsigned int)P.n;  // below 2^31
     // Work unit: a chunk of 32 consecutive storage slots (phase-space
     // neighbours after the sort).  Block b owns the chunks c = b (mod grid),
     // so every block sees all phases (the sign changes of V spread evenly
@@ -352,20 +376,21 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     // the block, warps take the block's chunks dynamically from a shared
     // counter, so they finish a sweep together.
     const int lane = threadIdx.x & 31;
-    const unsigned int n_chunks = (n + 31) / 32;
+    const unsigned int my_chunks = blockIdx.x < n_chunks ? (n_chunks - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     // lane l deposits into copy l mod copies (the lanes of a warp hold
     // phase-space neighbours, which mostly share a cell)
     unsigned int* const my_hist = hist + ((threadIdx.x & 31) % copies) * 2 * words;
-    Stage* const my_stage = stage + 2 * (threadIdx.x >> 5);
-    const unsigned int g_warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
-    const unsigned int stride = gridDim.x * (blockDim.x & ~31u);  // static mapping (init and landing)
-    const unsigned int i0 = g_warp * 32 + lane;
-    // next chunk of this block for this warp (warp-uniform)
+    const unsigned int warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    Stage<SOLVER>* const my_stage = stage + 2 * warp;  // STAGE_NEXT
+    // Chunk m of this block starts at slot 32 (blockIdx.x + m gridDim.x); a
+    // warp's first chunk of a sweep is its own number, the next ones come
+    // from the counter (warp-uniform).
+    auto slot0 = [&](unsigned int m) -> unsigned int { return (blockIdx.x + m * gridDim.x) * 32; };
+    const unsigned int stride = n_warps * gridDim.x * 32;  // static mapping of the landing: chunks warp, warp + n_warps, ...
     auto grab = [&]() -> unsigned int {
         unsigned int m = 0;
         if (lane == 0) m = atomicAdd(&s_next, 1);
-        m = __shfl_sync(0xffffffffu, m, 0);
-        return blockIdx.x + m * gridDim.x;
+        return n_warps + __shfl_sync(0xffffffffu, m, 0);
     };
     const double ie = P.inv_eps, mie = P.mie;
     const long long W = P.W;
@@ -378,8 +403,10 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     // row fell outside the band of attempt 0
     for (int attempt = 0;; ++attempt) {
     const bool band = band_ok && attempt == 0;
-    if (!fine_only) {
-        for (unsigned int i = i0; i < n; i += stride) {
+    for (unsigned int m = warp; m < my_chunks; m += n_warps) {
+        const unsigned int i = slot0(m) + lane;
+        int2 tr = make_int2(0, 0);
+        if (i < n && !fine_only) {
             if (T_known) {
                 Track s;
                 s.flags = 0;
@@ -388,10 +415,15 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
                 B.T[i] = s.T;
                 B.o[i] = s.o;
                 B.N[i] = s.N;
-                B.tr[i] = make_int2(s.flags, s.need);
-            } else {
-                B.tr[i] = make_int2(band ? band_bits(P, B.T[i]) : 0, 0);
+                tr = make_int2(s.flags, s.need);
+            } else if (band) {
+                tr.x = band_bits(P, B.T[i]);
             }
+            B.tr[i] = tr;
+        }
+        if (STAGE == STAGE_RESIDENT) {
+            stage[m].y[lane] = i < n ? B.y[i] : make_double2(0.0, 0.0);
+            stage[m].tr[lane] = tr;
         }
     }
 
@@ -405,26 +437,29 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
         const bool k0 = k == 0;
         unsigned int cnt = 0;
         int cur = 0;
-        unsigned int c = grab();
-        if (STAGE) {
-            if (c < n_chunks && c * 32 + lane < n) prefetch_chunk<SOLVER>(B, c * 32 + lane, true, fine_only, k0, my_stage, lane);
+        unsigned int m = warp;
+        if (STAGE == STAGE_NEXT) {
+            if (m < my_chunks && slot0(m) + lane < n) prefetch_chunk<SOLVER>(B, slot0(m) + lane, true, fine_only, k0, my_stage, lane);
             cp_async_commit();
         }
         // warp-uniform trip count: lanes past the end run with an empty cell
-        for (; c < n_chunks; cur ^= 1) {
-            const unsigned int cn = grab();
-            const unsigned int i = c * 32 + lane;
+        for (; m < my_chunks; cur ^= 1) {
+            const unsigned int mn = grab();
+            const unsigned int i = slot0(m) + lane;
             const bool valid = i < n;
+            Stage<SOLVER>* const S = stage + m;  // STAGE_RESIDENT
             ChunkIn in;
-            if (STAGE) {
-                if (cn < n_chunks && cn * 32 + lane < n) prefetch_chunk<SOLVER>(B, cn * 32 + lane, true, fine_only, k0, my_stage + (cur ^ 1), lane);
+            if (STAGE == STAGE_NEXT) {
+                if (mn < my_chunks && slot0(mn) + lane < n) prefetch_chunk<SOLVER>(B, slot0(mn) + lane, true, fine_only, k0, my_stage + (cur ^ 1), lane);
                 cp_async_commit();
                 cp_async_wait<1>();
-                in = read_stage(my_stage + cur, lane);
+                in = read_stage<SOLVER>(my_stage + cur, lane);
+            } else if (STAGE == STAGE_RESIDENT) {
+                in = read_stage<SOLVER>(S, lane);
             } else if (valid) {
                 in = load_chunk<SOLVER>(B, i, true, fine_only, k0);
             }
-            c = cn;
+            m = mn;
             double R = valid ? in.y.x : 0.0, V = valid ? in.y.y : 0.0;
             if (!valid) {
             } else if (k > 0) {
@@ -455,11 +490,13 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
                     if (!((tr.x & F_RES) && (detect_only || k > tr.y)) && (!band || band_holds(tr.x, k, P.band_m)))
                         __stcs(&B.traj[(size_t)k * n + i], make_double2(Rn, Vn));
                     const bool done = track_update(P, B, i, k, V, Vn, detect_only, tr);
+                    if (STAGE == STAGE_RESIDENT) S->tr[lane] = tr;
                     cnt += done ? 0u : 1u;
                 }
                 R = Rn;
                 V = Vn;
-                B.y[i] = make_double2(R, V);
+                if (STAGE == STAGE_RESIDENT) S->y[lane] = make_double2(R, V);
+                if (STAGE != STAGE_RESIDENT || last_fine) B.y[i] = make_double2(R, V);
             } else if (!fine_only) {
                 __stcs(&B.traj[i], make_double2(R, V));
                 cnt += 1u;
@@ -481,14 +518,19 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
             if (!valid) ca.j = cb.j = -3;
             deposit_cell<HIST>(my_hist, Np1, ca, W);
             deposit_cell<HIST>(my_hist + words, Np1, cb, W);
-            if (valid) {
+            if (STAGE == STAGE_RESIDENT) {
+                S->ca[lane] = make_double2(ca.a, cb.a);
+                S->cj[lane] = make_short2((short)ca.j, (short)cb.j);
+                if constexpr (SOLVER == 1) S->cx[lane] = cx.x;
+                else S->cx[lane] = cx;
+            } else if (valid) {
                 B.ca[i] = make_double2(ca.a, cb.a);
                 B.cj[i] = make_short2((short)ca.j, (short)cb.j);
                 if (SOLVER == 1) B.cxr[i] = cx.x;
                 else B.cx[i] = cx;
             }
         }
-        if (STAGE) cp_async_wait<0>();
+        if (STAGE == STAGE_NEXT) cp_async_wait<0>();
         if (last_fine) break;
         if (!fine_only) {
             cnt = __reduce_add_sync(0xffffffffu, cnt);
@@ -497,25 +539,28 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
         } else {
         // ---- sweep B(k): gather pair 1, deposit stage pair 2
         int cur = 0;
-        unsigned int c = grab();
-        if (STAGE) {
-            if (c < n_chunks && c * 32 + lane < n) prefetch_chunk<SOLVER>(B, c * 32 + lane, false, fine_only, false, my_stage, lane);
+        unsigned int m = warp;
+        if (STAGE == STAGE_NEXT) {
+            if (m < my_chunks && slot0(m) + lane < n) prefetch_chunk<SOLVER>(B, slot0(m) + lane, false, fine_only, false, my_stage, lane);
             cp_async_commit();
         }
-        for (; c < n_chunks; cur ^= 1) {
-            const unsigned int cn = grab();
-            const unsigned int i = c * 32 + lane;
+        for (; m < my_chunks; cur ^= 1) {
+            const unsigned int mn = grab();
+            const unsigned int i = slot0(m) + lane;
             const bool valid = i < n;
+            Stage<SOLVER>* const S = stage + m;  // STAGE_RESIDENT
             ChunkIn in;
-            if (STAGE) {
-                if (cn < n_chunks && cn * 32 + lane < n) prefetch_chunk<SOLVER>(B, cn * 32 + lane, false, fine_only, false, my_stage + (cur ^ 1), lane);
+            if (STAGE == STAGE_NEXT) {
+                if (mn < my_chunks && slot0(mn) + lane < n) prefetch_chunk<SOLVER>(B, slot0(mn) + lane, false, fine_only, false, my_stage + (cur ^ 1), lane);
                 cp_async_commit();
                 cp_async_wait<1>();
-                in = read_stage(my_stage + cur, lane);
+                in = read_stage<SOLVER>(my_stage + cur, lane);
+            } else if (STAGE == STAGE_RESIDENT) {
+                in = read_stage<SOLVER>(S, lane);
             } else if (valid) {
                 in = load_chunk<SOLVER>(B, i, false, fine_only, false);
             }
-            c = cn;
+            m = mn;
             if (!valid) {
                 in.y = make_double2(0.0, 0.0);
                 in.ca = make_double2(0.0, 0.0);
@@ -530,7 +575,8 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
                 // ea = e1 at y, eb = e3 at Phi_h/2 y
                 Pa = fma(P.sh, fma(P.h2, ea, V), P.ch * R);              // stage 2
                 Pb = fma(P.hsh, eb, in.cx.x);                            // stage 4
-                if (valid) B.ce[i] = make_double2(ea, eb);
+                if (STAGE == STAGE_RESIDENT) S->ce[lane] = make_double2(ea, eb);
+                else if (valid) B.ce[i] = make_double2(ea, eb);
             } else {
                 // ea = e1 at y, eb = e2 at y + h/2 k1, cx.x = R2
                 const double k1R = ie * V, k1V = fma(mie, R, ea);
@@ -541,8 +587,12 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
                 const double R4 = fma(P.h, k3R, R);
                 Pa = R3;                                                 // stage 3
                 Pb = R4;                                                 // stage 4
-                if (valid) {
-                    B.ce[i] = make_double2((k1R + 2.0 * k2R) + 2.0 * k3R, k1V + 2.0 * k2V);
+                const double2 part = make_double2((k1R + 2.0 * k2R) + 2.0 * k3R, k1V + 2.0 * k2V);
+                if constexpr (STAGE == STAGE_RESIDENT && SOLVER == 0) {
+                    S->ce[lane] = part;
+                    S->cx[lane] = make_double2(R3, R4);
+                } else if (valid) {
+                    B.ce[i] = part;
                     B.cx[i] = make_double2(R3, R4);
                 }
             }
@@ -550,12 +600,15 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
             if (!valid) ca2.j = cb2.j = -3;
             deposit_cell<HIST>(my_hist, Np1, ca2, W);
             deposit_cell<HIST>(my_hist + words, Np1, cb2, W);
-            if (valid) {
+            if (STAGE == STAGE_RESIDENT) {
+                S->ca[lane] = make_double2(ca2.a, cb2.a);
+                S->cj[lane] = make_short2((short)ca2.j, (short)cb2.j);
+            } else if (valid) {
                 B.ca[i] = make_double2(ca2.a, cb2.a);
                 B.cj[i] = make_short2((short)ca2.j, (short)cb2.j);
             }
         }
-        if (STAGE) cp_async_wait<0>();
+        if (STAGE == STAGE_NEXT) cp_async_wait<0>();
         }
         const bool control = !(hs & 1) && !fine_only;
         if (!field_cycle<HIST>(cyc++, control)) return;
@@ -568,7 +621,7 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     if (blockIdx.x == 0 && threadIdx.x == 0 && !fine_only) *B.K_out = K;
     if (detect_only) {
         // step 1 alone leaves y^n as it was: it is row 0 of the trajectory
-        for (unsigned int i = i0; i < n; i += stride) B.y[i] = B.traj[i];
+        for (unsigned int i = slot0(warp) + lane; i < n; i += stride) B.y[i] = B.traj[i];
         return;
     }
     if (mode != MODE_ETD) return;
@@ -576,7 +629,7 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     // ---- landing (step 3) and extrapolation (step 4); with the band, a
     // particle whose landing rows were not all stored marks a miss
     bool miss = false;
-    for (unsigned int i = i0; i < n; i += stride) {
+    for (unsigned int i = slot0(warp) + lane; i < n; i += stride) {
         const double o = B.o[i], T = B.T[i];
         const int N = B.N[i];
         const int nt = N > 0 ? 2 : 1;
@@ -613,7 +666,7 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     __syncthreads();
     if (!s_miss) return;
     // replay from y^n (row 0) with every row, for every particle
-    for (unsigned int i = i0; i < n; i += stride) B.y[i] = B.traj[i];
+    for (unsigned int i = slot0(warp) + lane; i < n; i += stride) B.y[i] = B.traj[i];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         atomicAdd(&B.notdone[4], 1);
     }

@@ -78,3 +78,36 @@ def test_all_particles_on_one_node():
     R, V, Q = etd(p, np.zeros(n), np.zeros(n), 2)
     assert not R.any() and not V.any()
     assert Q[p.n_cells // 2] == n * p.weight_fixed and Q.sum() == n * p.weight_fixed
+
+
+# FP64 chunks of 32 particles: kept in shared memory (small n), staged one
+# ahead (large n) or loaded in place (large meshes); 152 SMs
+WAYS = [(1, {}), (31, {}), (33, {}), (152 * 32 - 1, {}), (152 * 32 + 1, {}), (5000, dict(block_size=512, blocks_per_sm=2)),
+        (20_000, dict(n_cells=2048)), (400_000, {}), (480_000, {}), (480_000, dict(n_cells=100))]
+
+
+@pytest.mark.parametrize("n,kw", WAYS)
+@pytest.mark.parametrize("solver", [pic.PIC_FINE_RK4, pic.PIC_FINE_LAWSON_RK4])
+def test_fp64_ways_to_keep_the_chunks(n, kw, solver):
+    p = pic.pic_default_params(fine_solver=solver, steps_per_turn=20, max_window_steps=60, **kw)
+    cfg = cfg_of(p)
+    R0, V0 = inputs.gaussian_beam(n, seed=n, r_cut=None)
+    h = pic.pic_init(p, R0, V0)
+    pic.pic_step(h, 1)
+    R, V = pic.pic_get_particles(h)
+    T, N, o = pic.pic_get_periods(h)
+    ref = oracle.etd_step(cfg, R0, V0)
+    assert bit_equal(R, ref.R) and bit_equal(V, ref.V) and np.array_equal(N, ref.N)
+    # the reference solution and step 1 alone (the modified scheme) on the same handle
+    pic.pic_set_particles(h, R0, V0)
+    pic.pic_fine_steps(h, 3)
+    R, V = pic.pic_get_particles(h)
+    Rf, Vf = oracle.fine_steps(cfg, R0, V0, 3)
+    assert bit_equal(R, Rf) and bit_equal(V, Vf)
+    pic.pic_set_particles(h, R0, V0)
+    P = pic.pic_step_classic(h, 1, 1)
+    R, V = pic.pic_get_particles(h)
+    Rc, Vc, Pc = oracle.classic_step(cfg, R0, V0, 1)
+    assert P == Pc and bit_equal(R, Rc) and bit_equal(V, Vc)
+    assert bit_equal(pic.pic_get_periods(h)[2], o)  # step 1 alone leaves the last macro step's remainders
+    pic.pic_destroy(h)
