@@ -318,26 +318,6 @@ __device__ __forceinline__ void track_sample(Track& s, const DevParams& P, int k
     }
 }
 
-// Root of an extremum already known to lie between samples k-2 and k-1,
-// from the stencil V_{k-2} = v0, V_{k-1} = v1, V_k = v2.
-__device__ __forceinline__ void track_root(Track& s, const DevParams& P, int k, double v0, double v1, double v2,
-                                           bool detect_only) {
-    if (s.flags & F_RES) return;
-    const double t = (double)(k - 2) + quad_root01(v0, v1, v2);
-    const int ne = (s.flags & F_NEXT) + 1;
-    s.flags = (s.flags & ~F_NEXT) | (ne & F_NEXT);
-    if (ne == 1) s.t1 = t;
-    if (ne == 3) {
-        const double T = t - s.t1;
-        if (detect_only) {
-            s.T = T;
-            s.flags |= F_RES;
-        } else {
-            track_resolve(s, P, T);
-        }
-    }
-}
-
 // Window cap reached without a third extremum.
 __device__ __forceinline__ void track_cap(Track& s, const DevParams& P, bool detect_only) {
     if (s.flags & F_RES) return;

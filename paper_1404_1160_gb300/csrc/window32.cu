@@ -168,6 +168,13 @@ static __device__ __forceinline__ void clear_hist32(unsigned int* hist, int word
     // 16-byte stores: the region starts aligned and holds a multiple of four words
     for (int i = threadIdx.x; i < words / 4; i += blockDim.x) ((uint4*)hist)[i] = make_uint4(0u, 0u, 0u, 0u);
 }
+struct NodeField32 {
+    float E, S;  // the field and float(S_j) (float(Q_c) at the centre)
+};
+static __device__ __forceinline__ NodeField32 shfl_next(const NodeField32& v) {
+    return {__shfl_down_sync(0xffffffffu, v.E, 1), v.S};  // only E is used of the next lane's node
+}
+
 static __device__ __forceinline__ bool field_cycle32(int cyc, int pair, bool control) {
     __syncthreads();
     const int Nc = s_cyc.n_cells, Np1 = Nc + 1, c = s_cyc.c, copies = s_cyc.copies;
@@ -188,17 +195,20 @@ static __device__ __forceinline__ bool field_cycle32(int cyc, int pair, bool con
             s_next = 0;
         }
     };
-    auto field_at = [&](int j, long long S, long long qj) -> float { return __ll2float_rn(j == c ? qj : S) * cq[j]; };
-    auto edge = [&](int f, int j, long long S) {
+    auto field_at = [&](int j, long long S, long long qj) -> NodeField32 {
+        const float x = __ll2float_rn(j == c ? qj : S);
+        return {x * cq[j], x};
+    };
+    auto edge = [&](int f, int j, float x) {
         // odd reading: the lower edge value carries the sign flip (rE / |R|)
-        const float rE = __ll2float_rn(S) * s_cyc.q_half_f;
+        const float rE = x * s_cyc.q_half_f;
         if (j == 0) edges[2 * f] = s_cyc.parity_odd ? -rE : rE;
         if (j == Nc) edges[2 * f + 1] = rE;
     };
     if (field_in_regs(Nc, blockDim.x)) {
-        auto emit = [&](int f, int j, float e, float en, long long S) {
-            tab[f * Np1 + j] = make_float2(e, j < Nc ? en - e : 0.0f);
-            if (j == 0 || j == Nc) edge(f, j, S);
+        auto emit = [&](int f, int j, const NodeField32& v, const NodeField32& next) {
+            tab[f * Np1 + j] = make_float2(v.E, j < Nc ? next.E - v.E : 0.0f);
+            edge(f, j, v.S);
         };
         if (!field_build_regs(Q, prev, control, field_at, emit, clear)) return false;
         __syncthreads();
@@ -220,8 +230,9 @@ static __device__ __forceinline__ bool field_cycle32(int cyc, int pair, bool con
     for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
         const int f = idx >= Np1, j = idx - f * Np1;
         const long long S = g[idx] - s_tot[f];
-        if (j == 0 || j == Nc) edge(f, j, S);
-        e[2 * idx] = field_at(j, S, s_tot[2 + f]);
+        const NodeField32 v = field_at(j, S, s_tot[2 + f]);
+        edge(f, j, v.S);
+        e[2 * idx] = v.E;
     }
     __syncthreads();
     clear();
@@ -236,76 +247,62 @@ static __device__ __forceinline__ bool field_cycle32(int cyc, int pair, bool con
 // ------------------------------------------------------------ tracking
 
 // Period tracking of one particle at sample k >= 1 (the FP32 twin of
-// track_update in window.cu): a sign change of V between samples k-1 and
-// k is marked pending and its root taken at sample k+1 from V_{k-1}, V_k,
-// V_{k+1}, V_{k-1} being recomputed from row k-1 of the trajectory.  trw =
-// flags | need << 8.  Extremum times are kept as (integer, fraction).
-// This is the rare part (a root, a resolution or the window cap), kept out
-// of line so that a sweep never executes it for the other lanes.
-static __device__ __noinline__ unsigned int track32_slow(const DevParams& P, const WinBufs32& B, long long i, int k,
-                                                        float Vold, float Vnew, bool detect_only, unsigned int trw,
-                                                        const float2* row_km2, float2 rot_km2) {
+// track_update in window_coop.cuh): a sign change of V between samples k-1
+// and k is marked pending and counted as an extremum at sample k+1.  trw =
+// flags | need << 8; until the period is known `need` holds the sample k_1
+// before the first extremum.  Only the third extremum evaluates roots (with
+// V_m = (Phi(t_m) z_m)_V of the stored rows) and resolves the period; that
+// part, and the window cap, are out of line.
+// Extremum times are kept as (integer, fraction).
+static __device__ __noinline__ unsigned int track32_resolve(const DevParams& P, const WinBufs32& B, long long i, int k,
+                                                           float Vold, float Vnew, bool detect_only,
+                                                           unsigned int trw) {
     int flags = (int)(trw & 31u);
     int need = (int)(trw >> 8);
-    if (flags & F_PEND) {
-        const float2 zp = row_km2[i];
-        const float v0 = rot_V(rot_km2, zp.x, zp.y);
-        flags &= ~F_PEND;
-        const float s = quad_root01f(v0, Vold, Vnew);
-        const int ne = (flags & F_NEXT) + 1;
-        flags = (flags & ~F_NEXT) | (ne & F_NEXT);
-        if (ne == 1) {
-            CTime t1;
-            t1.i = k - 2;
-            t1.f = s;
-            B.t1[i] = t1;
-        }
-        if (ne == 3) {
-            const CTime t1 = B.t1[i];
-            const CTime T = ct_norm((long long)(k - 2) - t1.i, s - t1.f);
-            if (detect_only) {
-                flags |= F_RES;
-                B.T[i] = T;
-            } else {
-                const Decomp32 d = resolve32(P, T, true, flags);
-                B.T[i] = d.T;
-                B.o[i] = d.o;
-                B.N[i] = d.N;
-                need = d.need;
-            }
-        }
-    }
-    if (!(flags & F_RES) && positive32(Vold) != positive32(Vnew)) flags |= F_PEND;
-    if (k == P.Kmax && !(flags & F_RES)) {
-        // window cap without a third extremum: T = 2 pi eps
+    auto V = [&](int m) -> float {
+        const float2 z = m == 0 ? B.y[i] : B.traj[(size_t)(m - 1) * B.ld + i];
+        const float2 cs = P.rot[rot_index(P, 2ll * m)];
+        return rot_V(cs, z.x, z.y);
+    };
+    CTime T;
+    T.i = P.spt;  // window cap without a third extremum: T = 2 pi eps
+    T.f = 0.0f;
+    if ((flags & F_NEXT) == 3) {
+        const float s1 = quad_root01f(V(need), V(need + 1), V(need + 2));
+        const float s3 = quad_root01f(V(k - 2), Vold, Vnew);
+        T = ct_norm((long long)(k - 2) - need, s3 - s1);
+    } else {
         flags |= F_FB;
-        CTime Tfb;
-        Tfb.i = P.spt;
-        Tfb.f = 0.0f;
-        if (detect_only) {
-            flags |= F_RES;
-            B.T[i] = Tfb;
-        } else {
-            const Decomp32 d = resolve32(P, Tfb, true, flags);
-            B.T[i] = d.T;
-            B.o[i] = d.o;
-            B.N[i] = d.N;
-            need = d.need;
-        }
     }
-    trw = (unsigned int)flags | ((unsigned int)need << 8);
-    B.tr[i] = trw;
-    return trw;
+    if (detect_only) {
+        flags |= F_RES;
+        B.T[i] = T;
+        need = 0;
+    } else {
+        const Decomp32 d = resolve32(P, T, true, flags);
+        B.T[i] = d.T;
+        B.o[i] = d.o;
+        B.N[i] = d.N;
+        need = d.need;
+    }
+    return (unsigned int)flags | ((unsigned int)need << 8);
 }
 
 // Returns true when the particle is done at sample k (resolved and every
 // sample it needs is produced).
 __device__ __forceinline__ bool track32_update(const DevParams& P, const WinBufs32& B, long long i, int k, float Vold,
-                                               float Vnew, bool detect_only, unsigned int& trw,
-                                               const float2* row_km2, float2 rot_km2) {
+                                               float Vnew, bool detect_only, unsigned int& trw) {
     if (!(trw & (unsigned int)F_RES)) {
-        const bool event = (trw & (unsigned int)F_PEND) || positive32(Vold) != positive32(Vnew) || k == P.Kmax;
-        if (event) trw = track32_slow(P, B, i, k, Vold, Vnew, detect_only, trw, row_km2, rot_km2);
+        const bool pend = trw & (unsigned int)F_PEND, change = positive32(Vold) != positive32(Vnew);
+        if (pend || change || k == P.Kmax) {
+            if (pend) {
+                trw += 1u - (unsigned int)F_PEND;
+                if ((trw & 3u) == 1u) trw |= (unsigned int)(k - 2) << 8;
+            }
+            if ((trw & 3u) == 3u || k == P.Kmax) trw = track32_resolve(P, B, i, k, Vold, Vnew, detect_only, trw);
+            else if (change) trw |= (unsigned int)F_PEND;
+            B.tr[i] = trw;
+        }
         if (!(trw & (unsigned int)F_RES)) return false;
     }
     return detect_only || k >= (int)(trw >> 8);
@@ -458,15 +455,13 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
         if (!(hs & 1)) {
         // ---- sweep A(k): finish step k-1 (write row k), sample k, deposit stage pair 1 of step k
         const bool last_fine = fine_only && k == n_fine;
-        float2 ra = rb, rm = rp, rk2 = rb;
+        float2 ra = rb, rm = rp;
         if (k > 0) {
             ra = P.rot[rot_index(P, 2ll * k - 2)];  // Phi(t_{k-1})
             rm = P.rot[rot_index(P, 2ll * k - 1)];  // Phi(t_{k-1} + h/2)
         }
-        if (k > 1) rk2 = P.rot[rot_index(P, 2ll * k - 4)];
         const float2* src = row(k > 0 ? k - 1 : 0);
         float2* dst = last_fine ? B.y : row(k);
-        const float2* src2 = k > 1 ? row(k - 2) : nullptr;
         unsigned int cnt = 0;
         for (long long gi = grab(); gi >= 0; gi = grab()) {
             const long long base = gi * kGroup + lane * kG;
@@ -488,7 +483,7 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
                     if (track && valid) {
                         unsigned int trw = grp_tr(cur, q);
                         const bool done =
-                            track32_update(P, B, i, k, Vold, rot_V(rb, zR, zV), detect_only, trw, src2, rk2);
+                            track32_update(P, B, i, k, Vold, rot_V(rb, zR, zV), detect_only, trw);
                         cnt += done ? 0u : 1u;
                     }
                 } else if (track && valid) {

@@ -192,9 +192,9 @@ static __device__ __forceinline__ void poll_nodes(const unsigned long long* Qf, 
 // last node in the next lane.  q_j comes from the cycle's global charge;
 // the exact trapezoid sums g_j = sum_{m<j} (q_m + q_{m+1}) are a warp scan
 // plus the totals of the warps between the node's and the centre's (s_tot),
-// S_j = g_j - g_c, and the node field is field_at(j, S_j, q_j) (binary64 or
-// binary32: its type is the table's).  Each owned node is passed to
-// emit(f, j, E_j, E_{j+1}, S_j) (E_{j+1} unused at j = n_cells); after_scan()
+// S_j = g_j - g_c, and the node's field is field_at(j, S_j, q_j) (a struct of
+// the form's own, passed to the lane below by shfl_next).  Each owned node goes
+// to emit(f, j, field_j, field_{j+1}) (the latter unused at j = n_cells); after_scan()
 // runs behind the block barrier, when every thread has passed its flush.
 // Covers n_cells + 1 <= 31 R (blockDim/64) nodes.
 // The last thread of the block also reads the control word (a count of
@@ -281,10 +281,10 @@ static __device__ __forceinline__ bool field_build_regs_r(const unsigned long lo
 #pragma unroll
     for (int d = 8; d >= 1; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
     t = __shfl_sync(0xffffffffu, t, 0);
-    auto value = [&](int j, long long S, long long qj) -> Val { return j > Nc ? Val(0) : field_at(j, S, qj); };
+    auto value = [&](int j, long long S, long long qj) -> Val { return field_at(min(j, Nc), S, qj); };
     long long S = g0 + t - s_tot[f * 32 + 16];
     Val Ecur = value(j0, S, q[0]);
-    const Val En = __shfl_down_sync(0xffffffffu, Ecur, 1);
+    const Val En = shfl_next(Ecur);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int j = j0 + r;
@@ -294,7 +294,7 @@ static __device__ __forceinline__ bool field_build_regs_r(const unsigned long lo
             Sn = S + ((j < Nc) ? q[r] + q[(r + 1) % R] : 0ll);
             Enext = value(j + 1, Sn, q[(r + 1) % R]);
         }
-        if (lane != 31 && j <= Nc) emit(f, j, Ecur, Enext, S);
+        if (lane != 31 && j <= Nc) emit(f, j, Ecur, Enext);
         Ecur = Enext;
         S = Sn;
     }

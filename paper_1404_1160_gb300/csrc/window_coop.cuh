@@ -123,6 +123,13 @@ __device__ __forceinline__ unsigned long long hist_node(const unsigned int* h, i
 // One call ends a sweep: the block's histograms into the cycle's words, the
 // table from the words of all blocks, and the histograms and the sweep's
 // counters cleared for the next sweep.  false: a wait ran out of time.
+struct NodeField {
+    double E, rE;
+};
+static __device__ __forceinline__ NodeField shfl_next(const NodeField& v) {
+    return {__shfl_down_sync(0xffffffffu, v.E, 1), v.rE};  // only E is used of the next lane's node
+}
+
 template <int HIST>
 static __device__ __forceinline__ bool field_cycle(int cyc, bool control) {
     __syncthreads();
@@ -130,7 +137,7 @@ static __device__ __forceinline__ bool field_cycle(int cyc, bool control) {
     const int words = Hist<HIST>::kWordsPerNode * Np1;
     unsigned int* hist = (unsigned int*)(smem_raw + s_cyc.hist);
     double2* tab = (double2*)(smem_raw + s_cyc.tabA);
-    const double* inv_r = (const double*)(smem_raw + s_cyc.node_c);
+    const double* node_k = (const double*)(smem_raw + s_cyc.node_c);
     unsigned long long* prev;
     const unsigned long long* Q = cycle_exchange(cyc, control, &prev, [&](int f, int j) {
         return hist_node<HIST>(hist + f * words, Np1, j, s_cyc.W, 2 * words, copies);
@@ -143,27 +150,30 @@ static __device__ __forceinline__ bool field_cycle(int cyc, bool control) {
             s_next = 0;
         }
     };
-    auto field_at = [&](int j, long long S, long long qj) -> double {
-        if (j == c) return s_cyc.parity_odd ? 0.0 : (i64_to_double(qj) * s_cyc.q_unit) * s_cyc.inv_hr;
-        const double e = (i64_to_double(S) * s_cyc.q_half) * inv_r[j];
-        return (s_cyc.parity_odd && j < c) ? -e : e;  // odd reading: rE / |r|
+    // E_j = (S_j q_unit/2) (1/r_j), E_c = (Q_c q_unit) (1/h_r); node_k[c] is 1/h_r,
+    // and with the odd reading (rE / |r|) 0 there and -1/r_j left of it.  One
+    // code path for all nodes.
+    auto field_at = [&](int j, long long S, long long qj) -> NodeField {
+        NodeField v;
+        v.rE = i64_to_double(j == c ? qj : S) * (j == c ? s_cyc.q_unit : s_cyc.q_half);
+        v.E = v.rE * node_k[j];
+        return v;
     };
     auto slope = [&](double d) -> double {
         // d / W: exponent shift when the result stays normal (exact), else multiply
         const int ex = (int)((__double_as_longlong(d) >> 52) & 0x7ff);
         return (ex > s_cyc.log2W + 1 && ex < 0x7ff) ? scale_pow2(d, -s_cyc.log2W) : d * s_cyc.invW;
     };
-    auto edge = [&](int f, int j, long long S) {
+    auto edge = [&](int f, int j, double rE) {
         // the off-mesh gather divides the edge rE by R: the odd reading
         // (rE / |R|) carries the sign flip in the lower edge value
-        const double rE = i64_to_double(S) * s_cyc.q_half;
         if (j == 0) s_cyc.edges[2 * f] = s_cyc.parity_odd ? -rE : rE;
         if (j == Nc) s_cyc.edges[2 * f + 1] = rE;
     };
     if (field_in_regs(Nc, blockDim.x)) {
-        auto emit = [&](int f, int j, double e, double en, long long S) {
-            tab[f * Np1 + j] = make_double2(e, j < Nc ? slope(en - e) : 0.0);
-            if (j == 0 || j == Nc) edge(f, j, S);
+        auto emit = [&](int f, int j, const NodeField& v, const NodeField& next) {
+            tab[f * Np1 + j] = make_double2(v.E, j < Nc ? slope(next.E - v.E) : 0.0);
+            edge(f, j, v.rE);
         };
         if (!field_build_regs(Q, prev, control, field_at, emit, clear)) return false;
         __syncthreads();
@@ -179,8 +189,9 @@ static __device__ __forceinline__ bool field_cycle(int cyc, bool control) {
     for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
         const int f = idx >= Np1, j = idx - f * Np1;
         const long long S = g[idx] - g[f * Np1 + c];
-        tab[idx].x = field_at(j, S, q[f * Np1 + c]);
-        if (j == 0 || j == Nc) edge(f, j, S);
+        const NodeField v = field_at(j, S, q[f * Np1 + c]);
+        tab[idx].x = v.E;
+        edge(f, j, v.rE);
     }
     __syncthreads();
     clear();
@@ -192,46 +203,63 @@ static __device__ __forceinline__ bool field_cycle(int cyc, bool control) {
     return true;
 }
 
+// The third extremum (roots and resolution) or the window cap at sample k.
+static __device__ __noinline__ int2 track_resolved(const DevParams& P, const WinBufs& B, unsigned int i, int k,
+                                                   double Vold, double Vnew, bool detect_only, int2 tr) {
+    Track s;
+    s.flags = tr.x;
+    if ((tr.x & F_NEXT) == 3) {
+        const double v2 = detect_only ? B.traj[(size_t)(tr.y + 2) * P.n + i].y : B.o[i];
+        const double t1 = (double)tr.y + quad_root01(B.t1[i], B.T[i], v2);
+        s.T = ((double)(k - 2) + quad_root01(B.vp[i], Vold, Vnew)) - t1;
+    } else {
+        s.flags |= F_FB;
+        s.T = P.Tfb;
+    }
+    if (detect_only) {
+        s.flags |= F_RES;
+        s.need = 0;
+    } else {
+        track_resolve(s, P, s.T);
+        B.o[i] = s.o;
+        B.N[i] = s.N;
+    }
+    B.T[i] = s.T;
+    return make_int2(s.flags, s.need);
+}
+
 // Period tracking of one particle at sample k (k >= 1), V_{k-1} = Vold,
 // V_k = Vnew.  A sign change between samples k-1 and k is marked pending
-// and its root taken at sample k+1 from V_{k-1}, V_k, V_{k+1} (V_{k-1} kept
-// in vp when the change is found): the same crossings, stencils and order as
-// testing samples k-2, k-1 at sample k.  tr = (flags, need) is loaded by the
-// caller and updated here.  Returns true when the particle is done.
-__device__ __forceinline__ bool track_update(const DevParams& P, const WinBufs& B, long long i, int k,
+// (V_{k-1} kept in vp) and counted as an extremum at sample k+1, when its
+// stencil V_{k-1}, V_k, V_{k+1} is complete: the same crossings, stencils and
+// order as testing samples k-2, k-1 at sample k.  Only the third extremum
+// evaluates roots: the first one keeps its stencil (in t1, T and o, which
+// the resolution overwrites, and its sample in the word that later holds
+// `need`), the second one needs no time.  A root and a resolution are chains
+// of FP64 divisions, and one particle's holds up its block's sweep and with
+// it every block's cycle; this way no cycle before the first full turn has
+// one.  tr = (flags, need) is loaded by the caller and updated here.
+// Returns true when the particle is done.
+__device__ __forceinline__ bool track_update(const DevParams& P, const WinBufs& B, unsigned int i, int k,
                                              double Vold, double Vnew, bool detect_only, int2& tr) {
     if (!(tr.x & F_RES)) {
-        Track s;
-        s.flags = tr.x;
-        s.t1 = 0.0;
-        s.need = tr.y;
-        bool touched = false;
-        if (s.flags & F_PEND) {
-            const double v0 = B.vp[i];
-            if ((s.flags & F_NEXT) >= 1) s.t1 = B.t1[i];
-            s.flags &= ~F_PEND;
-            track_root(s, P, k, v0, Vold, Vnew, detect_only);
-            if ((s.flags & F_NEXT) == 1 && !(tr.x & F_NEXT)) B.t1[i] = s.t1;
-            touched = true;
-        }
-        if (!(s.flags & F_RES) && positive(Vold) != positive(Vnew)) {
-            s.flags |= F_PEND;
-            B.vp[i] = Vold;
-            touched = true;
-        }
-        if (k == P.Kmax) {
-            track_cap(s, P, detect_only);
-            touched = true;
-        }
-        if (touched) {
-            if (s.flags & F_RES) {
-                B.T[i] = s.T;
-                if (!detect_only) {
-                    B.o[i] = s.o;
-                    B.N[i] = s.N;
+        const bool pend = tr.x & F_PEND, change = positive(Vold) != positive(Vnew);
+        if (pend || change || k == P.Kmax) {
+            if (pend) {
+                tr.x += 1 - F_PEND;
+                if ((tr.x & F_NEXT) == 1) {
+                    B.t1[i] = B.vp[i];
+                    B.T[i] = Vold;
+                    if (!detect_only) B.o[i] = Vnew;  // step 1 alone leaves o as it was; its rows hold the sample
+                    tr.y = k - 2;
                 }
             }
-            tr = make_int2(s.flags, (s.flags & F_RES) && !detect_only ? s.need : tr.y);
+            if ((tr.x & F_NEXT) == 3 || k == P.Kmax) {
+                tr = track_resolved(P, B, i, k, Vold, Vnew, detect_only, tr);
+            } else if (change) {
+                tr.x |= F_PEND;
+                B.vp[i] = Vold;
+            }
             B.tr[i] = tr;
         }
     }
@@ -282,11 +310,6 @@ struct Stage : StageCx<SOLVER> {
 // How a window keeps its chunks: in global memory, loaded directly (0) or
 // through a double buffer per warp (1: the next chunk is in flight while the
 // current one is worked on), or in shared memory for the whole window (2).
-// A resident chunk saves the L2 round trip at the start of every sweep,
-// which a beam with one or two chunks per warp cannot hide.  Measured on
-// GB300 together with one block per SM instead of n/1024 blocks: two RK4 steps
-// of 20000 particles 9.17 -> 5.79 ms, the modified scheme on 150001 8.64 ->
-// 8.07 ms; 10^6 particles do not fit and stay staged (9.5 ms).
 enum WindowStage { STAGE_NONE = 0, STAGE_NEXT = 1, STAGE_RESIDENT = 2 };
 // Chunk buffers a block holds; `chunks`: the chunks of one block.
 __host__ __device__ constexpr size_t stage_buffers(int stage, int block, unsigned int chunks) {
@@ -356,7 +379,7 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
     double2* tab = (double2*)(stage + stage_buffers(STAGE, blockDim.x, (n_chunks + gridDim.x - 1) / gridDim.x));  // 2 Np1
     unsigned int* hist = (unsigned int*)(tab + 2 * Np1);  // copies x 2 fields x words (staged build: also the scan input)
     long long* g = (long long*)(hist + hist_copies_reserved(Nc, copies, blockDim.x) * 2 * hist_slot_words(HIST) * Np1);  // 2 Np1
-    double* inv_r = (double*)(g + cycle_words(Nc, blockDim.x, P.q_cb > 0));  // Np1
+    double* node_k = (double*)(g + cycle_words(Nc, blockDim.x, P.q_cb > 0));  // Np1
     // the region of g holds the last complete charge words of the two slots
     // instead where the field is built in registers
     unsigned long long* prev = (unsigned long long*)g;  // 2 x (2 Np1 + 1)
@@ -364,9 +387,10 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
         for (int i = threadIdx.x; i < 2 * (2 * Np1 + 1); i += blockDim.x) prev[i] = 0ull;
     for (int i = threadIdx.x; i < copies * 2 * words; i += blockDim.x) hist[i] = 0u;
     auto off = [&](const void* p) { return (int)((const unsigned char*)p - smem_raw); };
-    cycle_setup(P, B.Qring, B.bar, B.status, gridDim.x, blockIdx.x, off(hist), off(tab), 0, off(g), off(inv_r));
+    cycle_setup(P, B.Qring, B.bar, B.status, gridDim.x, blockIdx.x, off(hist), off(tab), 0, off(g), off(node_k));
     for (int j = threadIdx.x; j < Np1; j += blockDim.x)
-        inv_r[j] = (j == P.c) ? 0.0 : 1.0 / (P.r_min + (double)j * P.hr);
+        node_k[j] = j == P.c ? (P.parity_odd ? 0.0 : P.inv_hr)
+                             : ((P.parity_odd && j < P.c) ? -1.0 : 1.0) / (P.r_min + (double)j * P.hr);
 
     const bool detect_only = mode == MODE_PERIODS, fine_only = mode == MODE_FINE;
     // Work unit: a chunk of 32 consecutive storage slots (phase-space
