@@ -440,7 +440,6 @@ int init32(pic_handle* h, const double* r0, const double* v0, int ptr_kind) {
     ALLOC(B.y, LD);
     ALLOC(B.tr, LD);
     if (poisson) ALLOC(B.ce, LD);
-    ALLOC(B.t1, N);
     ALLOC(B.T, N);
     ALLOC(B.o, N);
     ALLOC(B.N, N);

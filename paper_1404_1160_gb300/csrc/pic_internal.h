@@ -46,7 +46,7 @@ cudaError_t launch_gather(const DevParams& P, const double* R, long long n, cons
 // interleaved so one 16-byte access moves both).
 struct WinBufs {
     double2* y;                 // current fine sample (R, V)
-    double *t1, *T, *o;         // first extremum, period, remainder (fine steps)
+    double *t1, *T, *o;         // stencil of the first extremum, then period and remainder (fine steps)
     double* vp;                 // V_{k-1} of a sign change found at sample k (its root is taken at k+1)
     int* N;                     // whole periods per macro step
     int2* tr;                   // (Track flags, last sample needed)
@@ -131,7 +131,7 @@ struct WinBufs32 {
     float2* traj;               // rows 1..Kmax: z_k, row k at traj + (k-1)*ld
     unsigned int* tr;           // Track flags | need << 8
     float2* ce;                 // (e1, e3) of the current step, from the second sweep to the first
-    CTime *t1, *T, *o;          // first extremum, period, remainder (fine steps)
+    CTime *T, *o;               // period, remainder (fine steps)
     int* N;                     // whole periods per macro step
     unsigned long long* Qring;  // as WinBufs
     int* notdone;
