@@ -1342,6 +1342,10 @@ cudaError_t batch_upload(pic_batch* b) {
                 cp *= 2;
         }
         d.P.hist_copies = cp;
+        if (d.n_blocks > 0) {
+            const long long units = h->B32.ld / pic::kWindow32Unit;
+            pic::hist32_split(&d.P, (units + d.n_blocks - 1) / d.n_blocks * pic::kWindow32Unit);
+        }
         d.P.q_cb = pic::q_count_bits(h->n, h->dp.W, d.n_blocks,
                                      pic::field_in_regs(h->prm.n_cells, b->block) &&
                                          pic::window32_batch_smem(h->prm.n_cells, cp, b->block, true) <= b->smem);
@@ -1472,11 +1476,11 @@ int batch_configure(pic_batch* b, int block, int bps_want, double power, int cop
     for (int i = 0; i < b->n; ++i) {
         pic_handle* h = b->hs[i];
         const bool coop = h->prm.field_model == PIC_FIELD_POISSON;
-        const long long groups = (h->B32.ld + 127) / 128;
-        need[i] = coop ? (groups + block / 32 - 1) / (block / 32) : (h->n + block - 1) / block;
+        const long long units = h->B32.ld / pic::kWindow32Unit;
+        need[i] = coop ? (units + block / 32 - 1) / (block / 32) : (h->n + block - 1) / block;
         if (need[i] < 1) need[i] = 1;
         // a Poisson beam's blocks deposit at most 2^21 positions each per cycle
-        lo[i] = coop ? std::max(1ll, (groups * 128 + (1ll << 21) - 1) >> 21) : 1;
+        lo[i] = coop ? std::max(1ll, (units * pic::kWindow32Unit + (1ll << 21) - 1) >> 21) : 1;
         if (lo[i] > need[i]) need[i] = lo[i];
         w[i] = (coop ? 1.0 : 0.25) * std::pow((double)(h->n > 0 ? h->n : 1), power);
         wsum += w[i];
@@ -1512,8 +1516,8 @@ int batch_configure(pic_batch* b, int block, int bps_want, double power, int cop
     for (int i = 0; i < b->n; ++i) {
         pic_handle* h = b->hs[i];
         if (h->prm.field_model == PIC_FIELD_POISSON) {
-            const long long groups = (h->B32.ld + 127) / 128;
-            if ((groups + nb[i] - 1) / nb[i] * 128 > (1ll << 21)) return PIC_ERR_UNSUPPORTED;
+            const long long units = h->B32.ld / pic::kWindow32Unit;
+            if ((units + nb[i] - 1) / nb[i] * pic::kWindow32Unit > (1ll << 21)) return PIC_ERR_UNSUPPORTED;
         }
         b->desc[i].first_block = first;
         b->desc[i].n_blocks = (int)nb[i];

@@ -53,6 +53,7 @@ struct DevParams {
     int bar_extra;                     // testing only: arrivals a barrier waits for beyond the grid
     int parity_odd;                    // 1: E = rE(r)/|r| (odd in r, 0 on the axis); 0: E = rE(r)/r
     int hist_copies;                   // copies of each block's charge histogram (window kernel)
+    int hs_a, hs_b, hs_fast;           // FP32 form: how a histogram splits the right weights (hist32_split)
     int q_cb;                          // count bits of the charge words; 0: the cycles end in a grid barrier
     // FP32 form (precision 1): the same quantities rounded once to binary32
     float r_min_f, inv_hr_f, ncells_f, Wf;

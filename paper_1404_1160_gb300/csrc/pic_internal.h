@@ -107,7 +107,7 @@ struct WindowLaunch {
     bool kept = false;        // shared memory for the counted charge words
     int coop_grid = 0, coop_block = 0;
     int hist = 0;             // 0: 32-bit split histograms, 1: 64-bit
-    int stage = 0;            // WindowStage: how the chunks are kept
+    int stage = 0;            // FP64: how the chunks are kept (WindowStage); FP32: the sweep's units (Sweep32)
     size_t coop_smem = 0;
 };
 
@@ -141,6 +141,11 @@ struct WinBufs32 {
     long long ld;               // row stride (slots)
 };
 long long window32_row_stride(long long n);
+constexpr int kWindow32Unit = 64;  // slots of a work unit of a batch's Poisson beams
+// Sets how the histogram words of the FP32 window split the right weights
+// (P->hs_*), for the positions a block deposits into one field per cycle and
+// P->hist_copies copies.
+void hist32_split(DevParams* P, long long positions_per_block);
 // Launch shape of the FP32 window; cudaErrorNotSupported when the mesh does
 // not fit in shared memory or a block would deposit more than 2^21
 // positions per field and cycle.

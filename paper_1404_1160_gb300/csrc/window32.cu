@@ -16,10 +16,10 @@
 //
 // Field cycle (Poisson): as in the FP64 kernel, stages pair up (1,3) and
 // (2,4); each pair is deposited by one sweep into per-block 32-bit
-// histograms, flushed with 64-bit global atomics, and after a grid barrier
-// every block turns the global int64 charge into its own field table of
-// binary32 (E_j, E_{j+1} - E_j), computed in binary32 from the exact int64
-// sums and per-node constants (build_fields32).  Two tables are kept: the
+// histograms, flushed with 64-bit global atomics, and when all blocks have
+// flushed every block turns the global int64 charge into its own field table
+// of binary32 (E_j, E_{j+1} - E_j), computed in binary32 from the exact int64
+// sums and per-node constants (field_cycle32).  Two tables are kept: the
 // one of pair 1 (fields of R1, R3) and the one of pair 2 (R2, R4), so the
 // first sweep of the next step can recompute e1 and e3 instead of reading
 // them back from memory.
@@ -29,39 +29,103 @@
 namespace pic {
 
 constexpr int kW32Threads = 1024;
-constexpr int kG = 4;             // consecutive particles per lane in a group
-constexpr int kGroup = 32 * kG;   // particles per warp group
-constexpr int kHist32Words = 4;   // 32-bit words per node and field
+constexpr int kRowPad = 128;      // rows are padded to a multiple of this many slots
 constexpr int kHist32CopiesMax = 4;  // histogram copies (lane l deposits into copy l mod copies)
 
 // ---------------------------------------------------------------- deposit
+//
+// Block histogram of one field: per cell and copy four 32-bit words, the
+// count C_j and the right weights qR in three parts summed separately,
+// qR = h 2^a + m 2^b + l, so that S_j = H_j 2^a + M_j 2^b + L_j and the node
+// charge is Q_j = W C_j - S_j + S_{j-1}, exactly.  hist32_split picks a and b
+// so that no word overflows for the positions a block deposits into one copy.
+// Every lane adds its own position with plain shared reductions: on this GPU
+// that is several times faster than merging the lanes of a warp that share a
+// cell first (match + reduce), and than 64-bit shared atomics.
+//
+// With W = 2^32 the weight of a position with x = (R - r_min)/h_r >= 1 is a
+// multiple of 2^9, since x - floor(x) is a multiple of 2^-23: such a position
+// (all but those in cell 0) takes its parts from the significand of 1 + f,
+// with b = 9 and l = 0.  On a mesh of 256 cells or more f has 16 bits or
+// fewer for most of the beam, so the middle part is 0 as well where h holds
+// 16 bits (up to 65536 positions per copy) and two reductions remain of the
+// four that a fixed 11/11/10-bit split with its count took.
+__host__ __device__ constexpr long long hist32_positions_max() { return 1ll << 21; }
 
-// Block histogram of one field: per cell j the count C_j and the right
-// weights qR split in 11/11/10-bit parts summed separately (A_j, B_j, C'_j),
-// so every word stays exact while a block deposits at most 2^21 positions
-// per field and cycle; S_j = A_j + 2^11 B_j + 2^22 C'_j and the node charge
-// is Q_j = W C_j - S_j + S_{j-1}.  Every lane adds its own position with
-// plain shared atomics: on this GPU that is several times faster than
-// merging the lanes of a warp that share a cell first (match + reduce), and
-// than 64-bit shared atomics.
-__device__ __forceinline__ void deposit32(unsigned int* h, int Np1, int j, unsigned int qR) {
-    const bool ok = j >= 0;
-    unsigned int* hj = h + (ok ? j : 0);
-    const unsigned int a = qR & 0x7ffu, b = (qR >> 11) & 0x7ffu, c = qR >> 22;
-    if (ok) atomicAdd(hj, 1u);
-    if (ok && a) atomicAdd(hj + Np1, a);
-    if (ok && b) atomicAdd(hj + 2 * Np1, b);
-    if (ok && c) atomicAdd(hj + 3 * Np1, c);
+void hist32_split(DevParams* P, long long positions_per_block) {
+    const long long M = (positions_per_block + P->hist_copies - 1) / P->hist_copies;
+    int m = 0;
+    while ((1ll << m) < M) ++m;
+    const int s = m > 9 ? m - 9 : 0;  // bits of the middle part: M 2^(23 - s) <= 2^32
+    if (m <= 20) {                    // M 2^s <= 2^32 too
+        P->hs_a = 9 + s;
+        P->hs_b = 9;
+        P->hs_fast = P->log2W == 32 ? 1 : 0;
+    } else {                          // 11/11/10 bits
+        P->hs_a = 21;
+        P->hs_b = 10;
+        P->hs_fast = 0;
+    }
 }
 
-// deposit32 of a cell known to be on the mesh (j >= 0)
-__device__ __forceinline__ void deposit32_on(unsigned int* h, int Np1, int j, unsigned int qR) {
-    unsigned int* hj = h + j;
-    const unsigned int a = qR & 0x7ffu, b = (qR >> 11) & 0x7ffu, c = qR >> 22;
-    atomicAdd(hj, 1u);
-    if (a) atomicAdd(hj + Np1, a);
-    if (b) atomicAdd(hj + 2 * Np1, b);
-    if (c) atomicAdd(hj + 3 * Np1, c);
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ float2 lds_f2(uint32_t a) {
+    float2 v;
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
+    return v;
+}
+// The sweeps' accesses to the histograms; block barriers separate them from
+// the flush and the clearing, so no memory clobber is needed.
+__device__ __forceinline__ void red_shared(uint32_t a, unsigned int v) {
+    asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v));
+}
+
+// The histograms of a stage pair as the lanes of a warp see them: byte
+// address of word w of cell j of this lane's copy = a (or b) + 4 jb + w plane,
+// with jb = kFloorBits + j.  Layout: copies x 2 fields x 4 words x (n_cells +
+// 1), so that the lanes of a warp meet different banks in different cells;
+// n_cells + 1 is odd, so a cell's words lie 8, 16 and 24 banks on in the
+// other copies.  (One 16-byte word per cell, four times fewer addresses, took
+// 46.7 instead of 43.5 ms on 2 10^7 particles: a reduction then meets only
+// every fourth bank.)
+struct Hist32 {
+    uint32_t a, b, plane;
+    int hs_a, hs_b;
+    unsigned int lim;   // fast form: bits(x) - bits(1) below this; 0: never
+};
+constexpr unsigned int kFloorBits = 0x4B000000u;  // bits of 2^23
+constexpr unsigned int kOneBits = 0x3F800000u;    // bits of 1
+
+// floor(x) as kFloorBits + j, and f = x - j (exact), for 0 <= x < 2^22: one
+// add rounded down in place of a floor and a conversion on the slow pipe.
+__device__ __forceinline__ unsigned int floor_bits(float x, float& f) {
+    const float t = __fadd_rd(x, 8388608.0f);
+    f = x - (t - 8388608.0f);
+    return __float_as_uint(t);
+}
+
+// fast form (see above)
+__device__ __forceinline__ void deposit32_fast(const Hist32& H, uint32_t base, float x) {
+    float f;
+    const unsigned int jb = floor_bits(x, f);
+    const unsigned int g = __float_as_uint(1.0f + f);  // exact: 1 <= x, so f is a multiple of 2^-23
+    const int s = H.hs_a - 9;
+    const uint32_t c = base + (jb << 2);
+    const unsigned int lo = g & ((1u << s) - 1u);
+    red_shared(c, 1u);
+    red_shared(c + H.plane, (g >> s) - (kOneBits >> s));
+    if (lo) red_shared(c + 2 * H.plane, lo);
+}
+
+__device__ __forceinline__ void deposit32(const Hist32& H, uint32_t base, const Cell32& c) {
+    if (c.j < 0) return;
+    const uint32_t w = base + ((kFloorBits + (unsigned int)c.j) << 2);
+    const unsigned int h = c.qR >> H.hs_a, m = (c.qR >> H.hs_b) & ((1u << (H.hs_a - H.hs_b)) - 1u),
+                       l = c.qR & ((1u << H.hs_b) - 1u);
+    red_shared(w, 1u);
+    if (h) red_shared(w + H.plane, h);
+    if (m) red_shared(w + 2 * H.plane, m);
+    if (l) red_shared(w + 3 * H.plane, l);
 }
 
 // ------------------------------------------ located pairs, warp-uniform path
@@ -69,84 +133,70 @@ __device__ __forceinline__ void deposit32_on(unsigned int* h, int Np1, int j, un
 // Nearly every warp has all its positions on the mesh.  The pair helpers
 // below test that once per pair of positions (one warp vote) and then run
 // the cell arithmetic without the off-mesh selects, the gather without the
-// edge division and the deposit without the on-mesh test; a warp with a lane
-// off the mesh (or at a NaN) runs the general locate32t / gather32 /
-// deposit32.  Both give the same cells, weights, fields and words.  Every
-// lane of the warp must make the call.
+// edge division and the deposit in its fast form; a warp with a lane off the
+// mesh (or at a NaN; for the deposits also in cell 0) runs the general
+// locate32t / gather32 / deposit32.  Both give the same cells, weights,
+// fields and sums.  Every lane of the warp must make the call.
 
-// Cell of an on-mesh x = (R - r_min)/h_r, 0 <= x < n_cells: the general
-// locate32t with its test known true.
-template <bool NEED_Q>
-__device__ __forceinline__ Cell32 cell_on_mesh(const DevParams& P, float x) {
-    const float fl = floorf(x);
-    const float f = x - fl;
-    Cell32 c;
-    c.j = (int)fl;
-    c.a = f;
-    c.qR = NEED_Q ? __float2uint_rz(f * P.Wf) : 0u;
-    return c;
-}
-
-// true when every lane of the warp has both positions on the mesh
-__device__ __forceinline__ bool warp_on_mesh(const DevParams& P, float xa, float xb) {
-    const bool in = xa >= 0.0f && xa < P.ncells_f && xb >= 0.0f && xb < P.ncells_f;
-    return __all_sync(0xffffffffu, in);
-}
-
-// Fields at Ra (table ta, edges ed[0..1]) and Rb (table tb, edges ed[2..3]).
-__device__ __forceinline__ void locate_gather2(const DevParams& P, float Ra, float Rb, const float2* ta,
-                                               const float2* tb, const float* ed, float& ea, float& eb) {
+// Fields at Ra (first table at ta, edges ed[0..1]) and Rb (second table tw
+// bytes on, edges ed[2..3]).
+__device__ __forceinline__ void locate_gather2(const DevParams& P, float Ra, float Rb, const float2* tab, int Np1,
+                                               const float* ed, float& ea, float& eb) {
     const float xa = (Ra - P.r_min_f) * P.inv_hr_f, xb = (Rb - P.r_min_f) * P.inv_hr_f;
-    if (warp_on_mesh(P, xa, xb)) {
-        const Cell32 ca = cell_on_mesh<false>(P, xa), cb = cell_on_mesh<false>(P, xb);
-        const float2 va = ta[ca.j], vb = tb[cb.j];
-        ea = fmaf(ca.a, va.y, va.x);
-        eb = fmaf(cb.a, vb.y, vb.x);
+    const unsigned int lim = __float_as_uint(P.ncells_f);  // as unsigned, negatives and NaN lie above
+    if (__all_sync(0xffffffffu, __float_as_uint(xa) < lim && __float_as_uint(xb) < lim)) {
+        float fa, fb;
+        const unsigned int ja = floor_bits(xa, fa), jb = floor_bits(xb, fb);
+        const uint32_t t = smem_u32(tab) - (kFloorBits << 3);
+        const float2 va = lds_f2(t + (ja << 3)), vb = lds_f2(t + 8u * (unsigned int)Np1 + (jb << 3));
+        ea = fmaf(fa, va.y, va.x);
+        eb = fmaf(fb, vb.y, vb.x);
     } else {
         const Cell32 ca = locate32t<false>(P, Ra), cb = locate32t<false>(P, Rb);
-        ea = gather32(ta, ed[0], ed[1], ca);
-        eb = gather32(tb, ed[2], ed[3], cb);
+        ea = gather32(tab, ed[0], ed[1], ca);
+        eb = gather32(tab + Np1, ed[2], ed[3], cb);
     }
 }
 
-// Deposits Ra into ha and Rb into hb when `valid`.
-__device__ __forceinline__ void locate_deposit2(const DevParams& P, float Ra, float Rb, unsigned int* ha,
-                                                unsigned int* hb, int Np1, bool valid) {
+// Deposits Ra into the first histogram and Rb into the second when `valid`.
+__device__ __forceinline__ void locate_deposit2(const DevParams& P, const Hist32& H, float Ra, float Rb, bool valid) {
     const float xa = (Ra - P.r_min_f) * P.inv_hr_f, xb = (Rb - P.r_min_f) * P.inv_hr_f;
-    if (warp_on_mesh(P, xa, xb)) {
-        const Cell32 ca = cell_on_mesh<true>(P, xa), cb = cell_on_mesh<true>(P, xb);
+    if (__all_sync(0xffffffffu, __float_as_uint(xa) - kOneBits < H.lim && __float_as_uint(xb) - kOneBits < H.lim)) {
         if (valid) {
-            deposit32_on(ha, Np1, ca.j, ca.qR);
-            deposit32_on(hb, Np1, cb.j, cb.qR);
+            deposit32_fast(H, H.a, xa);
+            deposit32_fast(H, H.b, xb);
         }
     } else {
         const Cell32 ca = locate32(P, Ra), cb = locate32(P, Rb);
         if (valid) {
-            deposit32(ha, Np1, ca.j, ca.qR);
-            deposit32(hb, Np1, cb.j, cb.qR);
+            deposit32(H, H.a, ca);
+            deposit32(H, H.b, cb);
         }
     }
 }
 
-__device__ __forceinline__ unsigned long long hist32_S(const unsigned int* h, int Np1, int j) {
-    return (unsigned long long)h[Np1 + j] + ((unsigned long long)h[2 * Np1 + j] << 11) +
-           ((unsigned long long)h[3 * Np1 + j] << 22);
-}
-
-// Node charge from the `copies` copies of a field's histogram, `stride`
-// words apart.
-__device__ __forceinline__ unsigned long long hist32_node(const unsigned int* h, int Np1, int j, long long W,
-                                                          int copies, int stride) {
-    unsigned long long C = 0, Sj = 0, Sm = 0;
-    for (int cp = 0; cp < copies; ++cp) {
-        const unsigned int* hc = h + cp * stride;
-        if (j < Np1 - 1) {
-            C += hc[j];
-            Sj += hist32_S(hc, Np1, j);
+// Node charge Q_j = W C_j - S_j + S_{j-1} of one field from its histogram.  The
+// lanes of a warp hold consecutive nodes, so S_{j-1} is the lane's below (the
+// first lane reads it).  Every lane of the warp calls this.
+__device__ __forceinline__ unsigned long long hist32_node(const unsigned int* h, int Np1, int j, int copies) {
+    const int a = s_cyc.hs_a, b = s_cyc.hs_b;
+    auto cell = [&](int m, unsigned int& C) -> unsigned long long {
+        unsigned long long H = 0, M = 0, L = 0;
+        for (int cp = 0; cp < copies; ++cp) {
+            const unsigned int* w = h + cp * 8 * Np1 + m;
+            C += w[0];
+            H += w[Np1];
+            M += w[2 * Np1];
+            L += w[3 * Np1];
         }
-        if (j >= 1) Sm += hist32_S(hc, Np1, j - 1);
-    }
-    return C * (unsigned long long)W - Sj + Sm;
+        return (H << a) + (M << b) + L;
+    };
+    unsigned int C = 0, none = 0;
+    const unsigned long long S = j < Np1 - 1 ? cell(j, C) : 0ull;
+    unsigned long long Sm = __shfl_up_sync(0xffffffffu, S, 1);
+    if (j == 0) Sm = 0ull;
+    else if ((threadIdx.x & 31) == 0) Sm = cell(j - 1, none);
+    return (unsigned long long)C * (unsigned long long)s_cyc.W - S + Sm;
 }
 
 // Field tables of one cycle from its global charge: exact int64 trapezoid
@@ -165,7 +215,7 @@ __device__ __forceinline__ unsigned long long hist32_node(const unsigned int* h,
 // histograms and the sweep's counters cleared for the next sweep.  false: a
 // wait ran out of time.
 static __device__ __forceinline__ void clear_hist32(unsigned int* hist, int words) {
-    // 16-byte stores: the region starts aligned and holds a multiple of four words
+    // 16-byte stores: the region starts aligned and holds a multiple of eight words
     for (int i = threadIdx.x; i < words / 4; i += blockDim.x) ((uint4*)hist)[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 struct NodeField32 {
@@ -178,18 +228,17 @@ static __device__ __forceinline__ NodeField32 shfl_next(const NodeField32& v) {
 static __device__ __forceinline__ bool field_cycle32(int cyc, int pair, bool control) {
     __syncthreads();
     const int Nc = s_cyc.n_cells, Np1 = Nc + 1, c = s_cyc.c, copies = s_cyc.copies;
-    const int hw = kHist32Words * Np1;
     unsigned int* hist = (unsigned int*)(smem_raw + s_cyc.hist);
     float2* tab = (float2*)(smem_raw + (pair ? s_cyc.tabB : s_cyc.tabA));
     float* edges = edges32(pair);
     const float* cq = (const float*)(smem_raw + s_cyc.node_c);
     unsigned long long* prev;
     const unsigned long long* Q = cycle_exchange(cyc, control, &prev, [&](int f, int j) {
-        return hist32_node(hist + f * hw, Np1, j, s_cyc.W, copies, 2 * hw);
+        return hist32_node(hist + f * 4 * Np1, Np1, j, copies);
     });
     if (!Q) return false;
     auto clear = [&]() {
-        clear_hist32(hist, copies * 2 * hw);
+        clear_hist32(hist, copies * 8 * Np1);
         if (threadIdx.x == 0) {
             s_cnt = 0;
             s_next = 0;
@@ -310,74 +359,66 @@ __device__ __forceinline__ bool track32_update(const DevParams& P, const WinBufs
 
 // ------------------------------------------------ cooperative Poisson window
 
-struct Grp32 {
-    float4 z0, z1;  // (R, V) of the lane's 4 consecutive particles
-    float4 e0, e1;  // (e1, e3) of the same particles, carried from the second sweep
-    uint4 tr;
+// G consecutive slots of one lane: (R, V) or (e1, e3) pairs.
+template <int G>
+__device__ __forceinline__ void load_pairs(const float2* p, float (&v)[2 * G]) {
+    if constexpr (G == 1) {
+        const float2 a = *p;
+        v[0] = a.x;
+        v[1] = a.y;
+    } else {
+        const float4 a = *(const float4*)p;
+        v[0] = a.x;
+        v[1] = a.y;
+        v[2] = a.z;
+        v[3] = a.w;
+    }
+}
+template <int G>
+__device__ __forceinline__ void store_pairs(float2* p, const float (&v)[2 * G]) {
+    if constexpr (G == 1) *p = make_float2(v[0], v[1]);
+    else *(float4*)p = make_float4(v[0], v[1], v[2], v[3]);
+}
+template <int G>
+__device__ __forceinline__ void load_words(const unsigned int* p, unsigned int (&v)[G]) {
+    if constexpr (G == 1) {
+        v[0] = *p;
+    } else {
+        static_assert(G == 2, "one or two slots per lane");
+        const uint2 a = *(const uint2*)p;
+        v[0] = a.x;
+        v[1] = a.y;
+    }
+}
+
+// What sweep A reads of a unit's slots of one lane.
+template <int G>
+struct UnitIn {
+    float z[2 * G], e[2 * G];
+    unsigned int tr[G];
 };
-
-__device__ __forceinline__ void load_grp(const float2* src, const unsigned int* tr, const float2* ce, long long base,
-                                         bool with_tr, bool with_ce, Grp32& G) {
-    const float4* p = (const float4*)(src + base);
-    G.z0 = p[0];
-    G.z1 = p[1];
-    if (with_tr) G.tr = *(const uint4*)(tr + base);
-    if (with_ce) {
-        const float4* c = (const float4*)(ce + base);
-        G.e0 = c[0];
-        G.e1 = c[1];
-    }
-}
-
-__device__ __forceinline__ float grp_e(const Grp32& G, int c) {
-    switch (c) {
-        case 0: return G.e0.x;
-        case 1: return G.e0.y;
-        case 2: return G.e0.z;
-        case 3: return G.e0.w;
-        case 4: return G.e1.x;
-        case 5: return G.e1.y;
-        case 6: return G.e1.z;
-        default: return G.e1.w;
-    }
-}
-
-__device__ __forceinline__ float grp_get(const Grp32& G, int c) {
-    switch (c) {
-        case 0: return G.z0.x;
-        case 1: return G.z0.y;
-        case 2: return G.z0.z;
-        case 3: return G.z0.w;
-        case 4: return G.z1.x;
-        case 5: return G.z1.y;
-        case 6: return G.z1.z;
-        default: return G.z1.w;
-    }
-}
-
-__device__ __forceinline__ unsigned int grp_tr(const Grp32& G, int q) {
-    return q == 0 ? G.tr.x : (q == 1 ? G.tr.y : (q == 2 ? G.tr.z : G.tr.w));
-}
 
 // Shared memory of the FP32 window kernel (bytes).
 static size_t coop32_smem_bytes(int n_cells, int copies, int block, bool kept) {
     const size_t Np1 = (size_t)n_cells + 1;
-    return (size_t)copies * 2 * kHist32Words * Np1 * sizeof(unsigned int)  // histograms; also the int64 scan input
+    return (size_t)copies * 8 * Np1 * sizeof(unsigned int)  // histograms; also the int64 scan input
            + 4 * Np1 * sizeof(float2)                     // tables of pair 1 and pair 2
            + cycle_words(n_cells, block, kept) * sizeof(long long)  // kept charge words, or scan output, then E
            + Np1 * sizeof(float);                         // field constants
 }
 
 // The window of one beam on blocks lb = 0..nb-1 of its own (the whole grid
-// for a single beam, or a beam's share of a batch).
+// for a single beam, or a beam's share of a batch), G slots per lane and unit.
+// AHEAD: the next unit's loads are issued before the current unit is worked on.
+template <int G, bool AHEAD>
 __device__ __forceinline__ void window32_coop_body(const DevParams& P, const WinBufs32& B, int mode, int T_known,
                                                    long long n_fine, const CTime* __restrict__ Tin, int lb, int nb) {
+    constexpr unsigned int U = 32 * G;  // slots of a unit
     const int Nc = P.n_cells, Np1 = Nc + 1;
-    const int hw = kHist32Words * Np1;
     const int copies = P.hist_copies;
-    unsigned int* hist = (unsigned int*)smem_raw;  // copies x 2 fields x hw words
-    float2* tabA = (float2*)(hist + copies * 2 * hw);  // 2 Np1: fields of R1, R3
-    float2* tabB = tabA + 2 * Np1;                  // 2 Np1: fields of R2, R4
+    unsigned int* hist = (unsigned int*)smem_raw;    // copies x 2 fields x 4 words x Np1 cells
+    float2* tabA = (float2*)(hist + copies * 8 * Np1);  // 2 Np1: fields of R1, R3
+    float2* tabB = tabA + 2 * Np1;                   // 2 Np1: fields of R2, R4
     // scan output of the staged build (2 Np1), or the last complete charge
     // words of the two slots where the field is built in registers
     long long* g = (long long*)(tabB + 2 * Np1);
@@ -385,7 +426,7 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
     float* cq = (float*)(g + cycle_words(Nc, blockDim.x, P.q_cb > 0));  // Np1
     if (P.q_cb)
         for (int i = threadIdx.x; i < 2 * (2 * Np1 + 1); i += blockDim.x) prev[i] = 0ull;
-    clear_hist32(hist, copies * 2 * hw);
+    clear_hist32(hist, copies * 8 * Np1);
     auto off = [&](const void* p) { return (int)((const unsigned char*)p - smem_raw); };
     cycle_setup(P, B.Qring, B.bar, B.status, nb, lb, off(hist), off(tabA), off(tabB), off(g), off(cq));
     for (int j = threadIdx.x; j < Np1; j += blockDim.x)
@@ -393,36 +434,37 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
                            : (float)(((P.parity_odd && j < P.c) ? -P.q_half : P.q_half) / (P.r_min + (double)j * P.hr));
 
     const bool detect_only = mode == MODE_PERIODS, fine_only = mode == MODE_FINE, track = !fine_only;
-    const long long n = P.n, ld = B.ld;
-    const int lane = threadIdx.x & 31;
-    // Work unit: a group of 128 consecutive storage slots, lane l holding
-    // slots 4l..4l+3.  Block b owns the groups g = b (mod grid); its warps
-    // take them dynamically, in alternating directions from one sweep to
-    // the next so that the first groups a sweep reads are the last ones the
-    // previous sweep touched (still in L2).
-    const long long n_groups = ld / kGroup;
-    const long long my_groups = (long long)lb < n_groups ? (n_groups - 1 - (long long)lb) / nb + 1 : 0;
+    const unsigned int n = (unsigned int)P.n, ld = (unsigned int)B.ld;  // below 2^31
+    const unsigned int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
+    // Work unit: U consecutive storage slots, lane l holding slots G l ..
+    // G l + G - 1.  Block b owns the units u = b (mod grid); a warp's first
+    // unit of a sweep is its own number, the next ones come from the counter,
+    // in alternating directions from one sweep to the next so that the first
+    // units a sweep reads are the last ones the previous sweep touched (still
+    // in L2).
+    const unsigned int n_units = ld / U;
+    const unsigned int my_units = (unsigned int)lb < n_units ? (n_units - 1 - lb) / nb + 1 : 0;
     bool rev = false;
-    auto grab = [&]() -> long long {
-        int m = 0;
+    auto grab = [&]() -> unsigned int {
+        unsigned int m = 0;
         if (lane == 0) m = atomicAdd(&s_next, 1);
-        m = __shfl_sync(0xffffffffu, m, 0);
-        if (m >= my_groups) return -1;
-        const long long mm = rev ? my_groups - 1 - m : m;
-        return (long long)lb + mm * nb;
+        return n_warps + __shfl_sync(0xffffffffu, m, 0);
     };
-    auto row = [&](long long k) -> float2* {
+    auto base_of = [&](unsigned int m) -> unsigned int {
+        return (lb + (rev ? my_units - 1 - m : m) * nb) * U + lane * G;
+    };
+    auto row = [&](unsigned int k) -> float2* {
         if (fine_only) return (k & 1) ? B.traj : B.y;
         return k == 0 ? B.y : B.traj + (size_t)(k - 1) * ld;
     };
     // Every slot is read and written by its own block only (set-up, sweeps and
     // landing alike): blocks exchange nothing but the charge words.
-    const int my_slots = (int)my_groups * kGroup;
-    auto slot_of = [&](int s) -> long long { return ((long long)lb + (long long)(s / kGroup) * nb) * kGroup + s % kGroup; };
+    const unsigned int my_slots = my_units * U;
+    auto slot_of = [&](unsigned int s) -> unsigned int { return (lb + (s / U) * nb) * U + s % U; };
 
     if (!fine_only) {
-        for (int s = threadIdx.x; s < my_slots; s += blockDim.x) {
-            const long long i = slot_of(s);
+        for (unsigned int s = threadIdx.x; s < my_slots; s += blockDim.x) {
+            const unsigned int i = slot_of(s);
             if (i >= n) break;
             if (T_known) {
                 int flags = 0;
@@ -441,9 +483,13 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
     int K = 0;
     // lane l deposits into copy l mod copies: the lanes of a warp hold
     // phase-space neighbours, which mostly fall into the same cell
-    unsigned int* histA = hist + (lane & (copies - 1)) * 2 * hw;
-    unsigned int* histB = histA + hw;
-
+    Hist32 H;
+    H.a = smem_u32(hist + (lane & (copies - 1)) * 8 * Np1) - (kFloorBits << 2);
+    H.b = H.a + 16u * (unsigned int)Np1;
+    H.plane = 4u * (unsigned int)Np1;
+    H.hs_a = P.hs_a;
+    H.hs_b = P.hs_b;
+    H.lim = P.hs_fast ? __float_as_uint(P.ncells_f) - kOneBits : 0u;
     __syncthreads();
 
     // half-steps: sweep A(k), cycle, sweep B(k), cycle (one copy of the cycle's code)
@@ -451,91 +497,107 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
         const int k = hs >> 1;
         const float2 rb = P.rot[rot_index(P, 2ll * k)];      // Phi(t_k)
         const float2 rp = P.rot[rot_index(P, 2ll * k + 1)];  // Phi(t_k + h/2)
-        Grp32 cur;
         if (!(hs & 1)) {
-        // ---- sweep A(k): finish step k-1 (write row k), sample k, deposit stage pair 1 of step k
-        const bool last_fine = fine_only && k == n_fine;
-        float2 ra = rb, rm = rp;
-        if (k > 0) {
-            ra = P.rot[rot_index(P, 2ll * k - 2)];  // Phi(t_{k-1})
-            rm = P.rot[rot_index(P, 2ll * k - 1)];  // Phi(t_{k-1} + h/2)
-        }
-        const float2* src = row(k > 0 ? k - 1 : 0);
-        float2* dst = last_fine ? B.y : row(k);
-        unsigned int cnt = 0;
-        for (long long gi = grab(); gi >= 0; gi = grab()) {
-            const long long base = gi * kGroup + lane * kG;
-            load_grp(src, B.tr, B.ce, base, track, k > 0, cur);
-            float zo[2 * kG];
-#pragma unroll
-            for (int q = 0; q < kG; ++q) {
-                const long long i = base + q;
-                const bool valid = i < n;
-                float zR = grp_get(cur, 2 * q), zV = grp_get(cur, 2 * q + 1);
-                if (k > 0) {
-                    const float R3 = rot_R(rm, zR, zV);
-                    const float e1 = grp_e(cur, 2 * q), e3 = grp_e(cur, 2 * q + 1);
-                    float e2, e4;
-                    locate_gather2(P, lawson32_R2(P, R3, e1), lawson32_R4(P, rb, zR, zV, e3), tabB, tabB + Np1,
-                                   edges32(1), e2, e4);
-                    const float Vold = rot_V(ra, zR, zV);
-                    lawson32_update(P, ra, rm, rb, e1, e2, e3, e4, zR, zV);
-                    if (track && valid) {
-                        unsigned int trw = grp_tr(cur, q);
-                        const bool done =
-                            track32_update(P, B, i, k, Vold, rot_V(rb, zR, zV), detect_only, trw);
-                        cnt += done ? 0u : 1u;
-                    }
-                } else if (track && valid) {
-                    cnt += 1u;
-                }
-                if (last_fine) {
-                    // the state leaves the rotating frame: y = Phi(t_k) z
-                    zo[2 * q] = rot_R(rb, zR, zV);
-                    zo[2 * q + 1] = rot_V(rb, zR, zV);
-                    continue;
-                }
-                zo[2 * q] = zR;
-                zo[2 * q + 1] = zV;
-                // stage pair 1 of step k: R1 = (Phi(t_k) z)_R, R3 = (Phi(t_k + h/2) z)_R
-                locate_deposit2(P, rot_R(rb, zR, zV), rot_R(rp, zR, zV), histA, histB, Np1, valid);
-            }
+            // ---- sweep A(k): finish step k-1 (write row k), sample k, deposit stage pair 1 of step k
+            const bool last_fine = fine_only && k == n_fine;
+            float2 ra = rb, rm = rp;
             if (k > 0) {
-                float4* o = (float4*)(dst + base);
-                o[0] = make_float4(zo[0], zo[1], zo[2], zo[3]);
-                o[1] = make_float4(zo[4], zo[5], zo[6], zo[7]);
+                ra = P.rot[rot_index(P, 2ll * k - 2)];  // Phi(t_{k-1})
+                rm = P.rot[rot_index(P, 2ll * k - 1)];  // Phi(t_{k-1} + h/2)
             }
-        }
-        rev = !rev;
-        if (last_fine) break;
-        if (track) {
-            cnt = __reduce_add_sync(0xffffffffu, cnt);
-            if (lane == 0 && cnt) atomicAdd(&s_cnt, (int)cnt);
-        }
-        } else {
-        // ---- sweep B(k): gather pair 1 of step k, deposit stage pair 2
-        const float2 rq = P.rot[rot_index(P, 2ll * k + 2)];  // Phi(t_k + h)
-        const float2* srcB = row(k);
-        for (long long gi = grab(); gi >= 0; gi = grab()) {
-            const long long base = gi * kGroup + lane * kG;
-            load_grp(srcB, nullptr, nullptr, base, false, false, cur);
-            float eo[2 * kG];
+            const float2* src = row(k > 0 ? k - 1 : 0);
+            float2* dst = last_fine ? B.y : row(k);
+            unsigned int cnt = 0;
+            UnitIn<G> in;
+            auto fetch = [&](unsigned int m) {
+                const unsigned int b = base_of(m);
+                load_pairs<G>(src + b, in.z);
+                if (k > 0) load_pairs<G>(B.ce + b, in.e);
+                if (track) load_words<G>(B.tr + b, in.tr);
+            };
+            unsigned int m = warp;
+            if (AHEAD && m < my_units) fetch(m);
+            while (m < my_units) {
+                const unsigned int base = base_of(m);
+                if (!AHEAD) fetch(m);
+                UnitIn<G> cur = in;
+                float(&z)[2 * G] = cur.z;
+                float(&e)[2 * G] = cur.e;
+                unsigned int(&tr)[G] = cur.tr;
+                if (AHEAD) {
+                    m = grab();
+                    if (m < my_units) fetch(m);
+                }
 #pragma unroll
-            for (int q = 0; q < kG; ++q) {
-                const bool valid = base + q < n;
-                const float zR = grp_get(cur, 2 * q), zV = grp_get(cur, 2 * q + 1);
-                const float R3 = rot_R(rp, zR, zV);
-                float e1, e3;
-                locate_gather2(P, rot_R(rb, zR, zV), R3, tabA, tabA + Np1, edges32(0), e1, e3);
-                eo[2 * q] = e1;
-                eo[2 * q + 1] = e3;
-                locate_deposit2(P, lawson32_R2(P, R3, e1), lawson32_R4(P, rq, zR, zV, e3), histA, histB, Np1, valid);
+                for (int q = 0; q < G; ++q) {
+                    const unsigned int i = base + q;
+                    const bool valid = i < n;
+                    float zR = z[2 * q], zV = z[2 * q + 1];
+                    if (k > 0) {
+                        const float R3 = rot_R(rm, zR, zV);
+                        const float e1 = e[2 * q], e3 = e[2 * q + 1];
+                        float e2, e4;
+                        locate_gather2(P, lawson32_R2(P, R3, e1), lawson32_R4(P, rb, zR, zV, e3), tabB, Np1,
+                                       edges32(1), e2, e4);
+                        const float Vold = rot_V(ra, zR, zV);
+                        lawson32_update(P, ra, rm, rb, e1, e2, e3, e4, zR, zV);
+                        if (track && valid)
+                            cnt += track32_update(P, B, i, k, Vold, rot_V(rb, zR, zV), detect_only, tr[q]) ? 0u : 1u;
+                    } else if (track && valid) {
+                        cnt += 1u;
+                    }
+                    if (last_fine) {
+                        // the state leaves the rotating frame: y = Phi(t_k) z
+                        z[2 * q] = rot_R(rb, zR, zV);
+                        z[2 * q + 1] = rot_V(rb, zR, zV);
+                        continue;
+                    }
+                    z[2 * q] = zR;
+                    z[2 * q + 1] = zV;
+                    // stage pair 1 of step k: R1 = (Phi(t_k) z)_R, R3 = (Phi(t_k + h/2) z)_R
+                    locate_deposit2(P, H, rot_R(rb, zR, zV), rot_R(rp, zR, zV), valid);
+                }
+                if (k > 0) store_pairs<G>(dst + base, z);
+                if (!AHEAD) m = grab();
             }
-            float4* o = (float4*)(B.ce + base);
-            o[0] = make_float4(eo[0], eo[1], eo[2], eo[3]);
-            o[1] = make_float4(eo[4], eo[5], eo[6], eo[7]);
-        }
-        rev = !rev;
+            rev = !rev;
+            if (last_fine) break;
+            if (track) {
+                cnt = __reduce_add_sync(0xffffffffu, cnt);
+                if (lane == 0 && cnt) atomicAdd(&s_cnt, (int)cnt);
+            }
+        } else {
+            // ---- sweep B(k): gather pair 1 of step k, deposit stage pair 2
+            const float2 rq = P.rot[rot_index(P, 2ll * k + 2)];  // Phi(t_k + h)
+            const float2* srcB = row(k);
+            float zn[2 * G];
+            unsigned int m = warp;
+            if (AHEAD && m < my_units) load_pairs<G>(srcB + base_of(m), zn);
+            while (m < my_units) {
+                const unsigned int base = base_of(m);
+                float z[2 * G], e[2 * G];
+                if (!AHEAD) load_pairs<G>(srcB + base, zn);
+#pragma unroll
+                for (int q = 0; q < 2 * G; ++q) z[q] = zn[q];
+                if (AHEAD) {
+                    m = grab();
+                    if (m < my_units) load_pairs<G>(srcB + base_of(m), zn);
+                }
+#pragma unroll
+                for (int q = 0; q < G; ++q) {
+                    const bool valid = base + q < n;
+                    const float zR = z[2 * q], zV = z[2 * q + 1];
+                    const float R3 = rot_R(rp, zR, zV);
+                    float e1, e3;
+                    locate_gather2(P, rot_R(rb, zR, zV), R3, tabA, Np1, edges32(0), e1, e3);
+                    e[2 * q] = e1;
+                    e[2 * q + 1] = e3;
+                    locate_deposit2(P, H, lawson32_R2(P, R3, e1), lawson32_R4(P, rq, zR, zV, e3), valid);
+                }
+                store_pairs<G>(B.ce + base, e);
+                if (!AHEAD) m = grab();
+            }
+            rev = !rev;
         }
         const bool control = !(hs & 1) && track;
         if (!field_cycle32(cyc++, hs & 1, control)) return;
@@ -549,8 +611,8 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
     if (mode != MODE_ETD) return;
 
     // ---- landing (step 3) and extrapolation (step 4); row k holds z_k
-    for (int s = threadIdx.x; s < my_slots; s += blockDim.x) {
-        const long long i = slot_of(s);
+    for (unsigned int s = threadIdx.x; s < my_slots; s += blockDim.x) {
+        const unsigned int i = slot_of(s);
         if (i >= n) break;
         const CTime o = B.o[i], T = B.T[i];
         const int N = B.N[i];
@@ -580,9 +642,10 @@ __device__ __forceinline__ void window32_coop_body(const DevParams& P, const Win
     }
 }
 
+template <int G, bool AHEAD>
 __global__ void __launch_bounds__(kW32Threads, 1) k_window32_coop(DevParams P, WinBufs32 B, int mode, int T_known,
                                                                   long long n_fine, const CTime* __restrict__ Tin) {
-    window32_coop_body(P, B, mode, T_known, n_fine, Tin, blockIdx.x, gridDim.x);
+    window32_coop_body<G, AHEAD>(P, B, mode, T_known, n_fine, Tin, blockIdx.x, gridDim.x);
 }
 
 // ------------------------------------------- per-particle window (analytic E)
@@ -812,6 +875,8 @@ __global__ void __launch_bounds__(256) k_window32_local(DevParams P, WinBufs32 B
 
 // ------------------------------------------------------------- batched form
 
+constexpr int kBatchG = kWindow32Unit / 32;
+
 // One cooperative launch advances every beam of a batch by one macro step:
 // each block finds its beam, copies the beam's descriptor to shared memory
 // and runs that beam's window on the beam's own blocks (its barriers count
@@ -837,7 +902,7 @@ __global__ void __launch_bounds__(kW32Threads, 1) k_window32_batch(const BeamDes
     __syncthreads();
     const int lb = (int)blockIdx.x - D.first_block;
     if (threadIdx.x == 0) atomicMin(&D.t_ns[0], (unsigned long long)global_ns());
-    if (D.coop) window32_coop_body(D.P, D.B, MODE_ETD, D.T_known, 0, D.Tin, lb, D.n_blocks);
+    if (D.coop) window32_coop_body<kBatchG, false>(D.P, D.B, MODE_ETD, D.T_known, 0, D.Tin, lb, D.n_blocks);
     else if (D.P.field == 1) window32_local_body<1>(D.P, D.B, MODE_ETD, D.T_known, 1, D.Tin, lb, D.n_blocks);
     else window32_local_body<2>(D.P, D.B, MODE_ETD, D.T_known, 1, D.Tin, lb, D.n_blocks);
     __syncthreads();  // the block's last thread is done before its end time
@@ -961,44 +1026,65 @@ __global__ void k_moments32(DevParams P, WinBufs32 B, double* part_d, long long*
 
 // ------------------------------------------------------------- launchers
 
+// Work units of a sweep: how many slots a lane takes at once, and whether the
+// next unit is loaded ahead.
+enum Sweep32 { SWEEP_1 = 0, SWEEP_2 = 1, SWEEP_2_AHEAD = 2 };
+static void* coop32_fn(int sweep) {
+    if (sweep == SWEEP_1) return (void*)k_window32_coop<1, false>;
+    return sweep == SWEEP_2 ? (void*)k_window32_coop<2, false> : (void*)k_window32_coop<2, true>;
+}
+
 cudaError_t window32_prepare(DevParams& P, int block, int blocks_per_sm, int sm_count, long long ld,
                              WindowLaunch* L) {
     L->coop_block = block;
-    // histogram copies: as many as fit (up to kHist32CopiesMax) while a block
-    // deposits enough positions per cycle for same-cell conflicts to matter
+    // Histogram copies (up to kHist32CopiesMax) relieve same-cell conflicts as
+    // long as a block deposits at least 512 positions per copy and cycle; their
+    // sums and clearing cost the cycle 2 n_cells words per copy, so copies x
+    // n_cells stays within 2048.  Windows with 1 / 2 / 4 copies on GB300: 10^6 on
+    // 256 cells 3.74 / 3.51 / 3.46 ms, 4 10^5 2.50 / 2.42 / 2.42, 1.5 10^5 1.90 /
+    // 1.90 / 1.95; 2 10^6 on 1024 cells 6.77 / 6.76 / 7.45, 2 10^7 47.6 / 42.6 / 42.5.
     int copies = kHist32CopiesMax;
     const long long per_block_est = P.n / (sm_count > 0 ? sm_count : 1);
-    while (copies > 1 && (coop32_smem_bytes(P.n_cells, copies, block, false) > 200 * 1024 || per_block_est < 64ll * copies * 32))
+    while (copies > 1 && (coop32_smem_bytes(P.n_cells, copies, block, false) > 200 * 1024 ||
+                          copies * P.n_cells > 2048 || per_block_est < 512ll * copies))
         copies >>= 1;
     P.hist_copies = copies;
     L->kept = field_in_regs(P.n_cells, block) && coop32_smem_bytes(P.n_cells, copies, block, true) <= kWindowSmemMax;
     L->coop_smem = coop32_smem_bytes(P.n_cells, copies, block, L->kept);
     L->hist = 0;
-    L->stage = 0;
+    // One slot per lane while a warp has up to four such units (the tail of a
+    // sweep is a unit, and a unit a chain of latencies); two beyond; and once
+    // the 20 bytes per slot that a sweep reads outgrow half of L2 (64 MB),
+    // loads one unit ahead.  Windows with SWEEP_1 / SWEEP_2 / SWEEP_2_AHEAD: 2 10^4
+    // 1.82 / 2.01 / 2.07 ms, 4 10^5 2.42 / 2.52 / 2.58, 10^6 3.49 / 3.46 / 3.60, 2 10^6 (1024
+    // cells) 7.14 / 6.76 / 6.78, 6 10^6 17.9 / 14.8 / 13.9, 2 10^7 55.4 / 42.6 / 38.9.
+    const long long warps = (long long)sm_count * (block / 32);
+    const int sweep = P.n <= 128 * warps ? SWEEP_1 : (20 * P.n <= (64ll << 20) ? SWEEP_2 : SWEEP_2_AHEAD);
+    const int unit = sweep == SWEEP_1 ? 32 : 64;
+    L->stage = sweep;
     if (L->coop_smem > 227 * 1024) return cudaErrorNotSupported;
-    cudaError_t e = cudaFuncSetAttribute(k_window32_coop, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(coop32_fn(sweep), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)L->coop_smem);
     if (e != cudaSuccess) return e;
     int bps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_window32_coop, block, L->coop_smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, coop32_fn(sweep), block, L->coop_smem);
     if (e != cudaSuccess) return e;
     if (bps < 1) return cudaErrorInvalidConfiguration;
     const int want = blocks_per_sm > 0 ? blocks_per_sm : 1;
     if (want < bps) bps = want;
-    const long long n_groups = ld / kGroup;
-    const long long warps = block / 32;
-    const long long need_blocks = (n_groups + warps - 1) / warps;
+    const long long n_units = ld / unit;
     long long grid = (long long)bps * sm_count;
-    if (need_blocks < grid) grid = need_blocks < 1 ? 1 : need_blocks;
+    if (n_units < grid) grid = n_units < 1 ? 1 : n_units;
     L->coop_grid = (int)grid;
     // the 32-bit histogram words stay exact up to 2^21 positions per block,
     // field and cycle
-    const long long per_block = (n_groups + grid - 1) / grid * kGroup;
-    if (per_block > (1ll << 21)) return cudaErrorNotSupported;
+    const long long per_block = (n_units + grid - 1) / grid * unit;
+    if (per_block > hist32_positions_max()) return cudaErrorNotSupported;
+    hist32_split(&P, per_block);
     return cudaSuccess;
 }
 
-long long window32_row_stride(long long n) { return (n + kGroup - 1) / kGroup * kGroup; }
+long long window32_row_stride(long long n) { return (n + kRowPad - 1) / kRowPad * kRowPad; }
 
 cudaError_t launch_window32_coop(const DevParams& P, const WinBufs32& B, const WindowLaunch& L, int mode,
                                  int T_known, long long n_fine, cudaStream_t st, long long* launches,
@@ -1007,7 +1093,7 @@ cudaError_t launch_window32_coop(const DevParams& P, const WinBufs32& B, const W
     Pc.q_cb = q_count_bits(P.n, P.W, (long long)L.coop_grid + P.bar_extra, L.kept);
     WinBufs32 Bc = B;
     void* args[] = {&Pc, &Bc, &mode, &T_known, &n_fine, &Tin};
-    cudaError_t e = cudaLaunchCooperativeKernel((void*)k_window32_coop, dim3(L.coop_grid), dim3(L.coop_block), args,
+    cudaError_t e = cudaLaunchCooperativeKernel(coop32_fn(L.stage), dim3(L.coop_grid), dim3(L.coop_block), args,
                                                 L.coop_smem, st);
     if (launches) ++*launches;
     return e;

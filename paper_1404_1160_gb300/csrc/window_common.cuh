@@ -95,6 +95,7 @@ struct CycleCtx {
     float q_half_f;
     int n_cells, c, log2W, parity_odd;
     int copies;                  // histogram copies
+    int hs_a, hs_b;              // FP32 form: split of the right weights
     int q_cb;                    // count bits of the words; 0: barrier form
     int n_blocks, expect, lb;    // blocks that share the words, arrivals of one use, this block's index
     int hist, tabA, tabB, g, node_c;  // byte offsets in the dynamic shared memory
@@ -127,6 +128,8 @@ static __device__ __forceinline__ void cycle_setup(const DevParams& P, unsigned 
     s_cyc.log2W = P.log2W;
     s_cyc.parity_odd = P.parity_odd;
     s_cyc.copies = P.hist_copies;
+    s_cyc.hs_a = P.hs_a;
+    s_cyc.hs_b = P.hs_b;
     s_cyc.q_cb = P.q_cb;
     s_cyc.n_blocks = n_blocks;
     s_cyc.expect = n_blocks + P.bar_extra;
@@ -323,13 +326,17 @@ static __device__ __forceinline__ void stage_charge(const unsigned long long* Q,
 }
 
 // Adds this block's charge of every node, node(f, j), and with `control` its
-// not-done count to a slot (see above).
+// not-done count to a slot (see above).  Every lane of a warp calls node (the
+// lanes hold consecutive nodes; past the end the last one).
 template <class Node>
 static __device__ __forceinline__ void flush_charge(unsigned long long* Q, bool control, Node node) {
     const int Nc = s_cyc.n_cells, Np1 = Nc + 1, cb = s_cyc.q_cb;
-    for (int idx = threadIdx.x; idx < 2 * Np1; idx += blockDim.x) {
+    for (int first = threadIdx.x & ~31; first < 2 * Np1; first += blockDim.x) {
+        const int mine = first + (threadIdx.x & 31);
+        const int idx = min(mine, 2 * Np1 - 1);
         const int f = idx >= Np1, j = idx - f * Np1;
         const unsigned long long v = node(f, j);
+        if (mine != idx) continue;
         unsigned long long* w = Q + (size_t)f * q_field_words(Nc) + q_node(j);
         if (cb) atomicAdd(w, (v << cb) + 1ull);
         else if (v) atomicAdd(w, v);

@@ -111,3 +111,43 @@ def test_fp64_ways_to_keep_the_chunks(n, kw, solver):
     assert P == Pc and bit_equal(R, Rc) and bit_equal(V, Vc)
     assert bit_equal(pic.pic_get_periods(h)[2], o)  # step 1 alone leaves the last macro step's remainders
     pic.pic_destroy(h)
+
+
+@pytest.mark.parametrize("n", [32, 3000, 100_000, 700_000, 2_000_000])
+@pytest.mark.parametrize("n_cells", [256, 100, 1024])
+def test_fp32_deposit_forms_agree(n, n_cells):
+    # a warp with an off-mesh lane deposits in the general form, another one in
+    # the fast form: the same particles give the same bits in both.  Every
+    # second slot of run B holds a far particle (off the mesh for these few
+    # steps); twice the charge keeps the charge unit.
+    rng = np.random.default_rng(n + n_cells)
+    R0 = rng.uniform(-3.7, 3.9, n)
+    V0 = rng.normal(0, 0.5, n)
+    far = np.where(np.arange(2 * n) % 2 == 0, 100.0, 0.0)
+    RB, VB = far.copy(), np.zeros(2 * n)
+    RB[1::2], VB[1::2] = R0, V0
+    out = []
+    for R, V, charge in ((R0, V0, 1.0), (RB, VB, 2.0)):
+        p = pic.pic_default_params(precision=1, n_cells=n_cells, sort_every=0, total_charge=charge)
+        h = pic.pic_init(p, R, V)
+        pic.pic_fine_steps(h, 3)
+        out.append(pic.pic_get_particles(h))
+        pic.pic_destroy(h)
+    (Ra, Va), (Rb, Vb) = out
+    assert np.array_equal(Ra, Rb[1::2]) and np.array_equal(Va, Vb[1::2])
+
+
+def test_fp32_blocks_past_the_parts_of_the_fast_split():
+    # more than 2^20 positions per block and copy: the 11/11/10-bit split
+    n = (1 << 20) + 4096
+    rng = np.random.default_rng(3)
+    R0, V0 = rng.normal(0, 1, n), rng.normal(0, 1, n)
+    kw = dict(precision=1, steps_per_turn=4, max_window_steps=10, r_min=-8.0, r_max=8.0)
+    a = etd(pic.pic_default_params(**kw), R0, V0)
+    params = [pic.pic_default_params(**kw)]
+    b = pic.pic_batch_create(params + [pic.pic_default_params(precision=1, field_model=pic.PIC_FIELD_ZERO)] * 151,
+                             [(R0, V0)] + [(np.ones(1), np.ones(1))] * 151)
+    pic.pic_batch_step(b, 1)  # 152 beams on 152 blocks: the large one has a single block
+    R, V = pic.pic_batch_get_particles(b, 0)
+    b.close()
+    assert np.array_equal(R, a[0]) and np.array_equal(V, a[1])
