@@ -64,14 +64,24 @@ struct WinBufs {
 };
 
 // Global charge words of one field cycle ("slot"): two fields of n_cells + 1
-// nodes and one control word.  Four consecutive nodes share a 32-byte sector
-// and every sector has a 128-byte line of its own: the adds and loads of
-// neighbouring lanes travel as one sector request, and the sectors spread
-// over the L2 slices.
+// nodes and one control word.  Four consecutive nodes share a 32-byte sector,
+// so the adds and loads of neighbouring lanes travel as one sector request;
+// the sectors lie 1 KB apart, which spreads the adds of all blocks best over
+// the L2 slices.  Windows on GB300 by that distance, 128 B / 256 B / 512 B / 1 KB /
+// 4 KB: FP32 2 10^4 particles 1.83 / 1.69 / 1.71 / 1.58 / 1.59 ms, 10^6 3.46 / 3.29 /
+// 3.27 / 3.22 / 3.19; two FP64 steps of 20000 4.49 / 4.14 / 4.26 / 4.15 / 4.20; FP64
+// 10^6 8.90 / 8.74 / 8.79 / 8.74 / 8.76.  (One node per 128 B 1.96, 3.68, 4.75, 8.88;
+// 16 nodes per 128 B 2.36, 4.10, 5.72, 9.42.)
 constexpr int kQSlots = 3;
-__host__ __device__ constexpr size_t q_node(int j) { return ((size_t)(j >> 2) << 4) + (size_t)(j & 3); }
-__host__ __device__ constexpr size_t q_field_words(int n_cells) { return ((size_t)(n_cells >> 2) + 1) << 4; }
+__host__ __device__ constexpr size_t q_node(int j) { return ((size_t)(j >> 2) << 7) + (size_t)(j & 3); }
+__host__ __device__ constexpr size_t q_field_words(int n_cells) { return ((size_t)(n_cells >> 2) + 1) << 7; }
 __host__ __device__ constexpr size_t q_slot_words(int n_cells) { return 2 * q_field_words(n_cells) + 16; }
+// Word idx of the 2 (n_cells + 1) + 1 words of a slot that are in use.
+__host__ __device__ constexpr size_t q_used(int n_cells, int idx) {
+    return idx <= n_cells ? q_node(idx)
+                          : (idx <= 2 * n_cells + 1 ? q_field_words(n_cells) + q_node(idx - n_cells - 1)
+                                                    : 2 * q_field_words(n_cells));
+}
 // Whether a block of `block` threads builds the field from the nodes in
 // registers (at most 4 nodes per thread, 31 of every 32 threads, half a
 // block per field) or stages them in shared memory.

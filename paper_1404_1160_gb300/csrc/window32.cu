@@ -914,8 +914,10 @@ __global__ void k_batch_reset(const BeamDesc32* __restrict__ beams, int n_beams)
     if (b >= n_beams) return;
     const BeamDesc32& D = beams[b];
     if (D.coop) {
-        const size_t q = (size_t)kQSlots * q_slot_words(D.P.n_cells);
-        for (size_t i = threadIdx.x; i < q; i += blockDim.x) D.B.Qring[i] = 0ull;
+        const int Nc = D.P.n_cells;
+        for (int s = 0; s < kQSlots; ++s)
+            for (int i = threadIdx.x; i < 2 * Nc + 3; i += blockDim.x)
+                D.B.Qring[s * q_slot_words(Nc) + q_used(Nc, i)] = 0ull;
         for (int i = threadIdx.x; i < 64; i += blockDim.x) D.B.bar[i] = 0u;
     }
     if (threadIdx.x == 0) {

@@ -350,8 +350,8 @@ static __device__ __forceinline__ void flush_charge(unsigned long long* Q, bool 
 
 // Barrier form: clears the slot of the cycle after (one block does).
 static __device__ __forceinline__ void clear_slot(unsigned long long* Q) {
-    const size_t words = q_slot_words(s_cyc.n_cells);
-    for (size_t i = threadIdx.x; i < words; i += blockDim.x) Q[i] = 0ull;
+    const int Nc = s_cyc.n_cells;
+    for (int i = threadIdx.x; i < 2 * Nc + 3; i += blockDim.x) Q[q_used(Nc, i)] = 0ull;
 }
 
 // Barrier of the n_blocks blocks that share s_cyc.bar (the whole grid, or the
