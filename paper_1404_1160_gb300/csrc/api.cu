@@ -940,10 +940,11 @@ int pic_get_field(pic_handle* h, int64_t* Q, double* E, double* rE_edges, int64_
     if (e == cudaSuccess && rE_edges)
         e = cudaMemcpyAsync(rE_edges, h->edges_f, sizeof(double) * 2, kind_from(ptr_kind), h->st);
     if (e == cudaSuccess && n_out) e = cudaMemcpyAsync(n_out, h->nout_f, sizeof(long long), kind_from(ptr_kind), h->st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(h->status_host, h->S.status, sizeof(int), cudaMemcpyDeviceToHost, h->st);
+    const bool waits = !pic::poisson_in_block(h->dp.n_cells);
+    if (e == cudaSuccess && waits) e = cudaMemcpyAsync(h->status_host, h->S.status, sizeof(int), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     if (e != cudaSuccess) return map_cuda(e);
-    return map_dev(*h->status_host);
+    return waits ? map_dev(*h->status_host) : PIC_OK;
 }
 
 int pic_moments(pic_handle* h, pic_moments_t* out) {
@@ -1176,18 +1177,21 @@ int pic_deposit_f32(const pic_params* p, int64_t n, const float* R_dev, int64_t*
 }  // extern "C"
 
 // Shared body of pic_poisson and pic_poisson_noalloc: S is the caller's
-// scratch (flags, tile counter and status are cleared here, on the stream).
+// scratch (flags, tile counter and status are cleared here, on the stream),
+// null for the meshes that need none.
 int pic::poisson_with_scratch(const pic_params* p, int64_t n_particles, const int64_t* Q_dev, double* E_dev,
                               double* rE_edges_dev, const pic::ScanScratch* S, void* stream) {
     int rc = check_params(p, true);
     if (rc) return rc;
-    if (n_particles <= 0 || !Q_dev || !E_dev || !rE_edges_dev || !S) return PIC_ERR_INVALID_ARG;
+    const bool in_block = rc == PIC_OK && pic::poisson_in_block(p->n_cells);
+    if (n_particles <= 0 || !Q_dev || !E_dev || !rE_edges_dev || (!S && !in_block)) return PIC_ERR_INVALID_ARG;
     if ((double)n_particles * (double)p->weight_fixed >= 4.611686018427388e18) return PIC_ERR_OVERFLOW;
     int sms = 0;
     if ((rc = current_sm_count(&sms))) return rc;
     DevParams d;
     make_devparams(p, n_particles, &d);
     cudaStream_t st = (cudaStream_t)stream;
+    if (in_block) return map_cuda(pic::launch_poisson(d, (const long long*)Q_dev, E_dev, rE_edges_dev, pic::ScanScratch(), st, nullptr));
     int status = 0;
     cudaError_t e = pic::launch_poisson(d, (const long long*)Q_dev, E_dev, rE_edges_dev, *S, st, nullptr);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&status, S->status, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -1203,6 +1207,8 @@ int pic_poisson(const pic_params* p, int64_t n_particles, const int64_t* Q_dev, 
     int rc = check_params(p, true);
     if (rc) return rc;
     if (n_particles <= 0 || !Q_dev || !E_dev || !rE_edges_dev) return PIC_ERR_INVALID_ARG;
+    if (pic::poisson_in_block(p->n_cells))
+        return pic::poisson_with_scratch(p, n_particles, Q_dev, E_dev, rE_edges_dev, nullptr, stream);
     cudaStream_t st = (cudaStream_t)stream;
     const int tiles = (p->n_cells + pic::kScanTile - 1) / pic::kScanTile;
     const size_t bytes = pic::scan_scratch_layout(p->n_cells, tiles, nullptr, nullptr);

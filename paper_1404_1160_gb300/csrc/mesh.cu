@@ -83,10 +83,123 @@ __global__ void k_deposit32(DevParams P, const float* __restrict__ R, long long 
     }
 }
 
-// ------------------------------------------------- decoupled look-back scan
+// Split form of the deposit: W <= 2^32 and at most kSplitPositions positions
+// per block.  Three 32-bit words per cell (count, low and high 16 bits of the
+// right weights) stay exact for that many positions, and 32-bit shared
+// reductions replace two 64-bit shared atomics per position; lane l deposits
+// into copy l mod copies.  A block is a whole SM's threads, so that few blocks
+// add to the mesh in global memory, and four positions per thread are in
+// flight.  Deposits of 10^6 positions on 256 cells: 12.2 us in the 64-bit form
+// (608 blocks of 256 threads), see launch_deposit.
+constexpr int kSplitThreads = 1024;
+constexpr long long kSplitPositions = 65536;
+constexpr int kSplitAhead = 4;
 
-__device__ __forceinline__ void st_release_s32(int* p, int v) {
-    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+__device__ __forceinline__ void split_add(unsigned int* h, int n_cells, int j, unsigned int q) {
+    atomicAdd(&h[j], 1u);
+    if (q & 0xffffu) atomicAdd(&h[n_cells + j], q & 0xffffu);
+    if (q >> 16) atomicAdd(&h[2 * n_cells + j], q >> 16);
+}
+
+template <class Real, class Locate>
+__device__ __forceinline__ void deposit_split(const DevParams& P, const Real* __restrict__ R, unsigned int n,
+                                              int r_stride, unsigned long long* __restrict__ Q,
+                                              unsigned long long* __restrict__ n_out, int copies, Locate locate) {
+    extern __shared__ unsigned int split_hist[];  // copies x 3 x n_cells
+    const int Nc = P.n_cells;
+    for (int i = threadIdx.x; i < copies * 3 * Nc; i += blockDim.x) split_hist[i] = 0u;
+    __syncthreads();
+    unsigned int* h = split_hist + (threadIdx.x & (copies - 1)) * 3 * Nc;
+    unsigned int out = 0;
+    const unsigned int stride = gridDim.x * blockDim.x;
+    for (unsigned long long i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (unsigned long long)kSplitAhead * stride) {
+        Real r[kSplitAhead];
+#pragma unroll
+        for (int k = 0; k < kSplitAhead; ++k) {
+            const unsigned long long m = i + (unsigned long long)k * stride;
+            r[k] = m < n ? R[m * r_stride] : Real(0);
+        }
+#pragma unroll
+        for (int k = 0; k < kSplitAhead; ++k) {
+            if (i + (unsigned long long)k * stride >= n) break;
+            int j;
+            const unsigned int q = locate(r[k], j);
+            if (j >= 0) split_add(h, Nc, j, q);
+            else ++out;
+        }
+    }
+    out = __reduce_add_sync(0xffffffffu, out);
+    if ((threadIdx.x & 31) == 0 && out) atomicAdd(n_out, (unsigned long long)out);
+    __syncthreads();
+    // node charge Q_j = W C_j - S_j + S_{j-1}
+    for (int j = threadIdx.x; j <= Nc; j += blockDim.x) {
+        unsigned long long v = 0;
+        for (int c = 0; c < copies; ++c) {
+            const unsigned int* w = split_hist + c * 3 * Nc;
+            if (j < Nc)
+                v += (unsigned long long)w[j] * (unsigned long long)P.W -
+                     (((unsigned long long)w[2 * Nc + j] << 16) + w[Nc + j]);
+            if (j > 0) v += ((unsigned long long)w[2 * Nc + j - 1] << 16) + w[Nc + j - 1];
+        }
+        if (v) atomicAdd(&Q[j], v);
+    }
+}
+
+template <int POW2>
+__global__ void __launch_bounds__(kSplitThreads) k_deposit_split(DevParams P, const double* __restrict__ R,
+                                                                 unsigned int n, int r_stride,
+                                                                 unsigned long long* __restrict__ Q,
+                                                                 unsigned long long* __restrict__ n_out, int copies) {
+    deposit_split(P, R, n, r_stride, Q, n_out, copies, [&](double r, int& j) -> unsigned int {
+        const Cell c = mesh_locate<POW2>(P, r);
+        j = c.j;
+        return (unsigned int)c.qR;
+    });
+}
+
+__global__ void __launch_bounds__(kSplitThreads) k_deposit32_split(DevParams P, const float* __restrict__ R,
+                                                                   unsigned int n, int r_stride,
+                                                                   unsigned long long* __restrict__ Q,
+                                                                   unsigned long long* __restrict__ n_out, int copies) {
+    deposit_split(P, R, n, r_stride, Q, n_out, copies, [&](float r, int& j) -> unsigned int {
+        const Cell32 c = locate32(P, r);
+        j = c.j;
+        return c.qR;
+    });
+}
+
+__global__ void k_zero_charge(unsigned long long* __restrict__ Q, int n, unsigned long long* __restrict__ n_out) {
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) Q[j] = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *n_out = 0ull;
+}
+
+// ------------------------------------------------- field of a small mesh, one block
+//
+// S_j = G_j - G_c of every node (see below for G) by one block, R consecutive
+// nodes per thread: no scratch, no status, no second launch up to
+// kFieldFusedCells cells, where the block also evaluates the field (FP64
+// divisions: 8 us on one SM for 512 nodes' worth would be too many beyond).
+// Larger meshes leave S_j in E's own storage for k_field_in_place.
+constexpr int kFieldBlock = 1024;
+constexpr int kFieldBlockCells = 4 * kFieldBlock - 2;
+constexpr int kFieldFusedCells = 512;
+
+__device__ __forceinline__ void field_node(const DevParams& P, const long long* __restrict__ Q, int j, long long S,
+                                           double* __restrict__ E, double* __restrict__ edges) {
+    const int Nc = P.n_cells, c = P.c;
+    double e;
+    if (j == c) {
+        e = P.parity_odd ? 0.0 : ((double)Q[c] * P.q_unit) * P.inv_hr;
+    } else {
+        const double r = P.r_min + (double)j * P.hr;
+        e = ((double)S * P.q_half) * (1.0 / r);
+        if (P.parity_odd && j < c) e = -e;  // odd reading: rE / |r|
+    }
+    E[j] = e;
+    // the off-mesh gather divides the edge rE by R; the odd reading's
+    // lower edge carries the sign flip
+    if (j == 0) edges[0] = P.parity_odd ? -((double)S * P.q_half) : (double)S * P.q_half;
+    if (j == Nc) edges[1] = (double)S * P.q_half;
 }
 
 __device__ __forceinline__ long long warp_incl_scan(long long x) {
@@ -97,6 +210,55 @@ __device__ __forceinline__ long long warp_incl_scan(long long x) {
         if (lane >= d) x += y;
     }
     return x;
+}
+
+template <int R>
+__global__ void __launch_bounds__(kFieldBlock) k_field_block(DevParams P, const long long* __restrict__ Q,
+                                                             double* __restrict__ E, double* __restrict__ edges,
+                                                             int fused) {
+    __shared__ long long s_tot[kFieldBlock / 32], s_c;
+    const int Nc = P.n_cells, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int j0 = threadIdx.x * R;
+    long long q[R + 1];
+#pragma unroll
+    for (int r = 0; r <= R; ++r) q[r] = j0 + r <= Nc ? Q[j0 + r] : 0ll;
+    long long L = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) L += j0 + r < Nc ? q[r] + q[r + 1] : 0ll;
+    const long long incl = warp_incl_scan(L);
+    if (lane == 31) s_tot[w] = incl;
+    __syncthreads();
+    long long t = lane < w ? s_tot[lane] : 0ll;
+#pragma unroll
+    for (int d = 16; d >= 1; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
+    long long g = t + incl - L, run = g;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (j0 + r == P.c) s_c = run;
+        run += j0 + r < Nc ? q[r] + q[r + 1] : 0ll;
+    }
+    __syncthreads();
+    g -= s_c;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int j = j0 + r;
+        if (j > Nc) break;
+        if (fused) field_node(P, Q, j, g, E, edges);
+        else E[j] = __longlong_as_double(g);
+        g += j < Nc ? q[r] + q[r + 1] : 0ll;
+    }
+}
+
+__global__ void k_field_in_place(DevParams P, const long long* __restrict__ Q, double* __restrict__ E,
+                                 double* __restrict__ edges) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j <= P.n_cells) field_node(P, Q, j, __double_as_longlong(E[j]), E, edges);
+}
+
+// ------------------------------------------------- decoupled look-back scan
+
+__device__ __forceinline__ void st_release_s32(int* p, int v) {
+    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 // G_j = sum_{m<j} (Q_m + Q_{m+1}), j = 0..n_cells, in one pass: each block
@@ -188,27 +350,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_pairs(DevParams P, const 
 __global__ void k_field_from_prefix(DevParams P, const long long* __restrict__ Q,
                                     const long long* __restrict__ G, double* __restrict__ E,
                                     double* __restrict__ edges) {
-    const int Nc = P.n_cells, c = P.c;
-    const long long Gc = G[c];
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j <= Nc; j += gridDim.x * blockDim.x) {
-        long long S = G[j] - Gc;
-        double e;
-        if (j == c) {
-            e = P.parity_odd ? 0.0 : ((double)Q[c] * P.q_unit) * P.inv_hr;
-        } else {
-            double r = P.r_min + (double)j * P.hr;
-            e = ((double)S * P.q_half) * (1.0 / r);
-            if (P.parity_odd && j < c) e = -e;  // odd reading: rE / |r|
-        }
-        E[j] = e;
-        // the off-mesh gather divides the edge rE by R; the odd reading's
-        // lower edge carries the sign flip
-        if (j == 0) edges[0] = P.parity_odd ? -((double)S * P.q_half) : (double)S * P.q_half;
-        if (j == Nc) edges[1] = (double)S * P.q_half;
-    }
+    const long long Gc = G[P.c];
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j <= P.n_cells; j += gridDim.x * blockDim.x)
+        field_node(P, Q, j, G[j] - Gc, E, edges);
 }
 
 // ------------------------------------------------------------------ gather
+
+constexpr int kGatherAhead = 4;
 
 template <int POW2>
 __global__ void k_gather(DevParams P, const double* __restrict__ R, long long n,
@@ -223,18 +372,26 @@ __global__ void k_gather(DevParams P, const double* __restrict__ R, long long n,
     }
     const double lo = edges[0], hi = edges[1];
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        Cell c = mesh_locate<POW2>(P, R[i]);
-        double e;
-        if (use_smem) {
-            e = mesh_gather(tab, lo, hi, c.j, c.a);
-        } else if (c.j >= 0) {
-            double ej = E[c.j];
-            e = fma(c.a, (E[c.j + 1] - ej) * P.invW, ej);
-        } else {
-            e = gather_outside(lo, hi, c.j, c.a);
+    // kGatherAhead positions per thread in flight
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kGatherAhead * stride) {
+        double r[kGatherAhead];
+#pragma unroll
+        for (int k = 0; k < kGatherAhead; ++k) r[k] = i + k * stride < n ? R[i + k * stride] : 0.0;
+#pragma unroll
+        for (int k = 0; k < kGatherAhead; ++k) {
+            if (i + k * stride >= n) break;
+            const Cell c = mesh_locate<POW2>(P, r[k]);
+            double e;
+            if (use_smem) {
+                e = mesh_gather(tab, lo, hi, c.j, c.a);
+            } else if (c.j >= 0) {
+                const double ej = E[c.j];
+                e = fma(c.a, (E[c.j + 1] - ej) * P.invW, ej);
+            } else {
+                e = gather_outside(lo, hi, c.j, c.a);
+            }
+            out[i + k * stride] = e;
         }
-        out[i] = e;
     }
 }
 
@@ -295,39 +452,52 @@ cudaError_t launch_unpack(const double2* y, double* R, double* V, long long n, i
     return cudaGetLastError();
 }
 
-cudaError_t launch_deposit(const DevParams& P, const double* R, long long n, int r_stride, long long* Q,
-                           long long* n_out, cudaStream_t st, int sm_count, long long* launches) {
+// Zeroed charge and out-of-mesh count, then the split form where it serves
+// (its histograms of 12 bytes per cell and copy within 48 KB, or 96 KB with one
+// copy), else the 64-bit form.
+template <class Real, class Split, class Wide>
+static cudaError_t deposit_with(Split split_fn, Wide wide_fn, const DevParams& P, const Real* R, long long n, int r_stride,
+                                long long* Q, long long* n_out, cudaStream_t st, int sm_count, long long* launches) {
     const int Np1 = P.n_cells + 1;
-    cudaError_t e = cudaMemsetAsync(Q, 0, sizeof(long long) * (size_t)Np1, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(n_out, 0, sizeof(long long), st);
+    k_zero_charge<<<(Np1 + 255) / 256, 256, 0, st>>>((unsigned long long*)Q, Np1, (unsigned long long*)n_out);
+    if (launches) ++*launches;
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || n == 0) return e;
-    size_t smem = sizeof(unsigned long long) * (size_t)Np1;
-    int use_smem = smem <= 96 * 1024;
-    auto fn = P.xs_fma ? k_deposit<1> : k_deposit<0>;
-    if (use_smem && smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    long long want = (n + 255) / 256;
-    int grid = (int)(want < (long long)sm_count * 4 ? want : (long long)sm_count * 4);
-    fn<<<grid, 256, use_smem ? smem : 0, st>>>(P, R, n, r_stride, (unsigned long long*)Q, (unsigned long long*)n_out,
-                                               use_smem);
+    const size_t per_copy = sizeof(unsigned int) * 3 * (size_t)P.n_cells;
+    if (P.W <= (1ll << 32) && per_copy <= 96 * 1024 && n < (1ll << 31)) {
+        const int copies = 4 * per_copy <= 48 * 1024 ? 4 : (2 * per_copy <= 48 * 1024 ? 2 : 1);
+        const size_t smem = copies * per_copy;
+        if (smem > 48 * 1024) cudaFuncSetAttribute(split_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // one block per SM, and no block beyond its positions: whole rounds of
+        // kSplitThreads positions each
+        const long long rounds = (n + kSplitThreads - 1) / kSplitThreads, most = kSplitPositions / kSplitThreads;
+        long long grid = rounds < sm_count ? rounds : sm_count;
+        if (grid * most < rounds) grid = (rounds + most - 1) / most;
+        split_fn<<<(int)grid, kSplitThreads, smem, st>>>(P, R, (unsigned int)n, r_stride, (unsigned long long*)Q,
+                                                         (unsigned long long*)n_out, copies);
+    } else {
+        const size_t smem = sizeof(unsigned long long) * (size_t)Np1;
+        const int use_smem = smem <= 96 * 1024;
+        if (use_smem && smem > 48 * 1024)
+            cudaFuncSetAttribute(wide_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const long long want = (n + 255) / 256;
+        const int grid = (int)(want < (long long)sm_count * 4 ? want : (long long)sm_count * 4);
+        wide_fn<<<grid, 256, use_smem ? smem : 0, st>>>(P, R, n, r_stride, (unsigned long long*)Q,
+                                                        (unsigned long long*)n_out, use_smem);
+    }
     if (launches) ++*launches;
     return cudaGetLastError();
 }
 
+cudaError_t launch_deposit(const DevParams& P, const double* R, long long n, int r_stride, long long* Q,
+                           long long* n_out, cudaStream_t st, int sm_count, long long* launches) {
+    return P.xs_fma ? deposit_with(k_deposit_split<1>, k_deposit<1>, P, R, n, r_stride, Q, n_out, st, sm_count, launches)
+                    : deposit_with(k_deposit_split<0>, k_deposit<0>, P, R, n, r_stride, Q, n_out, st, sm_count, launches);
+}
+
 cudaError_t launch_deposit32(const DevParams& P, const float* R, long long n, int r_stride, long long* Q,
                              long long* n_out, cudaStream_t st, int sm_count, long long* launches) {
-    const int Np1 = P.n_cells + 1;
-    cudaError_t e = cudaMemsetAsync(Q, 0, sizeof(long long) * (size_t)Np1, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(n_out, 0, sizeof(long long), st);
-    if (e != cudaSuccess || n == 0) return e;
-    size_t smem = sizeof(unsigned long long) * (size_t)Np1;
-    int use_smem = smem <= 96 * 1024;
-    if (use_smem && smem > 48 * 1024) cudaFuncSetAttribute(k_deposit32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    long long want = (n + 255) / 256;
-    int grid = (int)(want < (long long)sm_count * 4 ? want : (long long)sm_count * 4);
-    k_deposit32<<<grid, 256, use_smem ? smem : 0, st>>>(P, R, n, r_stride, (unsigned long long*)Q,
-                                                        (unsigned long long*)n_out, use_smem);
-    if (launches) ++*launches;
-    return cudaGetLastError();
+    return deposit_with(k_deposit32_split, k_deposit32, P, R, n, r_stride, Q, n_out, st, sm_count, launches);
 }
 
 size_t scan_scratch_bytes(int n_cells) {
@@ -360,8 +530,19 @@ size_t scan_scratch_layout(int n_cells, int tiles, void* base, ScanScratch* S) {
     return total;
 }
 
+bool poisson_in_block(int n_cells) { return n_cells <= kFieldBlockCells; }
+
 cudaError_t launch_poisson(const DevParams& P, const long long* Q, double* E, double* edges,
                            const ScanScratch& S, cudaStream_t st, long long* launches) {
+    if (poisson_in_block(P.n_cells)) {
+        const int fused = P.n_cells <= kFieldFusedCells;
+        if (P.n_cells < kFieldBlock) k_field_block<1><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
+        else if (P.n_cells < 2 * kFieldBlock) k_field_block<2><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
+        else k_field_block<4><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
+        if (!fused) k_field_in_place<<<(P.n_cells + 256) / 256, 256, 0, st>>>(P, Q, E, edges);
+        if (launches) *launches += fused ? 1 : 2;
+        return cudaGetLastError();
+    }
     const int tiles = (P.n_cells + kScanTile - 1) / kScanTile;
     cudaError_t e = cudaMemsetAsync((char*)S.flag, 0, S.zero_bytes, st);
     if (e != cudaSuccess) return e;
@@ -381,7 +562,8 @@ cudaError_t launch_gather(const DevParams& P, const double* R, long long n, cons
     auto fn = P.xs_fma ? k_gather<1> : k_gather<0>;
     if (use_smem && smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     long long want = (n + 255) / 256;
-    int grid = (int)(want < (long long)sm_count * 4 ? want : (long long)sm_count * 4);
+    want = (want + kGatherAhead - 1) / kGatherAhead;
+    int grid = (int)(want < (long long)sm_count * 8 ? want : (long long)sm_count * 8);
     fn<<<grid, 256, use_smem ? smem : 0, st>>>(P, R, n, E, edges, out, use_smem);
     if (launches) ++*launches;
     return cudaGetLastError();
@@ -432,5 +614,9 @@ extern "C" int pic_poisson_noalloc(const pic_params* p, int64_t n_particles, con
     if (pic::scan_scratch_layout(p->n_cells, tiles, nullptr, nullptr) > pic::kNoAllocScratchBytes) return PIC_ERR_TOO_LARGE;
     pic::ScanScratch S;
     pic::scan_scratch_layout(p->n_cells, tiles, base, &S);
-    return pic::poisson_with_scratch(p, n_particles, Q_dev, E_dev, rE_edges_dev, &S, stream);
+    const int rc = pic::poisson_with_scratch(p, n_particles, Q_dev, E_dev, rE_edges_dev, &S, stream);
+    // this entry point returns with the field solved for every mesh it takes
+    if (rc == PIC_OK && pic::poisson_in_block(p->n_cells) && cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess)
+        return PIC_ERR_CUDA;
+    return rc;
 }

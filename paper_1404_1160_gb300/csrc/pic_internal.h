@@ -36,6 +36,9 @@ cudaError_t launch_extrapolate_classic(double2* y, const double2* y0, long long 
                                        cudaStream_t st, long long* launches);
 cudaError_t launch_unpack(const double2* y, double* R, double* V, long long n, int sm_count, cudaStream_t st,
                           long long* launches);
+// Whether launch_poisson serves the mesh from one block: it then uses no scratch
+// and has no device-side wait whose status could be read.
+bool poisson_in_block(int n_cells);
 cudaError_t launch_poisson(const DevParams& P, const long long* Q, double* E, double* edges,
                            const ScanScratch& S, cudaStream_t st, long long* launches);
 cudaError_t launch_gather(const DevParams& P, const double* R, long long n, const double* E,

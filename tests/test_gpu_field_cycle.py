@@ -151,3 +151,55 @@ def test_fp32_blocks_past_the_parts_of_the_fast_split():
     R, V = pic.pic_batch_get_particles(b, 0)
     b.close()
     assert np.array_equal(R, a[0]) and np.array_equal(V, a[1])
+
+
+# ------------------------------------------------- standalone mesh operations
+
+
+@pytest.mark.parametrize("n", [1, 1023, 1025, 4097, 152 * 1024 - 1, 700_001])
+@pytest.mark.parametrize("n_cells,log2W", [(2, 32), (100, 32), (1024, 32), (1026, 24), (4094, 32), (8192, 32), (8194, 32), (256, 40)])
+def test_deposit_forms(n, n_cells, log2W):
+    p = pic.pic_default_params(n_cells=n_cells, weight_fixed=1 << log2W)
+    rng = np.random.default_rng(n + n_cells)
+    R = rng.normal(0, 2, n)
+    R[rng.random(n) < 0.3] = 0.01  # many positions in one cell
+    R[:: max(1, n // 7)] = [np.nan, -4.0, 4.0, np.inf, -np.inf, 3.9999999, -0.0][: len(R[:: max(1, n // 7)])] if n < 7 else np.resize(
+        [np.nan, -4.0, 4.0, np.inf, -np.inf, 3.9999999, -0.0], len(R[:: max(1, n // 7)]))
+    Q = torch.full((n_cells + 1,), 5, dtype=torch.int64, device="cuda")
+    n_out = torch.full((1,), 5, dtype=torch.int64, device="cuda")
+    pic.pic_deposit(p, torch.from_numpy(R).cuda(), Q, n_out)
+    Qo, no = oracle.deposit(cfg_of(p), R)
+    assert np.array_equal(Q.cpu().numpy(), Qo) and int(n_out) == no
+    Rf = R.astype(np.float32)
+    pic.pic_deposit_f32(p, torch.from_numpy(Rf).cuda(), Q, n_out)
+    Qo, no = oracle.deposit_f32(cfg_of(p), Rf)
+    assert np.array_equal(Q.cpu().numpy(), Qo) and int(n_out) == no
+
+
+@pytest.mark.parametrize("n_cells", [2, 30, 510, 512, 514, 1022, 1024, 2046, 2048, 4094, 4096])
+@pytest.mark.parametrize("parity", [pic.PIC_PARITY_EVEN, pic.PIC_PARITY_ODD])
+def test_field_from_one_block(n_cells, parity):
+    p = pic.pic_default_params(n_cells=n_cells, field_parity=parity)
+    Q = np.random.default_rng(n_cells).integers(0, 1 << 40, n_cells + 1).astype(np.int64)
+    E = torch.empty(n_cells + 1, dtype=torch.float64, device="cuda")
+    edges = torch.empty(2, dtype=torch.float64, device="cuda")
+    pic.pic_poisson(p, 12345, torch.from_numpy(Q).cuda(), E, edges)
+    _, Eo, eo = oracle.poisson(cfg_of(p), Q, 12345)
+    assert bit_equal(E.cpu().numpy(), Eo) and bit_equal(edges.cpu().numpy(), eo)
+
+
+@pytest.mark.parametrize("n_cells", [2, 6, 512, 1022, 1026, 65536])
+def test_frozen_potential_of_any_mesh(n_cells):
+    # psi at the nodes against long double sums: (n_cells + 4) binary64 roundings of
+    # the largest partial sum bound the run and scan sums of either side
+    p = pic.pic_default_params(n_cells=n_cells)
+    E = np.random.default_rng(n_cells).normal(0, 1, n_cells + 1)
+    hr, c = 8.0 / n_cells, n_cells // 2
+    inc = np.longdouble(0.5 * hr) * (E[:-1].astype(np.longdouble) + E[1:])
+    ref = np.concatenate([-np.cumsum(inc[:c][::-1])[::-1], [0], np.cumsum(inc[c:])])
+    psi = torch.empty(n_cells + 1, dtype=torch.float64, device="cuda")
+    out = torch.empty(1, dtype=torch.float64, device="cuda")
+    pic.pic_frozen_potential(p, torch.from_numpy(E).cuda(), torch.zeros(2, dtype=torch.float64, device="cuda"), psi,
+                             torch.zeros(1, dtype=torch.float64, device="cuda"), out)
+    bound = (n_cells + 4) * 2.0**-53 * float(np.sum(np.abs(inc)))
+    assert np.max(np.abs(psi.cpu().numpy() - ref.astype(np.float64))) <= bound
