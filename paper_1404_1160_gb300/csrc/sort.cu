@@ -50,41 +50,43 @@ __global__ void k_sort_keys(const Y* __restrict__ y, long long n, int* __restric
     }
 }
 
-// Exclusive scan of the bin counts in one block (kSortBins entries).
+// Exclusive scan of the bin counts in one block (kSortBins entries): warp w
+// takes 1024 consecutive bins in eight coalesced 16-byte loads per lane.  (One
+// run of 32 bins per thread, 32 lines per load, took 35 us.)
 __global__ void __launch_bounds__(kSortScanThreads) k_sort_scan(unsigned int* __restrict__ count) {
     __shared__ unsigned int s_warp[kSortScanThreads / 32];
-    constexpr int per = kSortBins / kSortScanThreads;
+    constexpr int per = kSortBins / kSortScanThreads / 4;  // 16-byte words per lane
+    static_assert(per * 4 * kSortScanThreads == kSortBins, "whole words");
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    unsigned int v[per];
-    unsigned int s = 0;
+    uint4* c4 = (uint4*)count + w * per * 32 + lane;
+    uint4 v[per];
+    unsigned int excl[per];
+#pragma unroll
+    for (int q = 0; q < per; ++q) v[q] = c4[q * 32];
+    unsigned int total = 0;
 #pragma unroll
     for (int q = 0; q < per; ++q) {
-        v[q] = count[t * per + q];
-        s += v[q];
-    }
-    unsigned int x = s;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned int y = __shfl_up_sync(0xffffffffu, x, d);
-        if (lane >= d) x += y;
-    }
-    if (lane == 31) s_warp[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        unsigned int y = s_warp[lane];
+        const unsigned int s = v[q].x + v[q].y + v[q].z + v[q].w;
+        unsigned int x = s;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const unsigned int z = __shfl_up_sync(0xffffffffu, y, d);
-            if (lane >= d) y += z;
+            const unsigned int y = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += y;
         }
-        s_warp[lane] = y;
+        excl[q] = total + x - s;
+        total += __shfl_sync(0xffffffffu, x, 31);
     }
+    if (lane == 0) s_warp[w] = total;
     __syncthreads();
-    unsigned int run = x - s + (w > 0 ? s_warp[w - 1] : 0u);
+    const unsigned int before = __reduce_add_sync(0xffffffffu, lane < w ? s_warp[lane] : 0u);
 #pragma unroll
     for (int q = 0; q < per; ++q) {
-        count[t * per + q] = run;
-        run += v[q];
+        uint4 o;
+        o.x = before + excl[q];
+        o.y = o.x + v[q].x;
+        o.z = o.y + v[q].y;
+        o.w = o.z + v[q].z;
+        c4[q * 32] = o;
     }
 }
 
