@@ -89,8 +89,12 @@ __global__ void k_deposit32(DevParams P, const float* __restrict__ R, long long 
 // reductions replace two 64-bit shared atomics per position; lane l deposits
 // into copy l mod copies.  A block is a whole SM's threads, so that few blocks
 // add to the mesh in global memory, and four positions per thread are in
-// flight.  Deposits of 10^6 positions on 256 cells: 12.2 us in the 64-bit form
-// (608 blocks of 256 threads), see launch_deposit.
+// flight.  The 64-bit form (608 blocks of 256 threads, one position at a time)
+// took 12.2 us for 10^6 positions on 256 cells, and stays for the rest.  With
+// the field from one block (10 us in two launches before, and an allocation
+// whose pool a synchronisation had emptied cost 200 us more) and four
+// positions per thread in the gather (12.6 us before), a whole cycle of calls
+// on 10^6 positions takes 24.6 us instead of 57.5.
 constexpr int kSplitThreads = 1024;
 constexpr long long kSplitPositions = 65536;
 constexpr int kSplitAhead = 4;
@@ -177,9 +181,10 @@ __global__ void k_zero_charge(unsigned long long* __restrict__ Q, int n, unsigne
 //
 // S_j = G_j - G_c of every node (see below for G) by one block, R consecutive
 // nodes per thread: no scratch, no status, no second launch up to
-// kFieldFusedCells cells, where the block also evaluates the field (FP64
-// divisions: 8 us on one SM for 512 nodes' worth would be too many beyond).
-// Larger meshes leave S_j in E's own storage for k_field_in_place.
+// kFieldFusedCells cells, where the block also evaluates the field.  Beyond, the
+// ~13 FP64 operations per node (a division among them) would take one SM's
+// pipe longer than a second launch: the block leaves S_j in E's own storage for
+// k_field_in_place.
 constexpr int kFieldBlock = 1024;
 constexpr int kFieldBlockCells = 4 * kFieldBlock - 2;
 constexpr int kFieldFusedCells = 512;
