@@ -326,7 +326,7 @@ typedef struct {
 
 int pic_mlp_num_params(void);
 /* Creates a network with all weights zero, able to train on batches of up to
-   max_batch samples (scratch of ~800 B per sample).  Work runs on stream. */
+   max_batch samples.  Work runs on stream. */
 int pic_mlp_create(int64_t max_batch, void* stream, pic_mlp** out);
 /* Copies PIC_MLP_PARAMS master weights in (and resets the Adam state) or out. */
 int pic_mlp_set_weights(pic_mlp* m, const float* w, int ptr_kind);

@@ -17,11 +17,11 @@
 //   dout = (out - y) / B, dW3 = dout^T bf16(h2), db3 = sum dout,
 //   dz2 = (dout W3) gelu'(z2), dW2 = bf16(dz2)^T bf16(h1), db2 = sum dz2,
 //   dz1 = (bf16(dz2) W2) gelu'(z1), dW1 = dz1^T x, db1 = sum dz1.
-// The per-sample part (forward, dz1, dz2) runs one sample per thread and 128
-// per MMA tile; the weight gradients are reduced over the batch by a second
-// kernel (dW2 on the tensor cores, the samples as the reduction dimension)
-// into per-block partials, which a third kernel sums in a fixed order before
-// the Adam update, so training is reproducible bit for bit.
+// One kernel takes a tile of 128 samples through forward, backward and the
+// tile's weight gradients (dW2 on the tensor cores, the samples as the
+// reduction dimension) into per-block partials; a second one sums them in a
+// fixed order, applies Adam and refreshes the rounded copies, so training is
+// reproducible bit for bit.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -46,25 +46,17 @@ static_assert(kMParams == 4674, "parameter count");
 constexpr int sW1 = 0, sb1 = sW1 + kMHid * kMIn, sb2 = sb1 + kMHid, sW3 = sb2 + kMHid, sb3 = sW3 + kMOut * kMHid,
               kMSmall = sb3 + kMOut;
 
-constexpr int kWgTile = 64;      // samples per staged tile of the weight gradients
-constexpr int kWgMaxBlocks = 256;
+constexpr int kLossHist = 4096;   // batch losses kept on the device between copies to the host
 
 struct MlpDev {
     float *master, *m, *v;
     __nv_bfloat16* W2b;   // [j][k]
     __nv_bfloat16* W2Tb;  // [k][j]
     float* small;         // kMSmall
-    // training scratch for up to max_batch samples
-    float* xs;            // [B][5]
-    float* dz1;           // [B][64]
-    float* dz2;           // [B][64]
-    __nv_bfloat16* h1b;   // [B][64]
-    __nv_bfloat16* h2b;   // [B][64]
-    float* dout;          // [B][2]
-    float* loss_part;     // per forward block
-    float* grad_part;     // [kWgMaxBlocks][kMParams]
+    float* loss_part;     // per training block
+    float* grad_part;     // [training blocks][kMParams]
     float* grad;          // [kMParams]
-    float* loss;          // [1]
+    float* loss;          // [kLossHist]
     int* err;             // set by a tensor-core wait that ran out of time
 };
 
@@ -91,33 +83,8 @@ struct AdamArgs {
     int apply;                            // 0: gradients only
 };
 
-// Sums the partials of n_part blocks in block order, writes the gradient and
-// the batch loss, applies Adam to the masters and refreshes the rounded copies.
-__global__ void k_mlp_update(MlpDev M, int n_part, int n_loss, AdamArgs A) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p == 0) {
-        float s = 0.f;
-        for (int b = 0; b < n_loss; ++b) s += M.loss_part[b];
-        *M.loss = s;
-    }
-    if (p >= kMParams) return;
-    float gsum = 0.f;
-    for (int b = 0; b < n_part; ++b) gsum += M.grad_part[(size_t)b * kMParams + p];
-    M.grad[p] = gsum;
-    if (!A.apply) return;
-    const float m = A.beta1 * M.m[p] + (1.f - A.beta1) * gsum;
-    const float v = A.beta2 * M.v[p] + (1.f - A.beta2) * gsum * gsum;
-    M.m[p] = m;
-    M.v[p] = v;
-    const float w = M.master[p] - A.lr * (m * A.c1) / (sqrtf(v * A.c2) + A.eps);
-    M.master[p] = w;
-}
-
-// bf16 / compact copies of the masters.
-__global__ void k_mlp_refresh(MlpDev M) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= kMParams) return;
-    const float w = M.master[p];
+// bf16 / compact copies of one master weight.
+__device__ __forceinline__ void mlp_refresh_one(const MlpDev& M, int p, float w) {
     if (p >= oW2 && p < ob2) {
         const int j = (p - oW2) / kMHid, k = (p - oW2) % kMHid;
         const __nv_bfloat16 b = __float2bfloat16_rn(w);
@@ -134,6 +101,47 @@ __global__ void k_mlp_refresh(MlpDev M) {
     } else {
         M.small[sb3 + (p - ob3)] = w;
     }
+}
+
+// x[0] + x[stride] + ... (n terms) added in this order, eight loads in flight.
+__device__ __forceinline__ float ordered_sum(const float* x, int n, size_t stride) {
+    float s = 0.f;
+    int b = 0;
+    for (; b + 8 <= n; b += 8) {
+        float v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = x[(size_t)(b + i) * stride];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s += v[i];
+    }
+    for (; b < n; ++b) s += x[(size_t)b * stride];
+    return s;
+}
+
+// Sums the partials of n_part blocks in block order, writes the gradient and
+// the batch loss (*loss), applies Adam to the masters and refreshes the rounded
+// copies.
+__global__ void k_mlp_update(MlpDev M, int n_part, int n_loss, float* loss, AdamArgs A) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p == kMParams) *loss = ordered_sum(M.loss_part, n_loss, 1);  // a thread past the parameters
+    if (p >= kMParams) return;
+    const float gsum = ordered_sum(M.grad_part + p, n_part, kMParams);
+    M.grad[p] = gsum;
+    if (!A.apply) return;
+    const float m = A.beta1 * M.m[p] + (1.f - A.beta1) * gsum;
+    const float v = A.beta2 * M.v[p] + (1.f - A.beta2) * gsum * gsum;
+    M.m[p] = m;
+    M.v[p] = v;
+    const float w = M.master[p] - A.lr * (m * A.c1) / (sqrtf(v * A.c2) + A.eps);
+    M.master[p] = w;
+    mlp_refresh_one(M, p, w);
+}
+
+constexpr int kUpdateBlocks = (kMParams + 1 + 127) / 128;  // one thread per parameter and one for the loss
+
+__global__ void k_mlp_refresh(MlpDev M) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < kMParams) mlp_refresh_one(M, p, M.master[p]);
 }
 
 // ------------------------------------------------------------ learned step
@@ -482,18 +490,42 @@ cudaError_t launch_mlp_tc(const MlpDev& D, const LearnedArgs& A, int mode, const
 
 // ------------------------------------------------------------ tensor-core training (tcgen05)
 //
-// The per-sample part of a training step: one sample per thread, 128 per
-// block and tile.  Forward as in k_mlp_tc (MMA 1: z2 = bf16(h1) W2^T + b2),
-// then dout = (out - y)/B, dz2 = (dout W3) gelu'(z2), and MMA 2 (same tensor
-// memory, same A buffer): dh1 = bf16(dz2) W2 against W2^T staged as the B
-// operand, dz1 = dh1 gelu'(z1) with z1 recomputed from x.  Every sample
-// leaves its records (x, bf16(h1), bf16(h2), dout, dz2, dz1) for the
-// weight-gradient kernel, every block its loss partial.
+// One block of 512 threads per tile of 128 samples: warp w works on the
+// samples (tensor-memory lanes) 32 (w mod 4) .. + 31 and the hidden units
+// 16 (w / 4) .. + 15, so a sample's units are spread over four warps.
+//   z1, h1                      -> A operand, and transposed for the gradients
+//   MMA 1: z2 = bf16(h1) W2^T   (then + b2), h2, the output layer: its four
+//                               chains (the order of k_mlp_tc) pass through the
+//                               four warps of a sample in turn
+//   dz2 = (dout W3) gelu'(z2)   -> A operand, and transposed
+//   MMA 2: dh1 = bf16(dz2) W2;  MMA 3: dW2 += bf16(dz2)^T h1 over the tile's
+//                               samples, kept in tensor memory over the block's
+//                               tiles (rows 64..127 of the operand are zero)
+//   dz1 = dh1 gelu'(z1)
+//   dW1, db1, db2, dW3, db3     on the CUDA cores, sums over the tile in registers
+// Nothing per sample goes through global memory.  The step is latency-bound
+// (64 tiles at the usual batch of 8192): with one thread per sample and a
+// second kernel that reloaded every record for the gradients, the two took 32
+// and 20 us and a third and fourth summed and refreshed in 11; now it is 23.5
+// and 4.9 us, without the wait for every loss: 5 steps and a gradient 551 -> 301 us.
+
+constexpr int kTrThreads = 512;
+constexpr int kTrRow = kMHid + 4;    // floats per row: 16-byte rows that start 4 banks apart
+constexpr int kTrRowB = kMHid + 8;   // bf16 per row, the same
+constexpr int kTrParts = kTrThreads / kMHid;
+constexpr int kTrSums = 9;           // dW1 (5), db1, db2, dW3 (2) of one hidden unit
 
 struct TcTrainSmem {
-    alignas(1024) unsigned char A[kTcThreads * kMHid * 2];  // bf16(h1), then bf16(dz2): 128 x 64, K-major
-    alignas(1024) unsigned char Bw[kMHid * kMHid * 2];      // W2: N = j, K = k
-    alignas(1024) unsigned char Bt[kMHid * kMHid * 2];      // W2^T: N = k, K = j
+    alignas(1024) unsigned char A[kTcThreads * kMHid * 2];      // bf16(h1), then bf16(dz2): 128 x 64, K-major
+    alignas(1024) unsigned char At[2][kTcThreads * kMHid * 2];  // bf16(dz2)^T: 64 (of 128) units x 64 samples, both halves
+    alignas(1024) unsigned char Bw[kMHid * kMHid * 2];          // W2: N = j, K = k
+    alignas(1024) unsigned char Bt[kMHid * kMHid * 2];          // W2^T: N = k, K = j
+    alignas(1024) unsigned char Ht[2][kMHid * kMHid * 2];       // bf16(h1)^T: 64 units x 64 samples, both halves
+    float d1[kTcThreads][kTrRow];             // z1, then gelu'(z1), then dz1
+    float d2[kTcThreads][kTrRow];             // z2, then dz2
+    __nv_bfloat16 h2[kTcThreads][kTrRowB];
+    float4 xd[kTcThreads][2];                 // x, dout
+    float4 acc[kTcThreads][kMOut];            // chains of the output layer between warps
     float4 l1[kMHid][2];
     float4 l3[kMHid];
     float b3[kMOut];
@@ -505,10 +537,9 @@ struct TcTrainSmem {
 };
 
 // Thread 0: the four K = 16 MMAs of a K = 64 product into the accumulator at
-// taddr (accumulating onto it when acc), committed to the mbarrier.
+// taddr (accumulating onto it when acc).
 __device__ __forceinline__ void tc_issue_k64(uint32_t taddr, uint32_t a_base, uint32_t b_base, uint32_t idesc,
-                                             bool acc, uint32_t mbar) {
-    tc_fence_after();
+                                             bool acc) {
 #pragma unroll
     for (int ks = 0; ks < kMHid / 16; ++ks) {
         const uint64_t ad = tc_smem_desc(a_base + ks * 2 * kTcLbo, kTcLbo, kTcSbo);
@@ -520,6 +551,8 @@ __device__ __forceinline__ void tc_issue_k64(uint32_t taddr, uint32_t a_base, ui
             "l"(ad), "l"(bd), "r"(idesc), "r"(en)
             : "memory");
     }
+}
+__device__ __forceinline__ void tc_commit(uint32_t mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
 }
 
@@ -532,15 +565,16 @@ __device__ __forceinline__ void tc_stage_b(unsigned char* dst, const __nv_bfloat
     }
 }
 
-// Block-wide: MMA issued by thread 0 after the A writes of every thread,
-// then every thread waits for it; false (and the block's fail flag) when
-// the wait ran out of time.
-__device__ __forceinline__ bool tc_block_mma(uint32_t taddr, uint32_t a_base, uint32_t b_base, uint32_t idesc, bool acc,
-                                             uint32_t mbar, uint32_t& parity, int& fail) {
+// Every thread's operand writes become visible to the tensor core behind the
+// block barrier.
+__device__ __forceinline__ void tc_operands_ready() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0) tc_issue_k64(taddr, a_base, b_base, idesc, acc, mbar);
+}
+// Every thread waits for the committed MMAs; false (and the block's fail flag)
+// when the wait ran out of time.
+__device__ __forceinline__ bool tc_block_wait(uint32_t mbar, uint32_t& parity, int& fail) {
     if (!tc_wait(mbar, parity)) fail = 1;
     parity ^= 1u;
     tc_fence_after();
@@ -548,13 +582,28 @@ __device__ __forceinline__ bool tc_block_mma(uint32_t taddr, uint32_t a_base, ui
     return !fail;
 }
 
-__global__ void __launch_bounds__(kTcThreads) k_mlp_train_tc(MlpDev M, const float* __restrict__ X,
+// Four consecutive units of one row of an operand and of its transpose.
+__device__ __forceinline__ void tc_put4(unsigned char* A, unsigned char* T, int row, int col, const float (&v)[4]) {
+    const unsigned int lo = pack_bf16(v[0], v[1]), hi = pack_bf16(v[2], v[3]);
+    *reinterpret_cast<uint2*>(A + tc_kmajor_offset(row, col)) = make_uint2(lo, hi);
+    const int k = row & (kMHid - 1);
+    *reinterpret_cast<unsigned short*>(T + tc_kmajor_offset(col, k)) = (unsigned short)lo;
+    *reinterpret_cast<unsigned short*>(T + tc_kmajor_offset(col + 1, k)) = (unsigned short)(lo >> 16);
+    *reinterpret_cast<unsigned short*>(T + tc_kmajor_offset(col + 2, k)) = (unsigned short)hi;
+    *reinterpret_cast<unsigned short*>(T + tc_kmajor_offset(col + 3, k)) = (unsigned short)(hi >> 16);
+}
+
+__global__ void __launch_bounds__(kTrThreads) k_mlp_train_tc(MlpDev M, const float* __restrict__ X,
                                                              const float* __restrict__ Y, long long B, long long first,
                                                              long long mul, long long n_data, float invB) {
-    __shared__ TcTrainSmem S;
+    extern __shared__ __align__(1024) unsigned char train_smem[];
+    TcTrainSmem& S = *reinterpret_cast<TcTrainSmem*>(train_smem);
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int cb = warp >> 2, row = (warp & 3) * 32 + lane;  // this thread's units 16 cb .. + 15 of sample `row`
     tc_stage_b(S.Bw, M.W2b);
     tc_stage_b(S.Bt, M.W2Tb);
+    for (int i = t; i < (int)(sizeof(S.At) / 16); i += kTrThreads)
+        reinterpret_cast<uint4*>(S.At)[i] = make_uint4(0, 0, 0, 0);
     if (t < kMHid) {
         const float* w1 = M.small + sW1 + t * kMIn;
         S.l1[t][0] = make_float4(w1[0], w1[1], w1[2], w1[3]);
@@ -570,264 +619,231 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_train_tc(MlpDev M, const flo
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.taddr)),
-                     "r"(kTcCols)
+                     "r"(2 * kTcCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t taddr = S.taddr, trow = taddr + ((uint32_t)(warp * 32) << 16);
+    // columns 0..63: z2, then dh1; columns 64..127: dW2
+    const uint32_t taddr = S.taddr, tgrad = taddr + kTcCols;
+    const uint32_t lane0 = (uint32_t)((warp & 3) * 32) << 16;
     const uint32_t idesc = tc_idesc_bf16_f32(kTcThreads, kMHid);
     const uint32_t a_base = smem_u32(S.A), mbar = smem_u32(&S.mbar);
+    unsigned char* const Atr = S.At[row >> 6];
+    unsigned char* const Htr = S.Ht[row >> 6];
     uint32_t parity = 0;
     float loss = 0.f;
+    float gs[kTrSums], gb3[kMOut] = {0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < kTrSums; ++i) gs[i] = 0.f;
+    bool any = false;
     const long long tiles = (B + kTcThreads - 1) / kTcThreads;
     for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const long long s = tile * kTcThreads + t;
+        const long long s = tile * kTcThreads + row;
         const bool valid = s < B;
         const long long idx = valid ? sample_index(s, first, mul, n_data) : 0;
         float x[kMIn];
 #pragma unroll
         for (int i = 0; i < kMIn; ++i) x[i] = valid ? X[idx * kMIn + i] : 0.f;
-        // layer 1 + GELU: the A operand and the h1 record
+        // layer 1 + GELU
 #pragma unroll 1
-        for (int kb = 0; kb < kMHid / 8; ++kb) {
-            unsigned int packed[4];
+        for (int c = cb * 16; c < cb * 16 + 16; c += 4) {
+            float z[4], h[4];
 #pragma unroll
-            for (int e = 0; e < 8; e += 2) {
-                float h[2];
+            for (int q = 0; q < 4; ++q) {
+                const float4 wa = S.l1[c + q][0], wb = S.l1[c + q][1];
+                z[q] = wb.y;
+                z[q] = fmaf(wa.x, x[0], z[q]);
+                z[q] = fmaf(wa.y, x[1], z[q]);
+                z[q] = fmaf(wa.z, x[2], z[q]);
+                z[q] = fmaf(wa.w, x[3], z[q]);
+                z[q] = fmaf(wb.x, x[4], z[q]);
+                h[q] = gelu_for_bf16(z[q], S.gtab);
+            }
+            *reinterpret_cast<float4*>(&S.d1[row][c]) = make_float4(z[0], z[1], z[2], z[3]);
+            tc_put4(S.A, Htr, row, c, h);
+        }
+        tc_operands_ready();
+        if (t == 0) {
+            tc_fence_after();
+            tc_issue_k64(taddr, a_base, smem_u32(S.Bw), idesc, false);
+            tc_commit(mbar);
+        }
+        if (!tc_block_wait(mbar, parity, S.fail)) break;
+        {
+            float d[16];
+            tc_ld16(taddr + lane0 + (uint32_t)(cb * 16), d);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int col = kb * 8 + e + q;
-                    const float4 wa = S.l1[col][0], wb = S.l1[col][1];
-                    float z = wb.y;
-                    z = fmaf(wa.x, x[0], z);
-                    z = fmaf(wa.y, x[1], z);
-                    z = fmaf(wa.z, x[2], z);
-                    z = fmaf(wa.w, x[3], z);
-                    z = fmaf(wb.x, x[4], z);
-                    h[q] = gelu_for_bf16(z, S.gtab);
+            for (int i = 0; i < 16; i += 4)
+                *reinterpret_cast<float4*>(&S.d2[row][cb * 16 + i]) =
+                    make_float4(d[i] + S.l3[cb * 16 + i].x, d[i + 1] + S.l3[cb * 16 + i + 1].x,
+                                d[i + 2] + S.l3[cb * 16 + i + 2].x, d[i + 3] + S.l3[cb * 16 + i + 3].x);
+        }
+#pragma unroll 1
+        for (int c = cb * 16; c < cb * 16 + 16; c += 4) {
+            const float4 z = *reinterpret_cast<const float4*>(&S.d2[row][c]);
+            *reinterpret_cast<uint2*>(&S.h2[row][c]) =
+                make_uint2(pack_bf16(gelu_for_bf16(z.x, S.gtab), gelu_for_bf16(z.y, S.gtab)),
+                           pack_bf16(gelu_for_bf16(z.z, S.gtab), gelu_for_bf16(z.w, S.gtab)));
+        }
+        // output layer: chain q takes the columns 8 nt + 2 q + e in order, warp by warp
+#pragma unroll 1
+        for (int g = 0; g < 4; ++g) {
+            if (cb == g) {
+                float acc[kMOut][4];
+#pragma unroll
+                for (int o = 0; o < kMOut; ++o) {
+                    const float4 a = g ? S.acc[row][o] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    acc[o][0] = a.x;
+                    acc[o][1] = a.y;
+                    acc[o][2] = a.z;
+                    acc[o][3] = a.w;
                 }
-                packed[e >> 1] = pack_bf16(h[0], h[1]);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const int q = (i & 7) >> 1;
+                    const float4 w = S.l3[g * 16 + i];
+                    const float h = __bfloat162float(S.h2[row][g * 16 + i]);
+                    acc[0][q] = fmaf(w.y, h, acc[0][q]);
+                    acc[1][q] = fmaf(w.z, h, acc[1][q]);
+                }
+                if (g < 3) {
+#pragma unroll
+                    for (int o = 0; o < kMOut; ++o)
+                        S.acc[row][o] = make_float4(acc[o][0], acc[o][1], acc[o][2], acc[o][3]);
+                } else {
+                    float dout[kMOut];
+#pragma unroll
+                    for (int o = 0; o < kMOut; ++o) {
+                        const float out = ((acc[o][0] + acc[o][1]) + (acc[o][2] + acc[o][3])) + S.b3[o];
+                        const float d = valid ? out - Y[idx * kMOut + o] : 0.f;
+                        loss = fmaf(d, d, loss);
+                        dout[o] = d * invB;
+                    }
+                    S.xd[row][0] = make_float4(x[0], x[1], x[2], x[3]);
+                    S.xd[row][1] = make_float4(x[4], dout[0], dout[1], 0.f);
+                }
             }
-            const uint4 v = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-            *reinterpret_cast<uint4*>(S.A + tc_kmajor_offset(t, kb * 8)) = v;
-            if (valid) *reinterpret_cast<uint4*>(M.h1b + s * kMHid + kb * 8) = v;
+            __syncthreads();
         }
-        if (!tc_block_mma(taddr, a_base, smem_u32(S.Bw), idesc, false, mbar, parity, S.fail)) break;
-        // output layer (the order of k_mlp_tc) and the h2 record
-        float acc[kMOut][4];
-#pragma unroll
-        for (int o = 0; o < kMOut; ++o)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[o][q] = 0.f;
+        // dz2 = (dout W3) gelu'(z2)
+        const float4 xd1 = S.xd[row][1];
 #pragma unroll 1
-        for (int cb = 0; cb < kMHid / 16; ++cb) {
-            float d[16], h2[16];
-            tc_ld16(trow + (uint32_t)(cb * 16), d);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        for (int c = cb * 16; c < cb * 16 + 16; c += 4) {
+            float4* zp = reinterpret_cast<float4*>(&S.d2[row][c]);
+            const float4 z4 = *zp;
+            float v[4] = {z4.x, z4.y, z4.z, z4.w};
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int q = (i & 7) >> 1;
-                const float4 w = S.l3[cb * 16 + i];
-                h2[i] = round_bf16(gelu_for_bf16(d[i] + w.x, S.gtab));
-                acc[0][q] = fmaf(w.y, h2[i], acc[0][q]);
-                acc[1][q] = fmaf(w.z, h2[i], acc[1][q]);
+            for (int q = 0; q < 4; ++q) {
+                const float4 w = S.l3[c + q];
+                v[q] = fmaf(w.z, xd1.z, w.y * xd1.y) * gelu_d(v[q]);
             }
-            if (valid) {
-                uint4* dst = reinterpret_cast<uint4*>(M.h2b + s * kMHid + cb * 16);
-                dst[0] = make_uint4(pack_bf16(h2[0], h2[1]), pack_bf16(h2[2], h2[3]), pack_bf16(h2[4], h2[5]),
-                                    pack_bf16(h2[6], h2[7]));
-                dst[1] = make_uint4(pack_bf16(h2[8], h2[9]), pack_bf16(h2[10], h2[11]), pack_bf16(h2[12], h2[13]),
-                                    pack_bf16(h2[14], h2[15]));
-            }
+            *zp = make_float4(v[0], v[1], v[2], v[3]);
+            tc_put4(S.A, Atr, row, c, v);
         }
-        float dout[kMOut];
-#pragma unroll
-        for (int o = 0; o < kMOut; ++o) {
-            const float out = ((acc[o][0] + acc[o][1]) + (acc[o][2] + acc[o][3])) + S.b3[o];
-            const float d = valid ? out - Y[idx * kMOut + o] : 0.f;
-            loss = fmaf(d, d, loss);
-            dout[o] = d * invB;
+        tc_operands_ready();
+        if (t == 0) {
+            tc_fence_after();
+            tc_issue_k64(taddr, a_base, smem_u32(S.Bt), idesc, false);
+            tc_issue_k64(tgrad, smem_u32(S.At[0]), smem_u32(S.Ht[0]), idesc, any);
+            tc_issue_k64(tgrad, smem_u32(S.At[1]), smem_u32(S.Ht[1]), idesc, true);
+            tc_commit(mbar);
         }
-        if (valid) {
-            M.dout[s * kMOut] = dout[0];
-            M.dout[s * kMOut + 1] = dout[1];
-#pragma unroll
-            for (int i = 0; i < kMIn; ++i) M.xs[s * kMIn + i] = x[i];
-        }
-        // dz2 = (dout W3) gelu'(z2): the dz2 record and bf16(dz2) as the next A operand
+        any = true;
+        // gelu'(z1) while the products run
 #pragma unroll 1
-        for (int cb = 0; cb < kMHid / 16; ++cb) {
+        for (int c = cb * 16; c < cb * 16 + 16; c += 4) {
+            float4* zp = reinterpret_cast<float4*>(&S.d1[row][c]);
+            const float4 z = *zp;
+            *zp = make_float4(gelu_d(z.x), gelu_d(z.y), gelu_d(z.z), gelu_d(z.w));
+        }
+        if (!tc_block_wait(mbar, parity, S.fail)) break;
+        {
             float d[16];
-            tc_ld16(trow + (uint32_t)(cb * 16), d);
+            tc_ld16(taddr + lane0 + (uint32_t)(cb * 16), d);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float4 w = S.l3[cb * 16 + i];
-                const float dh = fmaf(w.z, dout[1], w.y * dout[0]);
-                d[i] = dh * gelu_d(d[i] + w.x);
-            }
-            if (valid) {
-                float4* dst = reinterpret_cast<float4*>(M.dz2 + s * kMHid + cb * 16);
-#pragma unroll
-                for (int v = 0; v < 4; ++v) dst[v] = make_float4(d[4 * v], d[4 * v + 1], d[4 * v + 2], d[4 * v + 3]);
-            }
-#pragma unroll
-            for (int hf = 0; hf < 2; ++hf)
-                *reinterpret_cast<uint4*>(S.A + tc_kmajor_offset(t, cb * 16 + hf * 8)) =
-                    make_uint4(pack_bf16(d[8 * hf], d[8 * hf + 1]), pack_bf16(d[8 * hf + 2], d[8 * hf + 3]),
-                               pack_bf16(d[8 * hf + 4], d[8 * hf + 5]), pack_bf16(d[8 * hf + 6], d[8 * hf + 7]));
-        }
-        if (!tc_block_mma(taddr, a_base, smem_u32(S.Bt), idesc, false, mbar, parity, S.fail)) break;
-        // dz1 = dh1 gelu'(z1), z1 recomputed as in layer 1
-#pragma unroll 1
-        for (int cb = 0; cb < kMHid / 16; ++cb) {
-            float d[16];
-            tc_ld16(trow + (uint32_t)(cb * 16), d);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float4 wa = S.l1[cb * 16 + i][0], wb = S.l1[cb * 16 + i][1];
-                float z = wb.y;
-                z = fmaf(wa.x, x[0], z);
-                z = fmaf(wa.y, x[1], z);
-                z = fmaf(wa.z, x[2], z);
-                z = fmaf(wa.w, x[3], z);
-                z = fmaf(wb.x, x[4], z);
-                d[i] = d[i] * gelu_d(z);
-            }
-            if (valid) {
-                float4* dst = reinterpret_cast<float4*>(M.dz1 + s * kMHid + cb * 16);
-#pragma unroll
-                for (int v = 0; v < 4; ++v) dst[v] = make_float4(d[4 * v], d[4 * v + 1], d[4 * v + 2], d[4 * v + 3]);
+            for (int i = 0; i < 16; i += 4) {
+                float4* gp = reinterpret_cast<float4*>(&S.d1[row][cb * 16 + i]);
+                const float4 g = *gp;
+                *gp = make_float4(d[i] * g.x, d[i + 1] * g.y, d[i + 2] * g.z, d[i + 3] * g.w);
             }
         }
+        tc_fence_before();  // this tile's TMEM reads come before the next tile's MMA
+        __syncthreads();
+        // the small gradients: unit j, sixteen samples per thread
+        const int j = t & (kMHid - 1), s0 = (t / kMHid) * (kTcThreads / kTrParts);
+#pragma unroll 4
+        for (int q = s0; q < s0 + kTcThreads / kTrParts; ++q) {
+            const float4 xa = S.xd[q][0], xb = S.xd[q][1];
+            const float d1 = S.d1[q][j], d2 = S.d2[q][j], h = __bfloat162float(S.h2[q][j]);
+            gs[0] = fmaf(d1, xa.x, gs[0]);
+            gs[1] = fmaf(d1, xa.y, gs[1]);
+            gs[2] = fmaf(d1, xa.z, gs[2]);
+            gs[3] = fmaf(d1, xa.w, gs[3]);
+            gs[4] = fmaf(d1, xb.x, gs[4]);
+            gs[5] += d1;
+            gs[6] += d2;
+            gs[7] = fmaf(xb.y, h, gs[7]);
+            gs[8] = fmaf(xb.z, h, gs[8]);
+            gb3[0] += xb.y;
+            gb3[1] += xb.z;
+        }
+        __syncthreads();  // the next tile overwrites the rows
     }
-    // loss partial of this block (fixed reduction order)
+    // partials of this block: the loss (fixed reduction order) ...
+    if (cb == 3) {
 #pragma unroll
-    for (int dd = 16; dd >= 1; dd >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, dd);
-    if (lane == 0) S.loss[warp] = loss;
-    if (t == 0 && S.fail) atomicExch(M.err, 1);
-    tc_fence_before();
+        for (int dd = 16; dd >= 1; dd >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, dd);
+        if (lane == 0) S.loss[warp & 3] = loss;
+    }
+    // ... the small gradients, summed over the parts in order ...
     __syncthreads();
+    constexpr int kSumRow = kTrSums + kMOut;
+    float* sums = &S.d1[0][0];  // [part][unit][kSumRow]
+    static_assert(kTrParts * kMHid * kSumRow <= kTcThreads * kTrRow, "the partial sums fit the rows");
+    {
+        float* mine = sums + (size_t)t * kSumRow;
+#pragma unroll
+        for (int i = 0; i < kTrSums; ++i) mine[i] = gs[i];
+        mine[kTrSums] = gb3[0];
+        mine[kTrSums + 1] = gb3[1];
+    }
+    __syncthreads();
+    float* part = M.grad_part + (size_t)blockIdx.x * kMParams;
+    for (int i = t; i < kMHid * kSumRow; i += kTrThreads) {
+        const int unit = i / kSumRow, q = i % kSumRow;
+        float v = 0.f;
+#pragma unroll
+        for (int p = 0; p < kTrParts; ++p) v += sums[((size_t)p * kMHid + unit) * kSumRow + q];
+        if (q < kMIn) part[oW1 + unit * kMIn + q] = v;
+        else if (q == 5) part[ob1 + unit] = v;
+        else if (q == 6) part[ob2 + unit] = v;
+        else if (q < kTrSums) part[oW3 + (q - 7) * kMHid + unit] = v;
+        else if (unit == 0) part[ob3 + (q - kTrSums)] = v;
+    }
+    // ... and dW2: accumulator lanes 0..63 are the rows j
+    if (row < kMHid) {
+        float d[16];
+        tc_ld16(tgrad + lane0 + (uint32_t)(cb * 16), d);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < 16; ++i) part[oW2 + row * kMHid + cb * 16 + i] = any && !S.fail ? d[i] : 0.f;
+    }
     if (t == 0) {
         float sum = 0.f;
         for (int i = 0; i < kTcThreads / 32; ++i) sum += S.loss[i];
         M.loss_part[blockIdx.x] = 0.5f * sum * invB;
+        if (S.fail) atomicExch(M.err, 1);
     }
-    if (warp == 0) {
-        tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(kTcCols) : "memory");
-    }
-}
-
-// Weight gradients of a batch: block b sums samples [b chunk, (b+1) chunk)
-// into grad_part[b].  dW2[j][k] = sum_s bf16(dz2[s][j]) h1b[s][k] on the
-// tensor cores with the samples as the reduction dimension: per staged tile
-// of 64 samples, A = bf16(dz2)^T (rows 0..63 of a 128-row tile; rows 64..127
-// stay zero and their accumulator lanes are not read), B = h1b^T (N = k),
-// accumulated in tensor memory over the block's tiles.  The small gradients
-// (W1, b1, b2, W3, b3) on the CUDA cores, one column per thread.
-struct TcGradSmem {
-    alignas(1024) unsigned char A[kTcThreads * kWgTile * 2];  // bf16(dz2)^T, K-major (K = samples)
-    alignas(1024) unsigned char Bh[kMHid * kWgTile * 2];      // h1b^T, K-major
-    unsigned long long mbar;
-    unsigned int taddr;
-    int fail;
-};
-
-__global__ void __launch_bounds__(kTcThreads) k_mlp_wgrad_tc(MlpDev M, long long B, long long chunk) {
-    __shared__ TcGradSmem S;
-    const int t = threadIdx.x, warp = t >> 5;
-    for (int i = t; i < (int)(sizeof(S.A) / 16); i += kTcThreads) reinterpret_cast<uint4*>(S.A)[i] = make_uint4(0, 0, 0, 0);
-    if (t == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&S.mbar)) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        S.fail = 0;
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.taddr)),
-                     "r"(kTcCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t taddr = S.taddr, idesc = tc_idesc_bf16_f32(kTcThreads, kMHid);
-    const uint32_t a_base = smem_u32(S.A), b_base = smem_u32(S.Bh), mbar = smem_u32(&S.mbar);
-    const long long s_begin = (long long)blockIdx.x * chunk;
-    const long long s_end = s_begin + chunk < B ? s_begin + chunk : B;
-    uint32_t parity = 0;
-    bool any = false;
-    for (long long s0 = s_begin; s0 < s_end; s0 += kWgTile) {
-        // thread t stages sample s = t / 2, units [32 (t % 2), 32 (t % 2) + 32)
-        const int sl = t >> 1, j0 = (t & 1) * 32;
-        const long long ss = s0 + sl;
-        const bool ok = ss < s_end;
-#pragma unroll 4
-        for (int jj = 0; jj < 32; ++jj) {
-            const int j = j0 + jj;
-            const __nv_bfloat16 a = __float2bfloat16_rn(ok ? M.dz2[ss * kMHid + j] : 0.f);
-            const __nv_bfloat16 b = ok ? M.h1b[ss * kMHid + j] : __float2bfloat16_rn(0.f);
-            *reinterpret_cast<__nv_bfloat16*>(S.A + tc_kmajor_offset(j, sl)) = a;
-            *reinterpret_cast<__nv_bfloat16*>(S.Bh + tc_kmajor_offset(j, sl)) = b;
-        }
-        if (!tc_block_mma(taddr, a_base, b_base, idesc, any, mbar, parity, S.fail)) break;
-        any = true;
-    }
-    float* part = M.grad_part + (size_t)blockIdx.x * kMParams;
-    if (warp < 2) {  // accumulator lanes 0..63: rows j of dW2
-        const int j = t;
-#pragma unroll 1
-        for (int cb = 0; cb < kMHid / 16; ++cb) {
-            float d[16];
-            tc_ld16(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)(cb * 16), d);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-            for (int i = 0; i < 16; ++i) part[oW2 + j * kMHid + cb * 16 + i] = any && !S.fail ? d[i] : 0.f;
-        }
-    }
-    if (t < kMHid) {
-        const int j = t;
-        float gw[kMIn] = {0.f, 0.f, 0.f, 0.f, 0.f}, gb1 = 0.f, gb2 = 0.f;
-        for (long long s = s_begin; s < s_end; ++s) {
-            const float d1 = M.dz1[s * kMHid + j];
-#pragma unroll
-            for (int i = 0; i < kMIn; ++i) gw[i] = fmaf(d1, M.xs[s * kMIn + i], gw[i]);
-            gb1 += d1;
-            gb2 += M.dz2[s * kMHid + j];
-        }
-#pragma unroll
-        for (int i = 0; i < kMIn; ++i) part[oW1 + j * kMIn + i] = gw[i];
-        part[ob1 + j] = gb1;
-        part[ob2 + j] = gb2;
-    } else {
-        const int j = t - kMHid;
-        float g0 = 0.f, g1 = 0.f, d0 = 0.f, d1 = 0.f;
-        for (long long s = s_begin; s < s_end; ++s) {
-            const float h = __bfloat162float(M.h2b[s * kMHid + j]);
-            const float o0 = M.dout[s * kMOut], o1 = M.dout[s * kMOut + 1];
-            g0 = fmaf(o0, h, g0);
-            g1 = fmaf(o1, h, g1);
-            d0 += o0;
-            d1 += o1;
-        }
-        part[oW3 + j] = g0;
-        part[oW3 + kMHid + j] = g1;
-        if (j == 0) {
-            part[ob3] = d0;
-            part[ob3 + 1] = d1;
-        }
-    }
-    if (t == 0 && S.fail) atomicExch(M.err, 1);
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(kTcCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(2 * kTcCols) : "memory");
     }
 }
 
@@ -912,8 +928,6 @@ struct pic_mlp {
     int sm_count = 0;
     long long t = 0;  // Adam steps taken
     std::vector<void*> allocs;
-    float* loss_host = nullptr;  // pinned
-    int train_per_sm = 1;        // resident blocks of k_mlp_train_tc per SM
 };
 
 namespace {
@@ -936,24 +950,17 @@ cudaError_t mlp_alloc(pic_mlp* m, T** p, size_t count) {
 void mlp_free(pic_mlp* m) {
     for (void* p : m->allocs) cudaFree(p);
     m->allocs.clear();
-    if (m->loss_host) cudaFreeHost(m->loss_host);
-    m->loss_host = nullptr;
 }
 
-// Forward + backward + weight gradients + reduction (+ Adam when apply).
+// Forward, backward and gradients, then their sum (+ Adam when apply); the
+// batch loss goes to *loss (device).
 cudaError_t mlp_step(pic_mlp* m, long long B, const float* X, const float* Y, long long first, long long mul,
-                     long long n_data, int apply, const pic_adam_t* opt) {
+                     long long n_data, float* loss, int apply, const pic_adam_t* opt) {
     pic::MlpDev& D = m->D;
     const long long tiles = (B + pic::kTcThreads - 1) / pic::kTcThreads;
-    const long long cap = (long long)m->sm_count * m->train_per_sm;
-    const int gf = (int)(tiles < cap ? tiles : cap);
-    pic::k_mlp_train_tc<<<gf, pic::kTcThreads, 0, m->st>>>(D, X, Y, B, first, mul, n_data, 1.0f / (float)B);
-    long long nwg = (B + pic::kWgTile - 1) / pic::kWgTile;
-    if (nwg > pic::kWgMaxBlocks) nwg = pic::kWgMaxBlocks;
-    long long chunk = (B + nwg - 1) / nwg;
-    chunk = (chunk + pic::kWgTile - 1) / pic::kWgTile * pic::kWgTile;
-    nwg = (B + chunk - 1) / chunk;
-    pic::k_mlp_wgrad_tc<<<(int)nwg, pic::kTcThreads, 0, m->st>>>(D, B, chunk);
+    const int grid = (int)(tiles < m->sm_count ? tiles : m->sm_count);  // one block per SM (its shared memory)
+    pic::k_mlp_train_tc<<<grid, pic::kTrThreads, sizeof(pic::TcTrainSmem), m->st>>>(D, X, Y, B, first, mul, n_data,
+                                                                                   1.0f / (float)B);
     pic::AdamArgs A;
     std::memset(&A, 0, sizeof(A));
     if (apply) {
@@ -966,9 +973,7 @@ cudaError_t mlp_step(pic_mlp* m, long long B, const float* X, const float* Y, lo
         A.c2 = (float)(1.0 / (1.0 - std::pow((double)opt->beta2, (double)m->t)));
         A.apply = 1;
     }
-    const int gp = (pic::kMParams + 255) / 256;
-    pic::k_mlp_update<<<gp, 256, 0, m->st>>>(D, (int)nwg, gf, A);
-    if (apply) pic::k_mlp_refresh<<<gp, 256, 0, m->st>>>(D);
+    pic::k_mlp_update<<<pic::kUpdateBlocks, 128, 0, m->st>>>(D, grid, grid, loss, A);
     return cudaGetLastError();
 }
 
@@ -1024,7 +1029,6 @@ int pic_mlp_create(int64_t max_batch, void* stream, pic_mlp** out) {
     m->sm_count = sms;
     pic::MlpDev& D = m->D;
     std::memset(&D, 0, sizeof(D));
-    const size_t B = (size_t)max_batch;
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = mlp_alloc(m, &D.master, pic::kMParams);
     if (e == cudaSuccess) e = mlp_alloc(m, &D.m, pic::kMParams);
@@ -1032,19 +1036,12 @@ int pic_mlp_create(int64_t max_batch, void* stream, pic_mlp** out) {
     if (e == cudaSuccess) e = mlp_alloc(m, &D.W2b, pic::kMHid * pic::kMHid);
     if (e == cudaSuccess) e = mlp_alloc(m, &D.W2Tb, pic::kMHid * pic::kMHid);
     if (e == cudaSuccess) e = mlp_alloc(m, &D.small, pic::kMSmall);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.xs, B * pic::kMIn);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.dz1, B * pic::kMHid);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.dz2, B * pic::kMHid);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.h1b, B * pic::kMHid);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.h2b, B * pic::kMHid);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.dout, B * pic::kMOut);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.loss_part, (size_t)sms * 8);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.grad_part, (size_t)pic::kWgMaxBlocks * pic::kMParams);
+    if (e == cudaSuccess) e = mlp_alloc(m, &D.loss_part, (size_t)sms);
+    if (e == cudaSuccess) e = mlp_alloc(m, &D.grad_part, (size_t)sms * pic::kMParams);
     if (e == cudaSuccess) e = mlp_alloc(m, &D.grad, pic::kMParams);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.loss, 1);
+    if (e == cudaSuccess) e = mlp_alloc(m, &D.loss, pic::kLossHist);
     if (e == cudaSuccess) e = mlp_alloc(m, &D.err, 1);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.err, 0, sizeof(int), m->st);
-    if (e == cudaSuccess) e = cudaMallocHost(&m->loss_host, sizeof(float));
     if (e == cudaSuccess) e = cudaMemsetAsync(D.master, 0, sizeof(float) * pic::kMParams, m->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.m, 0, sizeof(float) * pic::kMParams, m->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.v, 0, sizeof(float) * pic::kMParams, m->st);
@@ -1052,11 +1049,9 @@ int pic_mlp_create(int64_t max_batch, void* stream, pic_mlp** out) {
         pic::k_mlp_refresh<<<(pic::kMParams + 255) / 256, 256, 0, m->st>>>(D);
         e = cudaGetLastError();
     }
-    for (const void* fn : {(const void*)pic::k_mlp_train_tc, (const void*)pic::k_mlp_wgrad_tc})
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess) m->train_per_sm = pic::tc_blocks_per_sm((const void*)pic::k_mlp_train_tc, 0);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(pic::k_mlp_train_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(pic::TcTrainSmem));
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->st);
     if (e != cudaSuccess) {
         mlp_free(m);
@@ -1105,7 +1100,7 @@ int pic_mlp_gradients(pic_mlp* m, int64_t n, const float* X_dev, const float* T_
     if (!m || n < 1 || n > m->max_batch || !X_dev || !T_dev || !grad || !loss) return PIC_ERR_INVALID_ARG;
     if (ptr_kind != PIC_PTR_HOST && ptr_kind != PIC_PTR_DEVICE) return PIC_ERR_INVALID_ARG;
     const cudaMemcpyKind k = ptr_kind == PIC_PTR_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-    cudaError_t e = mlp_step(m, n, X_dev, T_dev, 0, 1, n, 0, nullptr);
+    cudaError_t e = mlp_step(m, n, X_dev, T_dev, 0, 1, n, m->D.loss, 0, nullptr);
     if (e == cudaSuccess) e = cudaMemcpyAsync(grad, m->D.grad, sizeof(float) * pic::kMParams, k, m->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(loss, m->D.loss, sizeof(float), k, m->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->st);
@@ -1130,11 +1125,13 @@ int pic_mlp_train(pic_mlp* m, int64_t n_data, const float* X_dev, const float* T
     cudaError_t e = cudaSuccess;
     for (long long s = 0; s < steps && e == cudaSuccess; ++s) {
         const long long first = (s * batch) % n_data;
-        e = mlp_step(m, batch, X_dev, T_dev, first, mul, n_data, 1, opt);
-        if (e == cudaSuccess && loss_hist) {
-            e = cudaMemcpyAsync(m->loss_host, m->D.loss, sizeof(float), cudaMemcpyDeviceToHost, m->st);
+        // the losses stay on the device until kLossHist of them, or the last, are in
+        const long long at = s % pic::kLossHist;
+        e = mlp_step(m, batch, X_dev, T_dev, first, mul, n_data, m->D.loss + at, 1, opt);
+        if (e == cudaSuccess && loss_hist && (at == pic::kLossHist - 1 || s == steps - 1)) {
+            e = cudaMemcpyAsync(loss_hist + (s - at), m->D.loss, sizeof(float) * (size_t)(at + 1),
+                                cudaMemcpyDeviceToHost, m->st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(m->st);
-            if (e == cudaSuccess) loss_hist[s] = *m->loss_host;
         }
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->st);
@@ -1161,9 +1158,7 @@ int pic_mlp_apply_gradient(pic_mlp* m, const float* grad, int ptr_kind, const pi
         A.c1 = (float)(1.0 / (1.0 - std::pow((double)opt->beta1, (double)m->t)));
         A.c2 = (float)(1.0 / (1.0 - std::pow((double)opt->beta2, (double)m->t)));
         A.apply = 1;
-        const int gp = (pic::kMParams + 255) / 256;
-        pic::k_mlp_update<<<gp, 256, 0, m->st>>>(m->D, 1, 0, A);
-        pic::k_mlp_refresh<<<gp, 256, 0, m->st>>>(m->D);
+        pic::k_mlp_update<<<pic::kUpdateBlocks, 128, 0, m->st>>>(m->D, 1, 0, m->D.loss, A);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->st);
