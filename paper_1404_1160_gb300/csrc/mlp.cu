@@ -57,7 +57,7 @@ struct MlpDev {
     float* grad_part;     // [training blocks][kMParams]
     float* grad;          // [kMParams]
     float* loss;          // [kLossHist]
-    int* err;             // set by a tensor-core wait that ran out of time
+    int* err;             // set by a tensor-core wait that ran out of time (pinned host memory, mapped)
 };
 
 // ------------------------------------------------------------ device math
@@ -181,18 +181,24 @@ static __device__ __noinline__ bool frozen_keep_fp64(const LearnedArgs& A, doubl
 //
 // Inference of the network (pic_mlp_forward) and the learned step's
 // correction with the 64 x 64 hidden layer on the 5th-generation tensor
-// cores: a block of 128 threads owns 128 samples (one per thread), writes
-// bf16(gelu(z1)) as the A operand (128 x 64, K-major core matrices) to shared
-// memory, and one thread issues four tcgen05.mma (M = 128, N = 64, K = 16
-// each) against W2 (B operand, 64 x 64) into a 64-column f32 accumulator in
-// tensor memory and commits them to an mbarrier; each warp then reads its 32
-// rows back with tcgen05.ld.  The output layer adds the products of each
-// sample's 64 columns in four fused multiply-add chains of 16 (columns
-// 8 nt + 2 q + e for chain q) combined as (s0 + s1) + (s2 + s3).  Where a
+// cores: a block of 256 threads owns 128 samples, two threads each (warps 0..3
+// the hidden units 0..31, warps 4..7 the others), writes bf16(gelu(z1)) as the
+// A operand (128 x 64, K-major core matrices) to shared memory, and one thread
+// issues four tcgen05.mma (M = 128, N = 64, K = 16 each) against W2 (B operand,
+// 64 x 64) into a 64-column f32 accumulator in tensor memory and commits them
+// to an mbarrier; each warp then reads half of its 32 rows back with
+// tcgen05.ld.  The output layer adds the products of each sample's 64 columns
+// in four fused multiply-add chains of 16 (columns 8 nt + 2 q + e for chain q)
+// combined as (s0 + s1) + (s2 + s3); the first thread hands its chains to the
+// second.  (Up to a few tiles per SM a call is one tile's latency: with one
+// thread per sample, occupancy queries and a copy of the error flag on every
+// call, 10^5 samples took 58 us and 100 samples 45, now 46 and 32; from 10^6 on,
+// where issue binds, both take 0.17 us per 1000.)  Where a
 // GELU is rounded to bfloat16 at once it is evaluated by gelu_for_bf16
 // (gelu_fast.cuh), which rounds exactly as the erfc form does.
 
-constexpr int kTcThreads = 128;  // one sample per thread, one 128-row MMA tile per block
+constexpr int kTcThreads = 128;  // samples of a tile (rows of the MMA)
+constexpr int kInfThreads = 256; // two threads per sample
 constexpr int kTcCols = 64;      // TMEM columns of the accumulator (N = 64, f32)
 
 struct TcSmem {
@@ -202,6 +208,7 @@ struct TcSmem {
     float4 l3[kMHid];     // per hidden unit: (b2[j], W3[0][j], W3[1][j], 0)
     float b3[kMOut];
     float4 gtab[kGeluSeg + 1];  // segment table of gelu_for_bf16
+    float4 acc[kMOut][kTcThreads];  // chains of the output layer, from a sample's first thread to its second
     unsigned long long mbar;
     unsigned int taddr;
     int fail;
@@ -245,13 +252,14 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t parity) {
 // correction of an FP64 / FP32 state, kept where the frozen-field energy
 // check allows it.
 template <int MODE>
-__global__ void __launch_bounds__(kTcThreads) k_mlp_tc(MlpDev M, LearnedArgs A, const float* __restrict__ X,
-                                                       float* __restrict__ Y, long long n) {
+__global__ void __launch_bounds__(kInfThreads, 6) k_mlp_tc(MlpDev M, LearnedArgs A, const float* __restrict__ X,
+                                                        float* __restrict__ Y, long long n) {
     __shared__ TcSmem S;
     extern __shared__ float s_tab[];  // binary32 field tables of the energy check (MODE 2, Poisson)
     const int t = threadIdx.x, warp = t >> 5;
+    const int half = warp >> 2, row = t & (kTcThreads - 1);  // this thread's units 32 half .. + 31 of sample `row`
     // W2 as the B operand; the CUDA-core layers' weights packed per hidden unit
-    for (int i = t; i < kMHid * kMHid / 8; i += kTcThreads) {
+    for (int i = t; i < kMHid * kMHid / 8; i += kInfThreads) {
         const int nrow = i >> 3, kb = i & 7;  // 8 consecutive k of output row nrow
         *reinterpret_cast<uint4*>(S.Bw + tc_kmajor_offset(nrow, kb * 8)) =
             *reinterpret_cast<const uint4*>(M.W2b + nrow * kMHid + kb * 8);
@@ -265,7 +273,7 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_tc(MlpDev M, LearnedArgs A, 
     if (t < kMOut) S.b3[t] = M.small[sb3 + t];
     if (t <= kGeluSeg) S.gtab[t] = make_float4(c_gelu_tab[t][0], c_gelu_tab[t][1], c_gelu_tab[t][2], c_gelu_tab[t][3]);
     if (MODE == 2 && A.tab_f)
-        for (int i = t; i < 3 * (A.n_cells + 1); i += kTcThreads) s_tab[i] = A.tab_f[i];
+        for (int i = t; i < 3 * (A.n_cells + 1); i += kInfThreads) s_tab[i] = A.tab_f[i];
     if (t == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&S.mbar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -302,7 +310,7 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_tc(MlpDev M, LearnedArgs A, 
     uint32_t parity = 0;
     const long long tiles = (n + kTcThreads - 1) / kTcThreads;
     for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const long long s = tile * kTcThreads + t;
+        const long long s = tile * kTcThreads + row;
         const bool valid = s < n;
         float x[kMIn];
         if (MODE == 0) {
@@ -322,11 +330,11 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_tc(MlpDev M, LearnedArgs A, 
             x[3] = A.in_cos;
             x[4] = A.in_dt;
         }
-        // layer 1 + GELU into the A operand: row t, 8 columns (one 16-byte
-        // core-matrix row) per pass; the pass loop stays rolled, since 64
-        // inlined erfc evaluations per layer overflow the instruction cache
+        // layer 1 + GELU into the A operand: row `row`, 8 columns (one 16-byte
+        // core-matrix row) per pass; the pass loop stays rolled for the
+        // instruction cache
 #pragma unroll 1
-        for (int kb = 0; kb < kMHid / 8; ++kb) {
+        for (int kb = half * 4; kb < half * 4 + 4; ++kb) {
             unsigned int packed[4];
 #pragma unroll
             for (int e = 0; e < 8; e += 2) {
@@ -345,7 +353,7 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_tc(MlpDev M, LearnedArgs A, 
                 }
                 packed[e >> 1] = pack_bf16(h[0], h[1]);
             }
-            *reinterpret_cast<uint4*>(S.A + tc_kmajor_offset(t, kb * 8)) =
+            *reinterpret_cast<uint4*>(S.A + tc_kmajor_offset(row, kb * 8)) =
                 make_uint4(packed[0], packed[1], packed[2], packed[3]);
         }
         // the generic-proxy writes of A become visible to the tensor core
@@ -372,27 +380,47 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_tc(MlpDev M, LearnedArgs A, 
         tc_fence_after();
         __syncthreads();
         if (S.fail) break;
-        // z2 = D + b2 of this thread's row, GELU, bf16, output layer
-        float acc[kMOut][4];
+        // z2 = D + b2 of this thread's half row, GELU, bf16 (two per register)
+        unsigned int h2[16];
 #pragma unroll
-        for (int o = 0; o < kMOut; ++o)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[o][q] = 0.f;
-#pragma unroll 1
-        for (int cb = 0; cb < kMHid / 16; ++cb) {
+        for (int c = 0; c < 2; ++c) {
             float d[16];
-            tc_ld16(taddr + ((uint32_t)(warp * 32) << 16) + (uint32_t)(cb * 16), d);
+            tc_ld16(taddr + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(half * 32 + c * 16), d);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int q = (i & 7) >> 1;
-                const float4 w = S.l3[cb * 16 + i];
-                const float h2 = round_bf16(gelu_for_bf16(d[i] + w.x, S.gtab));
-                acc[0][q] = fmaf(w.y, h2, acc[0][q]);
-                acc[1][q] = fmaf(w.z, h2, acc[1][q]);
+            for (int i = 0; i < 16; i += 2) {
+                const int col = half * 32 + c * 16 + i;
+                h2[c * 8 + (i >> 1)] = pack_bf16(gelu_for_bf16(d[i] + S.l3[col].x, S.gtab),
+                                                 gelu_for_bf16(d[i + 1] + S.l3[col + 1].x, S.gtab));
             }
         }
         tc_fence_before();  // this tile's TMEM reads come before the next tile's MMA
+        // output layer: the chains of columns 0..31, then of 32..63
+        float acc[kMOut][4];
+        if (half == 1) asm volatile("bar.sync 1, %0;" ::"n"(kInfThreads) : "memory");
+#pragma unroll
+        for (int o = 0; o < kMOut; ++o) {
+            const float4 a = half ? S.acc[o][row] : make_float4(0.f, 0.f, 0.f, 0.f);
+            acc[o][0] = a.x;
+            acc[o][1] = a.y;
+            acc[o][2] = a.z;
+            acc[o][3] = a.w;
+        }
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            const int q = (i & 7) >> 1;
+            const float4 w = S.l3[half * 32 + i];
+            const float h = __uint_as_float((i & 1) ? (h2[i >> 1] & 0xffff0000u) : (h2[i >> 1] << 16));
+            acc[0][q] = fmaf(w.y, h, acc[0][q]);
+            acc[1][q] = fmaf(w.z, h, acc[1][q]);
+        }
+        if (half == 0) {
+#pragma unroll
+            for (int o = 0; o < kMOut; ++o) S.acc[o][row] = make_float4(acc[o][0], acc[o][1], acc[o][2], acc[o][3]);
+            // the second threads read the chains before the next tile's block barriers
+            asm volatile("bar.arrive 1, %0;" ::"n"(kInfThreads) : "memory");
+            continue;
+        }
         float out[kMOut];
 #pragma unroll
         for (int o = 0; o < kMOut; ++o) out[o] = ((acc[o][0] + acc[o][1]) + (acc[o][2] + acc[o][3])) + S.b3[o];
@@ -437,7 +465,7 @@ __global__ void __launch_bounds__(kTcThreads) k_mlp_tc(MlpDev M, LearnedArgs A, 
         for (int d = 16; d >= 1; d >>= 1) fallback += __shfl_xor_sync(0xffffffffu, fallback, d);
         if ((t & 31) == 0 && fallback) atomicAdd(A.n_fallback, (unsigned long long)fallback);
     }
-    if (t == 0 && S.fail) atomicExch(M.err, 1);
+    if (t == 0 && S.fail) *(volatile int*)M.err = 1;
     tc_fence_before();
     __syncthreads();
     if (warp == 0) {
@@ -458,33 +486,39 @@ static int tc_blocks_per_sm(const void* fn, size_t dyn_smem) {
         cudaDeviceGetAttribute(&resv, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess)
         return 1;
-    const int regs_block = ((fa.numRegs + 7) / 8) * 8 * kTcThreads;  // allocated per warp in units of 8 per thread
+    const int regs_block = ((fa.numRegs + 7) / 8) * 8 * kInfThreads;  // allocated per warp in units of 8 per thread
     int k = 512 / kTcCols;
-    k = std::min(k, 2048 / kTcThreads);
+    k = std::min(k, 2048 / kInfThreads);
     if (regs_block > 0) k = std::min(k, regs_sm / regs_block);
     k = std::min(k, (int)((size_t)smem_sm / (fa.sharedSizeBytes + dyn_smem + (size_t)resv)));
     return k < 1 ? 1 : k;
 }
 
-// Launch of the tensor-core inference over n samples: as many blocks as are
-// resident at once, no more blocks than tiles.
-cudaError_t launch_mlp_tc(const MlpDev& D, const LearnedArgs& A, int mode, const float* X, float* Y, long long n,
-                          int sm_count, cudaStream_t st) {
-    if (n == 0) return cudaSuccess;
-    const size_t smem = (mode == 2 && A.tab_f) ? sizeof(float) * 3 * (size_t)(A.n_cells + 1) : 0;
-    void* fn = mode == 0 ? (void*)k_mlp_tc<0> : mode == 1 ? (void*)k_mlp_tc<1> : (void*)k_mlp_tc<2>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+static void* tc_fn(int mode) {
+    return mode == 0 ? (void*)k_mlp_tc<0> : mode == 1 ? (void*)k_mlp_tc<1> : (void*)k_mlp_tc<2>;
+}
+// Sets up the inference kernel of a mode for its dynamic shared memory and
+// returns the blocks resident per SM.
+static cudaError_t tc_setup(int mode, size_t smem, int* per_sm) {
+    cudaError_t e = cudaFuncSetAttribute(tc_fn(mode), cudaFuncAttributePreferredSharedMemoryCarveout,
                                          (int)cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess && smem > 48 * 1024)
-        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int per_sm = tc_blocks_per_sm(fn, smem);
+        e = cudaFuncSetAttribute(tc_fn(mode), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) *per_sm = tc_blocks_per_sm(tc_fn(mode), smem);
+    return e;
+}
+
+// Launch of the tensor-core inference over n samples: as many blocks as are
+// resident at once (per_sm each, as tc_setup gave), no more blocks than tiles.
+static cudaError_t launch_mlp_tc(const MlpDev& D, const LearnedArgs& A, int mode, const float* X, float* Y, long long n,
+                                 size_t smem, int per_sm, int sm_count, cudaStream_t st) {
+    if (n == 0) return cudaSuccess;
     const long long tiles = (n + kTcThreads - 1) / kTcThreads;
     const long long cap = (long long)sm_count * per_sm;
     const int grid = (int)(tiles < cap ? tiles : cap);
-    if (mode == 0) k_mlp_tc<0><<<grid, kTcThreads, smem, st>>>(D, A, X, Y, n);
-    else if (mode == 1) k_mlp_tc<1><<<grid, kTcThreads, smem, st>>>(D, A, X, Y, n);
-    else k_mlp_tc<2><<<grid, kTcThreads, smem, st>>>(D, A, X, Y, n);
+    if (mode == 0) k_mlp_tc<0><<<grid, kInfThreads, smem, st>>>(D, A, X, Y, n);
+    else if (mode == 1) k_mlp_tc<1><<<grid, kInfThreads, smem, st>>>(D, A, X, Y, n);
+    else k_mlp_tc<2><<<grid, kInfThreads, smem, st>>>(D, A, X, Y, n);
     return cudaGetLastError();
 }
 
@@ -837,7 +871,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train_tc(MlpDev M, const flo
         float sum = 0.f;
         for (int i = 0; i < kTcThreads / 32; ++i) sum += S.loss[i];
         M.loss_part[blockIdx.x] = 0.5f * sum * invB;
-        if (S.fail) atomicExch(M.err, 1);
+        if (S.fail) *(volatile int*)M.err = 1;
     }
     tc_fence_before();
     __syncthreads();
@@ -927,6 +961,8 @@ struct pic_mlp {
     cudaStream_t st = nullptr;
     int sm_count = 0;
     long long t = 0;  // Adam steps taken
+    int forward_per_sm = 1;  // resident blocks of the inference kernel (pic_mlp_forward) per SM
+    int* err_host = nullptr;  // D.err as the host sees it
     std::vector<void*> allocs;
 };
 
@@ -950,6 +986,8 @@ cudaError_t mlp_alloc(pic_mlp* m, T** p, size_t count) {
 void mlp_free(pic_mlp* m) {
     for (void* p : m->allocs) cudaFree(p);
     m->allocs.clear();
+    if (m->err_host) cudaFreeHost(m->err_host);
+    m->err_host = nullptr;
 }
 
 // Forward, backward and gradients, then their sum (+ Adam when apply); the
@@ -992,7 +1030,11 @@ namespace pic {
 cudaError_t launch_learned_apply(const pic_mlp* m, const LearnedArgs& A, int sm_count, cudaStream_t st,
                                  long long* launches) {
     if (A.n == 0) return cudaSuccess;
-    const cudaError_t e = launch_mlp_tc(m->D, A, A.prec == 0 ? 1 : 2, nullptr, nullptr, A.n, sm_count, st);
+    const int mode = A.prec == 0 ? 1 : 2;
+    const size_t smem = (mode == 2 && A.tab_f) ? sizeof(float) * 3 * (size_t)(A.n_cells + 1) : 0;
+    int per_sm = 1;
+    cudaError_t e = tc_setup(mode, smem, &per_sm);
+    if (e == cudaSuccess) e = launch_mlp_tc(m->D, A, mode, nullptr, nullptr, A.n, smem, per_sm, sm_count, st);
     if (launches) ++*launches;
     return e;
 }
@@ -1000,14 +1042,12 @@ cudaError_t launch_learned_apply(const pic_mlp* m, const LearnedArgs& A, int sm_
 // PIC_ERR_TIMEOUT (and the flag cleared) when a tensor-core wait of the
 // inference kernel ran out of time since the last call; synchronises st.
 int mlp_take_error(const pic_mlp* m, cudaStream_t st) {
-    int err = 0;
-    cudaError_t e = cudaMemcpyAsync(&err, m->D.err, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    const cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? PIC_ERR_NO_MEMORY : PIC_ERR_CUDA;
-    if (!err) return PIC_OK;
-    e = cudaMemsetAsync(m->D.err, 0, sizeof(int), st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    return e == cudaSuccess ? PIC_ERR_TIMEOUT : PIC_ERR_CUDA;
+    volatile int* err = m->err_host;
+    if (!*err) return PIC_OK;
+    *err = 0;
+    return PIC_ERR_TIMEOUT;
 }
 }  // namespace pic
 
@@ -1040,8 +1080,10 @@ int pic_mlp_create(int64_t max_batch, void* stream, pic_mlp** out) {
     if (e == cudaSuccess) e = mlp_alloc(m, &D.grad_part, (size_t)sms * pic::kMParams);
     if (e == cudaSuccess) e = mlp_alloc(m, &D.grad, pic::kMParams);
     if (e == cudaSuccess) e = mlp_alloc(m, &D.loss, pic::kLossHist);
-    if (e == cudaSuccess) e = mlp_alloc(m, &D.err, 1);
-    if (e == cudaSuccess) e = cudaMemsetAsync(D.err, 0, sizeof(int), m->st);
+    if (e == cudaSuccess) e = cudaHostAlloc((void**)&m->err_host, sizeof(int), cudaHostAllocMapped);
+    if (e == cudaSuccess) *m->err_host = 0;
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&D.err, m->err_host, 0);
+    if (e == cudaSuccess) e = pic::tc_setup(0, 0, &m->forward_per_sm);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.master, 0, sizeof(float) * pic::kMParams, m->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.m, 0, sizeof(float) * pic::kMParams, m->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(D.v, 0, sizeof(float) * pic::kMParams, m->st);
@@ -1090,7 +1132,7 @@ int pic_mlp_forward(pic_mlp* m, int64_t n, const float* X_dev, float* Y_dev) {
     if (n == 0) return PIC_OK;
     pic::LearnedArgs A;
     std::memset(&A, 0, sizeof(A));
-    const cudaError_t e = pic::launch_mlp_tc(m->D, A, 0, X_dev, Y_dev, n, m->sm_count, m->st);
+    const cudaError_t e = pic::launch_mlp_tc(m->D, A, 0, X_dev, Y_dev, n, 0, m->forward_per_sm, m->sm_count, m->st);
     if (e != cudaSuccess) return mlp_map(e);
     return pic::mlp_take_error(m, m->st);
 }
