@@ -593,7 +593,11 @@ int pic_init(const pic_params* p, int64_t n, const double* r0, const double* v0,
     h->st = (cudaStream_t)stream;
     h->sm_count = sms;
     make_devparams(p, n, &h->dp);
-    h->block = p->block_size ? p->block_size : (p->field_model == PIC_FIELD_POISSON ? 1024 : 128);
+    // per-particle windows of up to 16 warps per SM run in blocks of one warp:
+    // they spread evenly, and the FP64 pipe is shared by an SM's warps (10^4
+    // particles, 313 warps: 3 instead of 4 on the fullest SM)
+    h->block = p->block_size ? p->block_size
+                             : (p->field_model == PIC_FIELD_POISSON ? 1024 : (n <= 16ll * 32 * sms ? 32 : 128));
 
     if (p->precision == 1) {
         rc = init32(h, r0, v0, ptr_kind);

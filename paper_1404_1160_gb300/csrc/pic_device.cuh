@@ -267,7 +267,9 @@ __device__ __forceinline__ double quad_root01(double v0, double v1, double v2) {
 constexpr int F_NEXT = 3, F_RES = 4, F_FB = 8, F_PEND = 16;
 
 struct Track {
-    double t1, T, o;
+    double T, o;
+    double v0, v1, v2;  // V around the first extremum, until the third one fixes the period
+    int k1;             // sample before the first extremum
     int N, need, flags;
 };
 
@@ -296,19 +298,33 @@ __device__ __forceinline__ void track_resolve(Track& s, const DevParams& P, doub
     s.flags |= F_RES;
 }
 
+// T = time between the extrema of two stencils (samples k1.. and k3..).  Out of
+// line: the lanes of a warp reach it at different samples.
+static __device__ __noinline__ double track_period(double a0, double a1, double a2, int k1, double b0, double b1,
+                                                   double b2, int k3) {
+    const double t1 = (double)k1 + quad_root01(a0, a1, a2);
+    return ((double)k3 + quad_root01(b0, b1, b2)) - t1;
+}
+
 // Sample k (k >= 2) has just been produced: V_{k-2} = v0, V_{k-1} = v1,
 // V_k = v2.  A sign change between k-2 and k-1 (V > 0 counts as +) is an
-// extremum of R (Remark CompOfThePeriodsRem).  detect_only: step 1 alone.
+// extremum of R (Remark CompOfThePeriodsRem).  The first one keeps its
+// stencil, and only the third evaluates roots (10^5 unsorted particles, periods
+// every step: 2 steps 3.83 -> 2.43 ms).  detect_only: step 1 alone.
 __device__ __forceinline__ void track_sample(Track& s, const DevParams& P, int k, double v0,
                                              double v1, double v2, bool detect_only) {
     if (s.flags & F_RES) return;
     if (positive(v0) != positive(v1)) {
-        double t = (double)(k - 2) + quad_root01(v0, v1, v2);
-        int ne = (s.flags & F_NEXT) + 1;
+        const int ne = (s.flags & F_NEXT) + 1;
         s.flags = (s.flags & ~F_NEXT) | (ne & F_NEXT);
-        if (ne == 1) s.t1 = t;
+        if (ne == 1) {
+            s.v0 = v0;
+            s.v1 = v1;
+            s.v2 = v2;
+            s.k1 = k - 2;
+        }
         if (ne == 3) {
-            double T = t - s.t1;
+            const double T = track_period(s.v0, s.v1, s.v2, s.k1, v0, v1, v2, k - 2);
             if (detect_only) {
                 s.T = T;
                 s.flags |= F_RES;
@@ -365,8 +381,7 @@ __device__ __forceinline__ void rk4_step_analytic(const DevParams& P, int field,
 }
 
 // Lawson RK4: exact rotation Phi(s) for (1/eps) M y, RK4 on the field term.
-__device__ __forceinline__ void lawson_step_analytic(const DevParams& P, int field, double& R,
-                                                     double& V) {
+__device__ __forceinline__ void lawson_step_analytic_fp64(const DevParams& P, int field, double& R, double& V) {
     double e1 = field_analytic(field, R);
     double R2 = fma(P.sh, fma(P.h2, e1, V), P.ch * R);
     double e2 = field_analytic(field, R2);
@@ -379,6 +394,42 @@ __device__ __forceinline__ void lawson_step_analytic(const DevParams& P, int fie
     double e23 = e2 + e3;
     R = fma(P.h6, fma(P.tsh, e23, P.s1 * e1), A);
     V = fma(P.h6, fma(P.tch, e23, fma(P.c1, e1, e4)), B);
+}
+
+// The same step with the eight products that do not lie on its longest chain
+// on the integer pipe (imul64, the same bits): an SM sub-core takes 64 clocks
+// per FP64 warp instruction, 24 of them a step, and the chain has nine.  All
+// eight are computed without a branch and tested together; a step with an
+// operand that imul64 does not take (a zero, say) runs in FP64.  20 macro steps
+// (periods known): 10^4 particles 1539 -> 1215 us, 4 10^4 4.45 -> 2.43 ms.  (With a
+// branch per product, or all twelve on the integer pipe, 10^4 took 2.8 and 3.6 ms:
+// a product's latency is then exposed.)
+__device__ __forceinline__ void lawson_step_analytic(const DevParams& P, int field, double& R,
+                                                     double& V) {
+    if (field != 1) {
+        lawson_step_analytic_fp64(P, field, R, V);
+        return;
+    }
+    double chR, c1R, s1R, s1e1, r3, e3n, r4, e4n;
+    bool ok = imul64(P.ch, R, chR) & imul64(P.c1, R, c1R) & imul64(P.s1, R, s1R);
+    const double e1 = field_analytic(field, R);
+    const double R3 = fma(P.sh, V, chR);
+    const double R2 = fma(P.sh, fma(P.h2, e1, V), chR);
+    ok = ok & imul64(R3, R3, r3) & imul64(P.s1, e1, s1e1);
+    const double e2 = field_analytic(field, R2);
+    ok = ok & imul64(r3, R3, e3n);
+    const double A = fma(P.s1, V, c1R);
+    const double R4 = fma(P.hsh, -e3n, A);
+    ok = ok & imul64(R4, R4, r4);
+    const double B = fma(P.c1, V, -s1R);
+    const double e23 = e2 + -e3n;
+    ok = ok & imul64(r4, R4, e4n);
+    if (!ok) {
+        lawson_step_analytic_fp64(P, field, R, V);
+        return;
+    }
+    R = fma(P.h6, fma(P.tsh, e23, s1e1), A);
+    V = fma(P.h6, fma(P.tch, e23, fma(P.c1, e1, -e4n)), B);
 }
 
 // ============================================================ FP32 form

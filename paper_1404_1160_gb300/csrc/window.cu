@@ -33,7 +33,6 @@ __global__ void __launch_bounds__(256) k_window_local(DevParams P, WinBufs B, in
         if (mode == MODE_PERIODS) {
             Track s;
             s.flags = 0;
-            s.t1 = 0.0;
             s.T = 0.0;
             double vkm2 = 0.0;
             int K = 0;
@@ -57,7 +56,6 @@ __global__ void __launch_bounds__(256) k_window_local(DevParams P, WinBufs B, in
         // MODE_ETD: n_iter macro steps of this particle
         Track base;
         base.flags = 0;
-        base.t1 = 0.0;
         if (T_known) track_resolve(base, P, Tin[i]);
         Track s = base;
         int K = 0;
@@ -94,8 +92,7 @@ __global__ void __launch_bounds__(256) k_window_local(DevParams P, WinBufs B, in
                 }
             } else {
                 s.flags = 0;
-                s.t1 = 0.0;
-                double vkm2 = 0.0;
+                    double vkm2 = 0.0;
                 K = 0;
                 B.traj[i] = make_double2(R, V);
                 for (;;) {

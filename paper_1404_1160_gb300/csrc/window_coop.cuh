@@ -440,7 +440,6 @@ __global__ void __launch_bounds__(kWinMaxThreads) k_window_coop(DevParams P, Win
             if (T_known) {
                 Track s;
                 s.flags = 0;
-                s.t1 = 0.0;
                 track_resolve(s, P, Tin[i]);
                 B.T[i] = s.T;
                 B.o[i] = s.o;
