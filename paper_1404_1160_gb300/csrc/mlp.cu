@@ -537,6 +537,8 @@ static cudaError_t launch_mlp_tc(const MlpDev& D, const LearnedArgs& A, int mode
 //                               tiles (rows 64..127 of the operand are zero)
 //   dz1 = dh1 gelu'(z1)
 //   dW1, db1, db2, dW3, db3     on the CUDA cores, sums over the tile in registers
+// Rows past the batch enter every sum as zeros, whatever the weights (an
+// infinite weight times a zero dout would be NaN).
 // Nothing per sample goes through global memory.  The step is latency-bound
 // (64 tiles at the usual batch of 8192): with one thread per sample and a
 // second kernel that reloaded every record for the gradients, the two took 32
@@ -694,7 +696,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train_tc(MlpDev M, const flo
                 z[q] = fmaf(wa.z, x[2], z[q]);
                 z[q] = fmaf(wa.w, x[3], z[q]);
                 z[q] = fmaf(wb.x, x[4], z[q]);
-                h[q] = gelu_for_bf16(z[q], S.gtab);
+                h[q] = valid ? gelu_for_bf16(z[q], S.gtab) : 0.f;
             }
             *reinterpret_cast<float4*>(&S.d1[row][c]) = make_float4(z[0], z[1], z[2], z[3]);
             tc_put4(S.A, Htr, row, c, h);
@@ -719,9 +721,9 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train_tc(MlpDev M, const flo
 #pragma unroll 1
         for (int c = cb * 16; c < cb * 16 + 16; c += 4) {
             const float4 z = *reinterpret_cast<const float4*>(&S.d2[row][c]);
-            *reinterpret_cast<uint2*>(&S.h2[row][c]) =
-                make_uint2(pack_bf16(gelu_for_bf16(z.x, S.gtab), gelu_for_bf16(z.y, S.gtab)),
-                           pack_bf16(gelu_for_bf16(z.z, S.gtab), gelu_for_bf16(z.w, S.gtab)));
+            const uint2 h = make_uint2(pack_bf16(gelu_for_bf16(z.x, S.gtab), gelu_for_bf16(z.y, S.gtab)),
+                                       pack_bf16(gelu_for_bf16(z.z, S.gtab), gelu_for_bf16(z.w, S.gtab)));
+            *reinterpret_cast<uint2*>(&S.h2[row][c]) = valid ? h : make_uint2(0u, 0u);
         }
         // output layer: chain q takes the columns 8 nt + 2 q + e in order, warp by warp
 #pragma unroll 1
@@ -773,7 +775,7 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train_tc(MlpDev M, const flo
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const float4 w = S.l3[c + q];
-                v[q] = fmaf(w.z, xd1.z, w.y * xd1.y) * gelu_d(v[q]);
+                v[q] = valid ? fmaf(w.z, xd1.z, w.y * xd1.y) * gelu_d(v[q]) : 0.f;
             }
             *zp = make_float4(v[0], v[1], v[2], v[3]);
             tc_put4(S.A, Atr, row, c, v);
@@ -803,7 +805,8 @@ __global__ void __launch_bounds__(kTrThreads) k_mlp_train_tc(MlpDev M, const flo
             for (int i = 0; i < 16; i += 4) {
                 float4* gp = reinterpret_cast<float4*>(&S.d1[row][cb * 16 + i]);
                 const float4 g = *gp;
-                *gp = make_float4(d[i] * g.x, d[i + 1] * g.y, d[i + 2] * g.z, d[i + 3] * g.w);
+                *gp = valid ? make_float4(d[i] * g.x, d[i + 1] * g.y, d[i + 2] * g.z, d[i + 3] * g.w)
+                            : make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
         tc_fence_before();  // this tile's TMEM reads come before the next tile's MMA

@@ -41,6 +41,24 @@ def test_gradients_at_tile_edges(n):
     m.close()
 
 
+@pytest.mark.parametrize("block", [(name, at) for name in ("W1", "b1", "W2", "b2", "W3", "b3") for at in (0, -1)])
+def test_rows_past_the_batch_add_nothing(block):
+    # one sample repeated: 127 rows and a whole tile of 128 have the same infinities
+    # and NaNs in every gradient, also where a weight is infinite
+    p = omlp.unflatten(weights(8).astype(np.float64))
+    p[block[0]].flat[block[1]] = np.inf
+    w = omlp.flatten(p).astype(np.float32)
+    X, T = batch(1, 4)
+    out = []
+    for n in (127, 128):
+        m = pic.pic_mlp_create(n)
+        pic.pic_mlp_set_weights(m, w)
+        out.append(pic.pic_mlp_gradients(m, dev(np.repeat(X, n, 0)), dev(np.repeat(T, n, 0)))[0])
+        m.close()
+    assert np.array_equal(np.isnan(out[0]), np.isnan(out[1]))
+    assert np.array_equal(np.isposinf(out[0]), np.isposinf(out[1])) and np.array_equal(np.isneginf(out[0]), np.isneginf(out[1]))
+
+
 @pytest.mark.parametrize("n", [127, 129, 12 * 152 * 128 + 1])
 def test_forward_at_tile_edges(n):
     m = pic.pic_mlp_create(16)
