@@ -184,7 +184,7 @@ __global__ void k_zero_charge(unsigned long long* __restrict__ Q, int n, unsigne
 // kFieldFusedCells cells, where the block also evaluates the field.  Beyond, the
 // ~13 FP64 operations per node (a division among them) would take one SM's
 // pipe longer than a second launch: the block leaves S_j in E's own storage for
-// k_field_in_place.
+// k_field_in_place (and finishes the axis node, whose field is no S_j).
 constexpr int kFieldBlock = 1024;
 constexpr int kFieldBlockCells = 4 * kFieldBlock - 2;
 constexpr int kFieldFusedCells = 512;
@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(kFieldBlock) k_field_block(DevParams P, const 
     for (int r = 0; r < R; ++r) {
         const int j = j0 + r;
         if (j > Nc) break;
-        if (fused) field_node(P, Q, j, g, E, edges);
+        if (fused || j == P.c) field_node(P, Q, j, g, E, edges);
         else E[j] = __longlong_as_double(g);
         g += j < Nc ? q[r] + q[r + 1] : 0ll;
     }
@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kFieldBlock) k_field_block(DevParams P, const 
 __global__ void k_field_in_place(DevParams P, const long long* __restrict__ Q, double* __restrict__ E,
                                  double* __restrict__ edges) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j <= P.n_cells) field_node(P, Q, j, __double_as_longlong(E[j]), E, edges);
+    if (j <= P.n_cells && j != P.c) field_node(P, Q, j, __double_as_longlong(E[j]), E, edges);
 }
 
 // ------------------------------------------------- decoupled look-back scan

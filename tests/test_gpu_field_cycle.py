@@ -188,6 +188,17 @@ def test_field_from_one_block(n_cells, parity):
     assert bit_equal(E.cpu().numpy(), Eo) and bit_equal(edges.cpu().numpy(), eo)
 
 
+@pytest.mark.parametrize("n_cells", [256, 1024, 4094, 8192])
+def test_field_in_the_storage_of_the_charge(n_cells):
+    p = pic.pic_default_params(n_cells=n_cells)
+    Q = np.random.default_rng(n_cells).integers(0, 1 << 40, n_cells + 1).astype(np.int64)
+    q = torch.from_numpy(Q).cuda()
+    edges = torch.empty(2, dtype=torch.float64, device="cuda")
+    pic.pic_poisson(p, 12345, q, q.view(torch.float64), edges)
+    _, Eo, eo = oracle.poisson(cfg_of(p), Q, 12345)
+    assert bit_equal(q.view(torch.float64).cpu().numpy(), Eo) and bit_equal(edges.cpu().numpy(), eo)
+
+
 @pytest.mark.parametrize("n_cells", [2, 6, 512, 1022, 1026, 65536])
 def test_frozen_potential_of_any_mesh(n_cells):
     # psi at the nodes against long double sums: (n_cells + 4) binary64 roundings of
