@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(256) k_window_local(DevParams P, WinBufs B, in
                 }
             } else {
                 s.flags = 0;
-                    double vkm2 = 0.0;
+                double vkm2 = 0.0;
                 K = 0;
                 B.traj[i] = make_double2(R, V);
                 for (;;) {
