@@ -261,7 +261,7 @@ int pic_deposit_f32(const pic_params* p, int64_t n, const float* R_dev, int64_t*
    then rE_j = S_j * q_unit/2, E_j = rE_j * (1/r_j), and at r = 0
    E = rho(0) = Q * q_unit / h_r, with q_unit = total_charge/(n_particles*W).
    Reads Q_dev (n_cells+1), writes E_dev (n_cells+1) and rE_edges_dev (2:
-   rE at r_min and r_max).  Meshes of up to 4094 cells are solved by one
+   rE at r_min and r_max).  Meshes of up to 16382 cells are solved by one
    block without scratch; larger ones use device scratch that the call
    allocates and frees on the stream, and synchronise it to read the
    status of the look-back. */
@@ -280,7 +280,7 @@ int pic_poisson(const pic_params* p, int64_t n_particles, const int64_t* Q_dev, 
    looks up the array's device address.  All calls share the one array:
    each call clears the parts that must start at zero, and calls whose work
    overlaps on the GPU (different streams, or different host threads,
-   without ordering between them) race on it (meshes of up to 4094 cells
+   without ordering between them) race on it (meshes of up to 16382 cells
    need no scratch).  Every call synchronises `stream`, so it cannot be made
    while `stream` is being captured into a graph. */
 int pic_poisson_noalloc(const pic_params* p, int64_t n_particles, const int64_t* Q_dev, double* E_dev,

@@ -1,6 +1,7 @@
 // mesh.cu -- standalone field-cycle kernels: CIC deposit, trapezoid prefix
 // integral (decoupled look-back int64 scan) and gather (Sec. 2.3 of Frenod,
 // Hirstoaga & Lutz; eq. VlasPoissAxSymBeam).
+#include <algorithm>
 #include <mutex>
 
 #include "pic.h"
@@ -179,15 +180,20 @@ __global__ void k_zero_charge(unsigned long long* __restrict__ Q, int n, unsigne
 
 // ------------------------------------------------- field of a small mesh, one block
 //
-// S_j = G_j - G_c of every node (see below for G) by one block, R consecutive
-// nodes per thread: no scratch, no status, no second launch up to
-// kFieldFusedCells cells, where the block also evaluates the field.  Beyond, the
-// ~13 FP64 operations per node (a division among them) would take one SM's
-// pipe longer than a second launch: the block leaves S_j in E's own storage for
-// k_field_in_place (and finishes the axis node, whose field is no S_j).
+// S_j = G_j - G_c of every node (see below for G) by one block: warp w takes 32 R
+// consecutive nodes, 32 at a time (coalesced), and scans them with shuffles.  No
+// scratch, no status, no second launch up to kFieldFusedCells cells, where the
+// block also evaluates the field.  Beyond, the ~13 FP64 operations per node (a
+// division among them) would take one SM's pipe longer than a second launch:
+// the block leaves S_j in E's own storage for k_field_in_place (and finishes the
+// axis node, whose field is no S_j).  The line lies where R = 16 still fits the
+// registers: 256 / 1024 / 4096 / 10000 cells take 4.6 / 8.2 / 12.4 / 14.4 us a call.
+// The look-back form beyond it allocates scratch and waits for the host (34 us a
+// call on these meshes, 200 us more after the pool was emptied).
 constexpr int kFieldBlock = 1024;
-constexpr int kFieldBlockCells = 4 * kFieldBlock - 2;
+constexpr int kFieldBlockCells = 16 * kFieldBlock - 2;
 constexpr int kFieldFusedCells = 512;
+static_assert(kFieldFusedCells < kFieldBlock, "one node per thread");
 
 __device__ __forceinline__ void field_node(const DevParams& P, const long long* __restrict__ Q, int j, long long S,
                                            double* __restrict__ E, double* __restrict__ edges) {
@@ -223,35 +229,37 @@ __global__ void __launch_bounds__(kFieldBlock) k_field_block(DevParams P, const 
                                                              int fused) {
     __shared__ long long s_tot[kFieldBlock / 32], s_c;
     const int Nc = P.n_cells, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int j0 = threadIdx.x * R;
-    long long q[R + 1];
+    const int j0 = w * 32 * R + lane;
+    long long g[R], total = 0;
 #pragma unroll
-    for (int r = 0; r <= R; ++r) q[r] = j0 + r <= Nc ? Q[j0 + r] : 0ll;
-    long long L = 0;
+    for (int r = 0; r < R; ++r) {
+        const int j = j0 + 32 * r;
+        g[r] = j < Nc ? Q[j] + Q[j + 1] : 0ll;
+    }
 #pragma unroll
-    for (int r = 0; r < R; ++r) L += j0 + r < Nc ? q[r] + q[r + 1] : 0ll;
-    const long long incl = warp_incl_scan(L);
-    if (lane == 31) s_tot[w] = incl;
+    for (int r = 0; r < R; ++r) {
+        const long long incl = warp_incl_scan(g[r]);
+        g[r] = total + incl - g[r];
+        total += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) s_tot[w] = total;
     __syncthreads();
     long long t = lane < w ? s_tot[lane] : 0ll;
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) t += __shfl_xor_sync(0xffffffffu, t, d);
-    long long g = t + incl - L, run = g;
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        if (j0 + r == P.c) s_c = run;
-        run += j0 + r < Nc ? q[r] + q[r + 1] : 0ll;
-    }
+    for (int r = 0; r < R; ++r)
+        if (j0 + 32 * r == P.c) s_c = t + g[r];
     __syncthreads();
-    g -= s_c;
+    t -= s_c;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int j = j0 + r;
+        const int j = j0 + 32 * r;
         if (j > Nc) break;
-        if (fused || j == P.c) field_node(P, Q, j, g, E, edges);
-        else E[j] = __longlong_as_double(g);
-        g += j < Nc ? q[r] + q[r + 1] : 0ll;
+        if (R == 1 && fused) field_node(P, Q, j, t + g[r], E, edges);
+        else if (j != P.c) E[j] = __longlong_as_double(t + g[r]);
     }
+    if (!(R == 1 && fused) && threadIdx.x == 0) field_node(P, Q, P.c, 0ll, E, edges);
 }
 
 __global__ void k_field_in_place(DevParams P, const long long* __restrict__ Q, double* __restrict__ E,
@@ -473,11 +481,14 @@ static cudaError_t deposit_with(Split split_fn, Wide wide_fn, const DevParams& P
         const int copies = 4 * per_copy <= 48 * 1024 ? 4 : (2 * per_copy <= 48 * 1024 ? 2 : 1);
         const size_t smem = copies * per_copy;
         if (smem > 48 * 1024) cudaFuncSetAttribute(split_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        // one block per SM, and no block beyond its positions: whole rounds of
-        // kSplitThreads positions each
+        // one block per SM, or as many full waves of them as keep every block
+        // within its positions (whole rounds of kSplitThreads positions each).  The
+        // least number of blocks instead left 2 of 306 to a wave of their own: 2 10^7
+        // positions on 1000 cells took 238 us, now 166 (64-bit form 167); on 256
+        // cells 117, now 84 (64-bit form 126).
         const long long rounds = (n + kSplitThreads - 1) / kSplitThreads, most = kSplitPositions / kSplitThreads;
-        long long grid = rounds < sm_count ? rounds : sm_count;
-        if (grid * most < rounds) grid = (rounds + most - 1) / most;
+        const long long waves = (rounds + most * sm_count - 1) / (most * sm_count);
+        const long long grid = rounds < sm_count ? rounds : waves * sm_count;
         split_fn<<<(int)grid, kSplitThreads, smem, st>>>(P, R, (unsigned int)n, r_stride, (unsigned long long*)Q,
                                                          (unsigned long long*)n_out, copies);
     } else {
@@ -542,8 +553,8 @@ cudaError_t launch_poisson(const DevParams& P, const long long* Q, double* E, do
     if (poisson_in_block(P.n_cells)) {
         const int fused = P.n_cells <= kFieldFusedCells;
         if (P.n_cells < kFieldBlock) k_field_block<1><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
-        else if (P.n_cells < 2 * kFieldBlock) k_field_block<2><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
-        else k_field_block<4><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
+        else if (P.n_cells < 4 * kFieldBlock) k_field_block<4><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
+        else k_field_block<16><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
         if (!fused) k_field_in_place<<<(P.n_cells + 256) / 256, 256, 0, st>>>(P, Q, E, edges);
         if (launches) *launches += fused ? 1 : 2;
         return cudaGetLastError();
@@ -567,8 +578,14 @@ cudaError_t launch_gather(const DevParams& P, const double* R, long long n, cons
     auto fn = P.xs_fma ? k_gather<1> : k_gather<0>;
     if (use_smem && smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     long long want = (n + 255) / 256;
-    want = (want + kGatherAhead - 1) / kGatherAhead;
-    int grid = (int)(want < (long long)sm_count * 8 ? want : (long long)sm_count * 8);
+    // one position per thread while the GPU has room, then kGatherAhead in flight.
+    // Each block builds its table (two FP64 operations per cell, about a quarter of
+    // four positions'), so the blocks per SM follow the positions per cell.
+    // (10^6 positions on 4096 cells: 977 blocks 30.8 us, 608 blocks 26.6, 304
+    // 16.5; 10^5 on 256 cells: 98 blocks 6.2, 391 blocks 5.1.)
+    long long per_sm = 8;
+    if (use_smem) per_sm = std::min(per_sm, 2 + n / (4ll * sm_count * P.n_cells));
+    const int grid = (int)std::min(want, per_sm * sm_count);
     fn<<<grid, 256, use_smem ? smem : 0, st>>>(P, R, n, E, edges, out, use_smem);
     if (launches) ++*launches;
     return cudaGetLastError();

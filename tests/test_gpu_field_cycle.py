@@ -176,7 +176,7 @@ def test_deposit_forms(n, n_cells, log2W):
     assert np.array_equal(Q.cpu().numpy(), Qo) and int(n_out) == no
 
 
-@pytest.mark.parametrize("n_cells", [2, 30, 510, 512, 514, 1022, 1024, 2046, 2048, 4094, 4096])
+@pytest.mark.parametrize("n_cells", [2, 30, 510, 512, 514, 1022, 1024, 2046, 2048, 4094, 4096, 8192, 16382, 16384])
 @pytest.mark.parametrize("parity", [pic.PIC_PARITY_EVEN, pic.PIC_PARITY_ODD])
 def test_field_from_one_block(n_cells, parity):
     p = pic.pic_default_params(n_cells=n_cells, field_parity=parity)
@@ -188,7 +188,7 @@ def test_field_from_one_block(n_cells, parity):
     assert bit_equal(E.cpu().numpy(), Eo) and bit_equal(edges.cpu().numpy(), eo)
 
 
-@pytest.mark.parametrize("n_cells", [256, 1024, 4094, 8192])
+@pytest.mark.parametrize("n_cells", [256, 1024, 4094, 8192, 16382, 16384])
 def test_field_in_the_storage_of_the_charge(n_cells):
     p = pic.pic_default_params(n_cells=n_cells)
     Q = np.random.default_rng(n_cells).integers(0, 1 << 40, n_cells + 1).astype(np.int64)
