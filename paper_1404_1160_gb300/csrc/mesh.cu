@@ -583,8 +583,10 @@ cudaError_t launch_gather(const DevParams& P, const double* R, long long n, cons
     // four positions'), so the blocks per SM follow the positions per cell.
     // (10^6 positions on 4096 cells: 977 blocks 30.8 us, 608 blocks 26.6, 304
     // 16.5; 10^5 on 256 cells: 98 blocks 6.2, 391 blocks 5.1.)
-    long long per_sm = 8;
-    if (use_smem) per_sm = std::min(per_sm, 2 + n / (4ll * sm_count * P.n_cells));
+    // Without a table the loads of E go to L2, where more blocks pay for the
+    // largest sets only: 65536 cells, 4 10^6 positions, 4 / 8 blocks per SM 29.5 / 31.4
+    // us; 2 10^7 positions 145 with 8 (157 with 4 and one position in flight).
+    const long long per_sm = use_smem ? std::min(8ll, 2 + n / (4ll * sm_count * P.n_cells)) : (n < (1ll << 23) ? 4 : 8);
     const int grid = (int)std::min(want, per_sm * sm_count);
     fn<<<grid, 256, use_smem ? smem : 0, st>>>(P, R, n, E, edges, out, use_smem);
     if (launches) ++*launches;
