@@ -1460,9 +1460,7 @@ int batch_configure(pic_batch* b, int block, int bps_want, double power, int cop
     if (smem > 227 * 1024) return PIC_ERR_UNSUPPORTED;
     const size_t smem_kept = pic::window32_batch_smem(b->max_cells, copies, block, true);
     if (smem > 0) {
-        // the larger of the new and the current size, so that the current
-        // configuration stays launchable if this one is refused below
-        cudaError_t e = pic::window32_batch_attr(smem > b->smem ? smem : b->smem);
+        cudaError_t e = pic::window32_batch_open();
         if (e != cudaSuccess) return map_cuda(e);
     }
     int bps = 0;
@@ -1473,8 +1471,7 @@ int batch_configure(pic_batch* b, int block, int bps_want, double power, int cop
     // room for the largest mesh's counted charge words where it costs no block
     if (smem_kept > smem && smem_kept <= pic::kWindowSmemMax) {
         int bps_kept = 0;
-        e = pic::window32_batch_attr(smem_kept > b->smem ? smem_kept : b->smem);
-        if (e == cudaSuccess) e = pic::window32_batch_occupancy(block, smem_kept, &bps_kept);
+        e = pic::window32_batch_occupancy(block, smem_kept, &bps_kept);
         if (e != cudaSuccess) return map_cuda(e);
         if (bps_kept >= bps) smem = smem_kept;
     }

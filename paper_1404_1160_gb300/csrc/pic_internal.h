@@ -116,6 +116,12 @@ __host__ __device__ constexpr size_t cycle_words(int n_cells, int block, bool ke
 // Dynamic shared memory a window kernel may take beside its static variables.
 constexpr size_t kWindowSmemMax = 227 * 1024 - 1024;
 
+// Opens all of a block's shared memory to the launches of `fn`: the opt-in limit
+// less what the kernel declares itself (*most, may be null).  The limit belongs to
+// the function, which every handle and batch of the process launches, so it
+// is only ever set to this one value and no caller can lower it under another.
+cudaError_t open_shared_memory(const void* fn, size_t* most);
+
 struct WindowLaunch {
     bool kept = false;        // shared memory for the counted charge words
     int coop_grid = 0, coop_block = 0;
@@ -181,7 +187,7 @@ struct BeamDesc32 {
     unsigned long long* t_ns;  // [2]: first start and last end (global timer, ns) of the beam's blocks
 };
 size_t window32_batch_smem(int max_cells, int copies, int block, bool kept);
-cudaError_t window32_batch_attr(size_t smem);
+cudaError_t window32_batch_open();
 cudaError_t window32_batch_occupancy(int block, size_t smem, int* blocks_per_sm);
 cudaError_t launch_window32_batch(const BeamDesc32* beams, int n_beams, int grid, int block, size_t smem,
                                   cudaStream_t st);

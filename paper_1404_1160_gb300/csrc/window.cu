@@ -222,6 +222,18 @@ static void* coop_fn(int solver, int hist, int pow2, int stage) {
     return solver == 1 ? window_coop_kernel_h1_s1(pow2, stage) : window_coop_kernel_h1_s0(pow2, stage);
 }
 
+cudaError_t open_shared_memory(const void* fn, size_t* most) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
+    if (e != cudaSuccess) return e;
+    const size_t room = (size_t)optin - fa.sharedSizeBytes;
+    if (most) *most = room;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room);
+}
+
 cudaError_t window_prepare(DevParams& P, int block, int blocks_per_sm, int sm_count, WindowLaunch* L) {
     L->coop_block = block;
     const size_t limit = 220 * 1024;
@@ -252,7 +264,7 @@ cudaError_t window_prepare(DevParams& P, int block, int blocks_per_sm, int sm_co
     int bps = 1 << 30;
     for (int hh = 0; hh < 3; ++hh) {
         void* fn = coop_fn(P.solver, hh, P.xs_fma, L->stage);
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L->coop_smem);
+        cudaError_t e = open_shared_memory(fn, nullptr);
         if (e != cudaSuccess) return e;
         int b = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, block, L->coop_smem);

@@ -937,9 +937,7 @@ size_t window32_batch_smem(int max_cells, int copies, int block, bool kept) {
     return max_cells > 0 ? coop32_smem_bytes(max_cells, copies, block, kept) : 0;
 }
 
-cudaError_t window32_batch_attr(size_t smem) {
-    return cudaFuncSetAttribute(k_window32_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
+cudaError_t window32_batch_open() { return open_shared_memory((const void*)k_window32_batch, nullptr); }
 
 cudaError_t window32_batch_occupancy(int block, size_t smem, int* blocks_per_sm) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_window32_batch, block, smem);
@@ -1065,8 +1063,7 @@ cudaError_t window32_prepare(DevParams& P, int block, int blocks_per_sm, int sm_
     const int unit = sweep == SWEEP_1 ? 32 : 64;
     L->stage = sweep;
     if (L->coop_smem > 227 * 1024) return cudaErrorNotSupported;
-    cudaError_t e = cudaFuncSetAttribute(coop32_fn(sweep), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)L->coop_smem);
+    cudaError_t e = open_shared_memory(coop32_fn(sweep), nullptr);
     if (e != cudaSuccess) return e;
     int bps = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, coop32_fn(sweep), block, L->coop_smem);

@@ -1,0 +1,93 @@
+"""The shared memory that a launch may take belongs to the kernel, which all
+handles and batches of a process share: no handle may take it from another.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1404_1160_gb300 import inputs
+from paper_1404_1160_gb300 import pic
+from tests.gpu_common import bit_equal, cfg_of
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SHORT = dict(steps_per_turn=20, max_window_steps=60)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1404_1160_gb300 import build
+
+    build.build()
+    torch.cuda.set_device(0)
+
+
+# (particles, cells) of handles that live at the same time, the one that takes
+# the most shared memory first
+TOGETHER = [[(20_000, 256), (2000, 256)], [(2000, 1024), (2000, 256)], [(400_000, 256), (3000, 128), (3000, 2048)]]
+
+
+@pytest.mark.parametrize("sizes", TOGETHER)
+@pytest.mark.parametrize("solver", [pic.PIC_FINE_RK4, pic.PIC_FINE_LAWSON_RK4])
+def test_fp64_handles_step_in_turn(sizes, solver):
+    runs = []
+    for n, cells in sizes:
+        p = pic.pic_default_params(n_cells=cells, fine_solver=solver, **SHORT)
+        y = inputs.gaussian_beam(n, seed=n, r_cut=4.0)
+        runs.append([p, y, pic.pic_init(p, *y)])
+    for _ in range(2):
+        for r in runs:
+            pic.pic_step(r[2], 1)
+            ref = oracle.etd_step(cfg_of(r[0]), *r[1])
+            R, V = pic.pic_get_particles(r[2])
+            assert bit_equal(R, ref.R) and bit_equal(V, ref.V)
+            r[1] = (ref.R, ref.V)
+    for r in runs:
+        pic.pic_destroy(r[2])
+
+
+def alone(p, y, steps):
+    h = pic.pic_init(p, *y)
+    pic.pic_step(h, steps)
+    out = pic.pic_get_particles(h)
+    pic.pic_destroy(h)
+    return out
+
+
+@pytest.mark.parametrize("sizes", TOGETHER + [[(700_000, 512), (650_000, 100)]])
+def test_fp32_handles_step_in_turn(sizes):
+    ps = [pic.pic_default_params(precision=1, n_cells=cells, **SHORT) for _, cells in sizes]
+    ys = [inputs.gaussian_beam(n, seed=n, r_cut=4.0) for n, _ in sizes]
+    ref = [alone(p, y, 2) for p, y in zip(ps, ys)]
+    hs = [pic.pic_init(p, *y) for p, y in zip(ps, ys)]
+    for _ in range(2):
+        for h in hs:
+            pic.pic_step(h, 1)
+    for h, (R0, V0) in zip(hs, ref):
+        R, V = pic.pic_get_particles(h)
+        pic.pic_destroy(h)
+        assert bit_equal(R, R0) and bit_equal(V, V0)
+
+
+@pytest.mark.parametrize("cells,copies", [(2048, 1), (1752, 1)])
+def test_batches_step_in_turn(cells, copies):
+    specs = [[(cells, 3000), (128, 2000)], [(128, 4000), (256, 1000)]]
+    bs, ref = [], []
+    for k, spec in enumerate(specs):
+        ps = [pic.pic_default_params(precision=1, n_cells=c, **SHORT) for c, _ in spec]
+        ys = [inputs.gaussian_beam(n, seed=n, r_cut=4.0) for _, n in spec]
+        ref.append([alone(p, y, 2) for p, y in zip(ps, ys)])
+        bs.append(pic.pic_batch_create(ps, ys))
+        if k == 0:
+            pic.pic_batch_set_config(bs[0], 1024, 1, 0.85, 1, copies)
+    for _ in range(2):
+        for b in bs:
+            pic.pic_batch_step(b, 1)
+    for b, rs in zip(bs, ref):
+        for i, (R0, V0) in enumerate(rs):
+            R, V = pic.pic_batch_get_particles(b, i)
+            assert bit_equal(R, R0) and bit_equal(V, V0)
+        b.close()
