@@ -502,8 +502,9 @@ static void* tc_fn(int mode) {
 static cudaError_t tc_setup(int mode, size_t smem, int* per_sm) {
     cudaError_t e = cudaFuncSetAttribute(tc_fn(mode), cudaFuncAttributePreferredSharedMemoryCarveout,
                                          (int)cudaSharedmemCarveoutMaxShared);
-    if (e == cudaSuccess && smem > 48 * 1024)
-        e = cudaFuncSetAttribute(tc_fn(mode), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // 48 KB without opting in hold the kernel's own arrays and the energy check's
+    // tables together: 33 KB leave room for 1278 cells
+    if (e == cudaSuccess && smem > 0) e = open_shared_memory(tc_fn(mode), nullptr);
     if (e == cudaSuccess) *per_sm = tc_blocks_per_sm(tc_fn(mode), smem);
     return e;
 }

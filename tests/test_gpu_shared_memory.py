@@ -1,13 +1,17 @@
 """The shared memory that a launch may take belongs to the kernel, which all
-handles and batches of a process share: no handle may take it from another.
+handles and batches of a process share: no handle may take it from another,
+and every mesh that the windows serve has to launch.
 """
 import numpy as np
 import pytest
 
 import oracle
+from oracle import learned as OL
+from oracle import mlp as omlp
 from paper_1404_1160_gb300 import inputs
 from paper_1404_1160_gb300 import pic
 from tests.gpu_common import bit_equal, cfg_of
+from tests.test_gpu_f32 import f32
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -91,3 +95,33 @@ def test_batches_step_in_turn(cells, copies):
             R, V = pic.pic_batch_get_particles(b, i)
             assert bit_equal(R, R0) and bit_equal(V, V0)
         b.close()
+
+
+@pytest.mark.parametrize("cells", [1278, 1280, 1620, 1622, 2048])
+def test_learned_step_of_the_fp32_form_on_fine_meshes(cells):
+    # a constant correction (W3 = 0: the output is b3 exactly) judged by the
+    # frozen-field energy, with the tables of the check in shared memory
+    n, scale, tol = 20_001, (2.0**-9, 2.0**-10), 2e-3
+    p = pic.pic_default_params(precision=1, dt=0.4, n_cells=cells, r_min=-2.0, r_max=2.0)
+    c = cfg_of(p)
+    R0, V0 = (f32(x).astype(np.float64) for x in inputs.gaussian_beam(n, seed=21))
+    w = np.zeros(omlp.N_PARAMS, np.float32)
+    w[-2:] = (1.0, -0.75)
+    m = pic.pic_mlp_create(16)
+    pic.pic_mlp_set_weights(m, w)
+    Rp, Vp = alone(p, (R0, V0), 1)
+    h = pic.pic_init(p, R0, V0)
+    n_fb = pic.pic_step_learned(h, m, 1, scale=scale, drift_tol=tol)
+    R, V = pic.pic_get_particles(h)
+    assert pic.pic_moments(h)["n_steps"] == 1
+    pic.pic_destroy(h)
+    m.close()
+    E, edges = OL.mesh_field(c, R0, n, precision=1)
+    Ro, Vo, keep, margin = OL.learned_apply(c, Rp, Vp, np.full(n, scale[0]), np.full(n, -0.75 * scale[1]), tol, E, edges, 1)
+    # the decision is the oracle's but within the rounding of H on either side
+    psi = float(np.abs(OL.node_potential(c, E)).max())
+    sure = np.abs(margin) > 1e-10 * (np.abs(OL.frozen_energy(c, Rp, Vp, E, edges)) + c.eps * psi)
+    assert sure.mean() > 0.999 and 0.05 < keep.mean() < 0.95
+    assert bit_equal(R[sure], Ro[sure]) and bit_equal(V[sure], Vo[sure])
+    fb = int((~keep & sure).sum())
+    assert fb <= n_fb <= fb + int((~sure).sum())
