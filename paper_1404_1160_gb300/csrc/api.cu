@@ -1457,19 +1457,18 @@ int batch_configure(pic_batch* b, int block, int bps_want, double power, int cop
     if (block < 128 || block > 1024 || (block & 31)) return PIC_ERR_INVALID_ARG;
     if (copies != 1 && copies != 2 && copies != 4) return PIC_ERR_INVALID_ARG;
     size_t smem = pic::window32_batch_smem(b->max_cells, copies, block, false);
-    if (smem > 227 * 1024) return PIC_ERR_UNSUPPORTED;
+    size_t room = 0;
+    cudaError_t e = pic::window32_batch_open(&room);
+    if (e != cudaSuccess) return map_cuda(e);
+    if (smem > room) return PIC_ERR_UNSUPPORTED;
     const size_t smem_kept = pic::window32_batch_smem(b->max_cells, copies, block, true);
-    if (smem > 0) {
-        cudaError_t e = pic::window32_batch_open();
-        if (e != cudaSuccess) return map_cuda(e);
-    }
     int bps = 0;
-    cudaError_t e = pic::window32_batch_occupancy(block, smem, &bps);
+    e = pic::window32_batch_occupancy(block, smem, &bps);
     if (e != cudaSuccess) return map_cuda(e);
     if (bps < 1) return PIC_ERR_UNSUPPORTED;
     if (bps_want > 0 && bps_want < bps) bps = bps_want;
     // room for the largest mesh's counted charge words where it costs no block
-    if (smem_kept > smem && smem_kept <= pic::kWindowSmemMax) {
+    if (smem_kept > smem && smem_kept <= room) {
         int bps_kept = 0;
         e = pic::window32_batch_occupancy(block, smem_kept, &bps_kept);
         if (e != cudaSuccess) return map_cuda(e);

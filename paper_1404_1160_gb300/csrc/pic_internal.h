@@ -113,9 +113,6 @@ enum WindowMode { MODE_PERIODS = 0, MODE_ETD = 1, MODE_FINE = 2 };
 __host__ __device__ constexpr size_t cycle_words(int n_cells, int block, bool kept) {
     return field_in_regs(n_cells, block) ? (kept ? 2 * (2 * ((size_t)n_cells + 1) + 1) : 0) : 2 * ((size_t)n_cells + 1);
 }
-// Dynamic shared memory a window kernel may take beside its static variables.
-constexpr size_t kWindowSmemMax = 227 * 1024 - 1024;
-
 // Opens all of a block's shared memory to the launches of `fn`: the opt-in limit
 // less what the kernel declares itself (*most, may be null).  The limit belongs to
 // the function, which every handle and batch of the process launches, so it
@@ -187,7 +184,8 @@ struct BeamDesc32 {
     unsigned long long* t_ns;  // [2]: first start and last end (global timer, ns) of the beam's blocks
 };
 size_t window32_batch_smem(int max_cells, int copies, int block, bool kept);
-cudaError_t window32_batch_open();
+// Opens the batch kernel's shared memory; *most: what a launch can take.
+cudaError_t window32_batch_open(size_t* most);
 cudaError_t window32_batch_occupancy(int block, size_t smem, int* blocks_per_sm);
 cudaError_t launch_window32_batch(const BeamDesc32* beams, int n_beams, int grid, int block, size_t smem,
                                   cudaStream_t st);

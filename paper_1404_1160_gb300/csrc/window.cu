@@ -259,15 +259,20 @@ cudaError_t window_prepare(DevParams& P, int block, int blocks_per_sm, int sm_co
     else L->stage = smem(1, STAGE_NEXT, false) <= limit ? STAGE_NEXT : STAGE_NONE;
     while (copies > 1 && smem(copies, L->stage, false) > limit) copies >>= 1;
     P.hist_copies = copies;
-    L->kept = regs && smem(copies, L->stage, true) <= kWindowSmemMax;
+    size_t room = ~(size_t)0;
+    for (int hh = 0; hh < 3; ++hh) {
+        size_t most = 0;
+        const cudaError_t e = open_shared_memory(coop_fn(P.solver, hh, P.xs_fma, L->stage), &most);
+        if (e != cudaSuccess) return e;
+        room = most < room ? most : room;
+    }
+    L->kept = regs && smem(copies, L->stage, true) <= room;
     L->coop_smem = smem(copies, L->stage, L->kept);
     int bps = 1 << 30;
     for (int hh = 0; hh < 3; ++hh) {
-        void* fn = coop_fn(P.solver, hh, P.xs_fma, L->stage);
-        cudaError_t e = open_shared_memory(fn, nullptr);
-        if (e != cudaSuccess) return e;
         int b = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, block, L->coop_smem);
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &b, coop_fn(P.solver, hh, P.xs_fma, L->stage), block, L->coop_smem);
         if (e != cudaSuccess) return e;
         bps = b < bps ? b : bps;
     }

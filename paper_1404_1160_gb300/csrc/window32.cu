@@ -937,7 +937,7 @@ size_t window32_batch_smem(int max_cells, int copies, int block, bool kept) {
     return max_cells > 0 ? coop32_smem_bytes(max_cells, copies, block, kept) : 0;
 }
 
-cudaError_t window32_batch_open() { return open_shared_memory((const void*)k_window32_batch, nullptr); }
+cudaError_t window32_batch_open(size_t* most) { return open_shared_memory((const void*)k_window32_batch, most); }
 
 cudaError_t window32_batch_occupancy(int block, size_t smem, int* blocks_per_sm) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_window32_batch, block, smem);
@@ -1049,8 +1049,6 @@ cudaError_t window32_prepare(DevParams& P, int block, int blocks_per_sm, int sm_
                           copies * P.n_cells > 2048 || per_block_est < 512ll * copies))
         copies >>= 1;
     P.hist_copies = copies;
-    L->kept = field_in_regs(P.n_cells, block) && coop32_smem_bytes(P.n_cells, copies, block, true) <= kWindowSmemMax;
-    L->coop_smem = coop32_smem_bytes(P.n_cells, copies, block, L->kept);
     L->hist = 0;
     // One slot per lane while a warp has up to four such units (the tail of a
     // sweep is a unit, and a unit a chain of latencies); two beyond; and once
@@ -1062,9 +1060,12 @@ cudaError_t window32_prepare(DevParams& P, int block, int blocks_per_sm, int sm_
     const int sweep = P.n <= 128 * warps ? SWEEP_1 : (20 * P.n <= (64ll << 20) ? SWEEP_2 : SWEEP_2_AHEAD);
     const int unit = sweep == SWEEP_1 ? 32 : 64;
     L->stage = sweep;
-    if (L->coop_smem > 227 * 1024) return cudaErrorNotSupported;
-    cudaError_t e = open_shared_memory(coop32_fn(sweep), nullptr);
+    size_t room = 0;
+    cudaError_t e = open_shared_memory(coop32_fn(sweep), &room);
     if (e != cudaSuccess) return e;
+    L->kept = field_in_regs(P.n_cells, block) && coop32_smem_bytes(P.n_cells, copies, block, true) <= room;
+    L->coop_smem = coop32_smem_bytes(P.n_cells, copies, block, L->kept);
+    if (L->coop_smem > room) return cudaErrorNotSupported;
     int bps = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, coop32_fn(sweep), block, L->coop_smem);
     if (e != cudaSuccess) return e;

@@ -76,7 +76,8 @@ def test_fp32_handles_step_in_turn(sizes):
         assert bit_equal(R, R0) and bit_equal(V, V0)
 
 
-@pytest.mark.parametrize("cells,copies", [(2048, 1), (1752, 1)])
+# 1752 cells with two histogram copies: within 1 KB of all the shared memory a block can have
+@pytest.mark.parametrize("cells,copies", [(2048, 1), (1752, 2), (1752, 1)])
 def test_batches_step_in_turn(cells, copies):
     specs = [[(cells, 3000), (128, 2000)], [(128, 4000), (256, 1000)]]
     bs, ref = [], []
