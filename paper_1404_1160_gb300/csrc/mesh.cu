@@ -465,6 +465,16 @@ cudaError_t launch_unpack(const double2* y, double* R, double* V, long long n, i
     return cudaGetLastError();
 }
 
+// Shared memory that a block's histograms or field table may take.  A kernel that
+// needs more than the 48 KB it has without asking is given all of it: the limit is
+// the kernel's, and a thread that set its own mesh's size could lower it between
+// another thread's setting and launch.
+constexpr size_t kMeshSmem = 96 * 1024;
+static cudaError_t open_mesh_smem(const void* fn, size_t smem) {
+    return smem > 48 * 1024 ? cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMeshSmem)
+                            : cudaSuccess;
+}
+
 // Zeroed charge and out-of-mesh count, then the split form where it serves
 // (its histograms of 12 bytes per cell and copy within 48 KB, or 96 KB with one
 // copy), else the 64-bit form.
@@ -477,10 +487,10 @@ static cudaError_t deposit_with(Split split_fn, Wide wide_fn, const DevParams& P
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || n == 0) return e;
     const size_t per_copy = sizeof(unsigned int) * 3 * (size_t)P.n_cells;
-    if (P.W <= (1ll << 32) && per_copy <= 96 * 1024 && n < (1ll << 31)) {
+    if (P.W <= (1ll << 32) && per_copy <= kMeshSmem && n < (1ll << 31)) {
         const int copies = 4 * per_copy <= 48 * 1024 ? 4 : (2 * per_copy <= 48 * 1024 ? 2 : 1);
         const size_t smem = copies * per_copy;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(split_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if ((e = open_mesh_smem((const void*)split_fn, smem)) != cudaSuccess) return e;
         // one block per SM, or as many full waves of them as keep every block
         // within its positions (whole rounds of kSplitThreads positions each).  The
         // least number of blocks instead left 2 of 306 to a wave of their own: 2 10^7
@@ -493,9 +503,8 @@ static cudaError_t deposit_with(Split split_fn, Wide wide_fn, const DevParams& P
                                                          (unsigned long long*)n_out, copies);
     } else {
         const size_t smem = sizeof(unsigned long long) * (size_t)Np1;
-        const int use_smem = smem <= 96 * 1024;
-        if (use_smem && smem > 48 * 1024)
-            cudaFuncSetAttribute(wide_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const int use_smem = smem <= kMeshSmem;
+        if (use_smem && (e = open_mesh_smem((const void*)wide_fn, smem)) != cudaSuccess) return e;
         const long long want = (n + 255) / 256;
         const int grid = (int)(want < (long long)sm_count * 4 ? want : (long long)sm_count * 4);
         wide_fn<<<grid, 256, use_smem ? smem : 0, st>>>(P, R, n, r_stride, (unsigned long long*)Q,
@@ -574,9 +583,12 @@ cudaError_t launch_gather(const DevParams& P, const double* R, long long n, cons
                           long long* launches) {
     if (n == 0) return cudaSuccess;
     size_t smem = sizeof(double2) * (size_t)P.n_cells;
-    int use_smem = smem <= 96 * 1024;
+    int use_smem = smem <= kMeshSmem;
     auto fn = P.xs_fma ? k_gather<1> : k_gather<0>;
-    if (use_smem && smem > 48 * 1024) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (use_smem) {
+        const cudaError_t e = open_mesh_smem((const void*)fn, smem);
+        if (e != cudaSuccess) return e;
+    }
     long long want = (n + 255) / 256;
     // one position per thread while the GPU has room, then kGatherAhead in flight.
     // Each block builds its table (two FP64 operations per cell, about a quarter of

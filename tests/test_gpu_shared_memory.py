@@ -2,6 +2,9 @@
 handles and batches of a process share: no handle may take it from another,
 and every mesh that the windows serve has to launch.
 """
+import ctypes as C
+import threading
+
 import numpy as np
 import pytest
 
@@ -126,3 +129,32 @@ def test_learned_step_of_the_fp32_form_on_fine_meshes(cells):
     assert bit_equal(R[sure], Ro[sure]) and bit_equal(V[sure], Vo[sure])
     fb = int((~keep & sure).sum())
     assert fb <= n_fb <= fb + int((~sure).sum())
+
+
+def test_mesh_calls_of_several_threads():
+    # threads on meshes whose tables need different sizes above 48 KB, on their own streams and buffers
+    cells = [4098, 6000, 8190]
+    bad = []
+
+    def work(c):
+        p = pic.pic_default_params(n_cells=c)
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            R = torch.randn(500, dtype=torch.float64, device="cuda")
+            Q = torch.empty(c + 1, dtype=torch.int64, device="cuda")
+            n_out = torch.empty(1, dtype=torch.int64, device="cuda")
+        s.synchronize()
+        call = pic.load().pic_deposit
+        args = (C.byref(p), R.numel(), R.data_ptr(), Q.data_ptr(), n_out.data_ptr(), s.cuda_stream)
+        status = [call(*args) for _ in range(10_000)]
+        s.synchronize()
+        Qo, no = oracle.deposit(cfg_of(p), R.cpu().numpy())
+        if any(status) or not np.array_equal(Q.cpu().numpy(), Qo) or int(n_out) != no:
+            bad.append((c, sum(x != 0 for x in status)))
+
+    threads = [threading.Thread(target=work, args=(c,)) for c in cells]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad
