@@ -261,7 +261,8 @@ int pic_deposit_f32(const pic_params* p, int64_t n, const float* R_dev, int64_t*
    then rE_j = S_j * q_unit/2, E_j = rE_j * (1/r_j), and at r = 0
    E = rho(0) = Q * q_unit / h_r, with q_unit = total_charge/(n_particles*W).
    Reads Q_dev (n_cells+1), writes E_dev (n_cells+1) and rE_edges_dev (2:
-   rE at r_min and r_max).  Meshes of up to 16382 cells are solved by one
+   rE at r_min and r_max).  E_dev may be Q_dev's own storage; any other overlap
+   is not allowed.  Meshes of up to 16382 cells are solved by one
    block without scratch; larger ones use device scratch that the call
    allocates and frees on the stream, and synchronise it to read the
    status of the look-back. */

@@ -195,8 +195,10 @@ constexpr int kFieldBlockCells = 16 * kFieldBlock - 2;
 constexpr int kFieldFusedCells = 512;
 static_assert(kFieldFusedCells < kFieldBlock, "one node per thread");
 
-__device__ __forceinline__ void field_node(const DevParams& P, const long long* __restrict__ Q, int j, long long S,
-                                           double* __restrict__ E, double* __restrict__ edges) {
+// E may be Q's own storage: neither is __restrict__, and E is accessed as its
+// bits, in the type of Q.
+__device__ __forceinline__ void field_node(const DevParams& P, const long long* Q, int j, long long S, long long* E,
+                                           double* __restrict__ edges) {
     const int Nc = P.n_cells, c = P.c;
     double e;
     if (j == c) {
@@ -206,7 +208,7 @@ __device__ __forceinline__ void field_node(const DevParams& P, const long long* 
         e = ((double)S * P.q_half) * (1.0 / r);
         if (P.parity_odd && j < c) e = -e;  // odd reading: rE / |r|
     }
-    E[j] = e;
+    E[j] = __double_as_longlong(e);
     // the off-mesh gather divides the edge rE by R; the odd reading's
     // lower edge carries the sign flip
     if (j == 0) edges[0] = P.parity_odd ? -((double)S * P.q_half) : (double)S * P.q_half;
@@ -224,9 +226,8 @@ __device__ __forceinline__ long long warp_incl_scan(long long x) {
 }
 
 template <int R>
-__global__ void __launch_bounds__(kFieldBlock) k_field_block(DevParams P, const long long* __restrict__ Q,
-                                                             double* __restrict__ E, double* __restrict__ edges,
-                                                             int fused) {
+__global__ void __launch_bounds__(kFieldBlock) k_field_block(DevParams P, const long long* Q, long long* E,
+                                                             double* __restrict__ edges, int fused) {
     __shared__ long long s_tot[kFieldBlock / 32], s_c;
     const int Nc = P.n_cells, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int j0 = w * 32 * R + lane;
@@ -257,15 +258,14 @@ __global__ void __launch_bounds__(kFieldBlock) k_field_block(DevParams P, const 
         const int j = j0 + 32 * r;
         if (j > Nc) break;
         if (R == 1 && fused) field_node(P, Q, j, t + g[r], E, edges);
-        else if (j != P.c) E[j] = __longlong_as_double(t + g[r]);
+        else if (j != P.c) E[j] = t + g[r];
     }
     if (!(R == 1 && fused) && threadIdx.x == 0) field_node(P, Q, P.c, 0ll, E, edges);
 }
 
-__global__ void k_field_in_place(DevParams P, const long long* __restrict__ Q, double* __restrict__ E,
-                                 double* __restrict__ edges) {
+__global__ void k_field_in_place(DevParams P, const long long* Q, long long* E, double* __restrict__ edges) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j <= P.n_cells && j != P.c) field_node(P, Q, j, __double_as_longlong(E[j]), E, edges);
+    if (j <= P.n_cells && j != P.c) field_node(P, Q, j, E[j], E, edges);
 }
 
 // ------------------------------------------------- decoupled look-back scan
@@ -360,8 +360,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_pairs(DevParams P, const 
 
 // S_j = G_j - G_c (the integral from r = 0), rE_j = S_j q_unit/2,
 // E_j = rE_j * (1/r_j); at r = 0, E = rho(0) = Q_c q_unit / h_r.
-__global__ void k_field_from_prefix(DevParams P, const long long* __restrict__ Q,
-                                    const long long* __restrict__ G, double* __restrict__ E,
+__global__ void k_field_from_prefix(DevParams P, const long long* Q, const long long* __restrict__ G, long long* E,
                                     double* __restrict__ edges) {
     const long long Gc = G[P.c];
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j <= P.n_cells; j += gridDim.x * blockDim.x)
@@ -559,12 +558,13 @@ bool poisson_in_block(int n_cells) { return n_cells <= kFieldBlockCells; }
 
 cudaError_t launch_poisson(const DevParams& P, const long long* Q, double* E, double* edges,
                            const ScanScratch& S, cudaStream_t st, long long* launches) {
+    long long* const Eb = (long long*)E;  // as bits (field_node)
     if (poisson_in_block(P.n_cells)) {
         const int fused = P.n_cells <= kFieldFusedCells;
-        if (P.n_cells < kFieldBlock) k_field_block<1><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
-        else if (P.n_cells < 4 * kFieldBlock) k_field_block<4><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
-        else k_field_block<16><<<1, kFieldBlock, 0, st>>>(P, Q, E, edges, fused);
-        if (!fused) k_field_in_place<<<(P.n_cells + 256) / 256, 256, 0, st>>>(P, Q, E, edges);
+        if (P.n_cells < kFieldBlock) k_field_block<1><<<1, kFieldBlock, 0, st>>>(P, Q, Eb, edges, fused);
+        else if (P.n_cells < 4 * kFieldBlock) k_field_block<4><<<1, kFieldBlock, 0, st>>>(P, Q, Eb, edges, fused);
+        else k_field_block<16><<<1, kFieldBlock, 0, st>>>(P, Q, Eb, edges, fused);
+        if (!fused) k_field_in_place<<<(P.n_cells + 256) / 256, 256, 0, st>>>(P, Q, Eb, edges);
         if (launches) *launches += fused ? 1 : 2;
         return cudaGetLastError();
     }
@@ -573,7 +573,7 @@ cudaError_t launch_poisson(const DevParams& P, const long long* Q, double* E, do
     if (e != cudaSuccess) return e;
     k_scan_pairs<<<tiles, kScanThreads, 0, st>>>(P, Q, S);
     int fgrid = (P.n_cells + 1 + 255) / 256;
-    k_field_from_prefix<<<fgrid, 256, 0, st>>>(P, Q, S.G, E, edges);
+    k_field_from_prefix<<<fgrid, 256, 0, st>>>(P, Q, S.G, Eb, edges);
     if (launches) *launches += 2;
     return cudaGetLastError();
 }
