@@ -263,9 +263,12 @@ int pic_deposit_f32(const pic_params* p, int64_t n, const float* R_dev, int64_t*
    Reads Q_dev (n_cells+1), writes E_dev (n_cells+1) and rE_edges_dev (2:
    rE at r_min and r_max).  E_dev may be Q_dev's own storage; any other overlap
    is not allowed.  Meshes of up to 16382 cells are solved by one
-   block without scratch; larger ones use device scratch that the call
-   allocates and frees on the stream, and synchronise it to read the
-   status of the look-back. */
+   block without scratch, and the call returns without waiting: E_dev and
+   rE_edges_dev are ready in the order of `stream` (another stream or a host
+   thread has to wait for it), and an error while the kernel runs is reported
+   by the next call that synchronises.  Larger meshes use device scratch that
+   the call allocates and frees on the stream; that call synchronises the
+   stream to read the status of the look-back, and returns that status. */
 int pic_poisson(const pic_params* p, int64_t n_particles, const int64_t* Q_dev, double* E_dev,
                 double* rE_edges_dev, void* stream);
 
