@@ -369,9 +369,7 @@ __global__ void k_field_from_prefix(DevParams P, const long long* Q, const long 
 
 // ------------------------------------------------------------------ gather
 
-constexpr int kGatherAhead = 4;
-
-template <int POW2>
+template <int POW2, int AHEAD>
 __global__ void k_gather(DevParams P, const double* __restrict__ R, long long n,
                          const double* __restrict__ E, const double* __restrict__ edges,
                          double* __restrict__ out, int use_smem) {
@@ -384,13 +382,13 @@ __global__ void k_gather(DevParams P, const double* __restrict__ R, long long n,
     }
     const double lo = edges[0], hi = edges[1];
     const long long stride = (long long)gridDim.x * blockDim.x;
-    // kGatherAhead positions per thread in flight
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kGatherAhead * stride) {
-        double r[kGatherAhead];
+    // AHEAD positions per thread in flight
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += AHEAD * stride) {
+        double r[AHEAD];
 #pragma unroll
-        for (int k = 0; k < kGatherAhead; ++k) r[k] = i + k * stride < n ? R[i + k * stride] : 0.0;
+        for (int k = 0; k < AHEAD; ++k) r[k] = i + k * stride < n ? R[i + k * stride] : 0.0;
 #pragma unroll
-        for (int k = 0; k < kGatherAhead; ++k) {
+        for (int k = 0; k < AHEAD; ++k) {
             if (i + k * stride >= n) break;
             const Cell c = mesh_locate<POW2>(P, r[k]);
             double e;
@@ -584,20 +582,24 @@ cudaError_t launch_gather(const DevParams& P, const double* R, long long n, cons
     if (n == 0) return cudaSuccess;
     size_t smem = sizeof(double2) * (size_t)P.n_cells;
     int use_smem = smem <= kMeshSmem;
-    auto fn = P.xs_fma ? k_gather<1> : k_gather<0>;
+    // Without a table the loads of E go to L2, and one position at a time in four
+    // blocks per SM is as fast or faster up to 36 positions per thread (5.6 10^6).  One /
+    // four in flight on 65536 cells: 10^6 positions 10.3 / 11.7 us, 2 10^6 16.5 / 18.2,
+    // 4 10^6 28.8 / 29.1, 6 10^6 45.2 / 43.2, 8 10^6 66.4 / 57.8, 2 10^7 157 / 145.
+    const int one = !use_smem && n <= 36ll * 4 * 256 * sm_count;
+    auto fn = one ? (P.xs_fma ? k_gather<1, 1> : k_gather<0, 1>) : (P.xs_fma ? k_gather<1, 4> : k_gather<0, 4>);
     if (use_smem) {
         const cudaError_t e = open_mesh_smem((const void*)fn, smem);
         if (e != cudaSuccess) return e;
     }
     long long want = (n + 255) / 256;
-    // one position per thread while the GPU has room, then kGatherAhead in flight.
-    // Each block builds its table (two FP64 operations per cell, about a quarter of
-    // four positions'), so the blocks per SM follow the positions per cell.
+    // one position per thread while the GPU has room, then four in flight.  Each block
+    // builds its table (two FP64 operations per cell, about a quarter of four
+    // positions'), so the blocks per SM follow the positions per cell.
     // (10^6 positions on 4096 cells: 977 blocks 30.8 us, 608 blocks 26.6, 304
-    // 16.5; 10^5 on 256 cells: 98 blocks 6.2, 391 blocks 5.1.)
-    // Without a table the loads of E go to L2, where more blocks pay for the
-    // largest sets only: 65536 cells, 4 10^6 positions, 4 / 8 blocks per SM 29.5 / 31.4
-    // us; 2 10^7 positions 145 with 8 (157 with 4 and one position in flight).
+    // 16.5; 10^5 on 256 cells: 98 blocks 6.2, 391 blocks 5.1.)  Without a table eight
+    // blocks pay for the largest sets only (four / eight with four in flight: 6 10^6 43.2 /
+    // 48.4 us, 8 10^6 57.8 / 62.2).
     const long long per_sm = use_smem ? std::min(8ll, 2 + n / (4ll * sm_count * P.n_cells)) : (n < (1ll << 23) ? 4 : 8);
     const int grid = (int)std::min(want, per_sm * sm_count);
     fn<<<grid, 256, use_smem ? smem : 0, st>>>(P, R, n, E, edges, out, use_smem);

@@ -214,3 +214,19 @@ def test_frozen_potential_of_any_mesh(n_cells):
                              torch.zeros(1, dtype=torch.float64, device="cuda"), out)
     bound = (n_cells + 4) * 2.0**-53 * float(np.sum(np.abs(inc)))
     assert np.max(np.abs(psi.cpu().numpy() - ref.astype(np.float64))) <= bound
+
+
+# without a field table in shared memory (more than 6144 cells): one position per thread in flight, or
+# four beyond 36 per thread of four blocks on each of 152 SMs
+@pytest.mark.parametrize("n", [1, 255, 257, 4 * 256 * 152 + 1, 36 * 4 * 256 * 152, 36 * 4 * 256 * 152 + 1])
+@pytest.mark.parametrize("n_cells,r_max", [(6146, 4.0), (65536, 8.0)])
+def test_gather_without_a_table(n, n_cells, r_max):
+    p = pic.pic_default_params(n_cells=n_cells, r_min=-r_max, r_max=r_max)
+    rng = np.random.default_rng(n)
+    R, E, edges = rng.normal(0, 0.5 * r_max, n), rng.normal(0, 1, n_cells + 1), rng.normal(0, 1, 2)
+    R[: min(n, 5)] = [r_max, -r_max, 0.0, np.nan, -np.inf][: min(n, 5)]
+    e = torch.empty(n, dtype=torch.float64, device="cuda")
+    pic.pic_gather(p, torch.from_numpy(R).cuda(), torch.from_numpy(E).cuda(), torch.from_numpy(edges).cuda(), e)
+    eo = oracle.gather(cfg_of(p), R, E, edges)
+    nan = np.isnan(eo)
+    assert np.array_equal(nan, np.isnan(e.cpu().numpy())) and bit_equal(e.cpu().numpy()[~nan], eo[~nan])
