@@ -530,6 +530,26 @@ int init32(pic_handle* h, const double* r0, const double* v0, int ptr_kind) {
     return map_cuda(cudaStreamSynchronize(h->st));
 }
 
+// Threads of a window's blocks where the caller names none.
+//
+// Poisson: 1024, one block per SM.  A beam of up to 16 chunks of 32 particles per SM on
+// a mesh of few nodes per thread takes 512, which leaves room for another handle's
+// block on the same SM and costs one beam nothing: windows with 512 / 1024 threads,
+// 2 10^4 particles on 256 cells FP64 2.07 / 2.08 ms, binary32 1.34 / 1.46; FP64 on 100 cells
+// 1.69 / 1.81, but on 512 cells (three nodes per thread) 2.65 / 2.54; binary32 on 512 cells
+// 1.68 / 1.74, on 1024 (no register build with 512 threads) 3.31 / 2.35; FP64 1.5 10^5
+// particles 3.35 / 3.03.
+//
+// Analytic fields: per-particle windows of up to 16 warps per SM run in blocks of
+// one warp: they spread evenly, and the FP64 pipe is shared by an SM's warps (10^4
+// particles, 313 warps: 3 instead of 4 on the fullest SM).
+int default_block(const pic_params* p, long long n, int sms) {
+    const bool small = n <= 16ll * 32 * sms;
+    if (p->field_model != PIC_FIELD_POISSON) return small ? 32 : 128;
+    const int nodes = p->precision == 1 ? 3 : 2;
+    return small && p->blocks_per_sm <= 1 && p->n_cells + 1 <= nodes * 31 * (512 >> 6) ? 512 : 1024;
+}
+
 }  // namespace
 
 extern "C" {
@@ -593,11 +613,7 @@ int pic_init(const pic_params* p, int64_t n, const double* r0, const double* v0,
     h->st = (cudaStream_t)stream;
     h->sm_count = sms;
     make_devparams(p, n, &h->dp);
-    // per-particle windows of up to 16 warps per SM run in blocks of one warp:
-    // they spread evenly, and the FP64 pipe is shared by an SM's warps (10^4
-    // particles, 313 warps: 3 instead of 4 on the fullest SM)
-    h->block = p->block_size ? p->block_size
-                             : (p->field_model == PIC_FIELD_POISSON ? 1024 : (n <= 16ll * 32 * sms ? 32 : 128));
+    h->block = p->block_size ? p->block_size : default_block(p, n, sms);
 
     if (p->precision == 1) {
         rc = init32(h, r0, v0, ptr_kind);

@@ -237,12 +237,16 @@ cudaError_t open_shared_memory(const void* fn, size_t* most) {
 cudaError_t window_prepare(DevParams& P, int block, int blocks_per_sm, int sm_count, WindowLaunch* L) {
     L->coop_block = block;
     const size_t limit = 220 * 1024;
-    // One chunk per block fills the GPU before a block takes a second one: the
-    // sweeps of a small beam are a chain of FP64 latencies, which more warps
-    // on one SM only lengthen (the FP64 pipe takes 16 clocks per warp
-    // instruction), and a block costs the exchange next to nothing.
+    // A block takes four chunks, one for each quarter of its SM, before another block
+    // takes any: the sweeps of a small beam are a chain of FP64 latencies, which more
+    // warps on one SM only lengthen (the FP64 pipe takes 16 clocks per warp
+    // instruction), while more blocks than that shorten nothing and take SMs from
+    // the windows of other handles.  Chunks per block 1 / 4 / 8 / 16: 2000 particles on 256
+    // cells, Lawson 2.25 / 2.26 / 2.36 / 2.50 ms, RK4 2.26 / 2.27 / 2.42 / 2.78; 2 10^4 (at least
+    // 4.1 chunks) Lawson 2.07 / 2.07 / 2.11 / 2.30, RK4 2.11 / 2.11 / 2.23 / 2.58.
     const long long n_chunks = (P.n + 31) / 32;
-    const long long most = n_chunks < 1 ? 1 : n_chunks;
+    const long long per = block / 32 < 4 ? block / 32 : 4;
+    const long long most = n_chunks < 1 ? 1 : (n_chunks + per - 1) / per;
     const long long min_grid = most < sm_count ? most : sm_count;  // with at least one block per SM
     const unsigned int chunks = (unsigned int)((n_chunks + min_grid - 1) / min_grid);
     // positions one block deposits into one field per cycle: its chunks of 32
