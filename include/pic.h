@@ -96,7 +96,8 @@ typedef struct {
                                   (Poisson 1024, or 512 up to 512 particles per
                                   SM on meshes of up to 494 cells (FP64) or 742
                                   (FP32); otherwise 128, or 32 up to 512
-                                  particles per SM).  Results don't depend on it */
+                                  particles per SM in FP64).  Results don't
+                                  depend on it                                  */
     int32_t  blocks_per_sm;    /* Poisson window blocks per SM, 0 = default (1)   */
     int32_t  sort_every;       /* macro steps between phase-space sorts of the
                                   particle storage (0 = never, default 1); the

@@ -540,12 +540,15 @@ int init32(pic_handle* h, const double* r0, const double* v0, int ptr_kind) {
 // 1.68 / 1.74, on 1024 (no register build with 512 threads) 3.31 / 2.35; FP64 1.5 10^5
 // particles 3.35 / 3.03.
 //
-// Analytic fields: per-particle windows of up to 16 warps per SM run in blocks of
-// one warp: they spread evenly, and the FP64 pipe is shared by an SM's warps (10^4
-// particles, 313 warps: 3 instead of 4 on the fullest SM).
+// Analytic fields: FP64 windows of up to 16 warps per SM run in blocks of one
+// warp: they spread evenly, and the FP64 pipe is shared by an SM's warps (10^4
+// particles, 313 warps: 3 instead of 4 on the fullest SM).  One Duffing step, periods
+// every step, blocks of 32 / 128 threads: 5000 particles 261 / 273 us, 2 10^4 308 / 420,
+// 77824 1134 / 1183.  The binary32 window has no FP64 in its loop and keeps 128: 1000
+// particles 70 / 63 us, 5000 75 / 64, from 2 10^4 on the same.
 int default_block(const pic_params* p, long long n, int sms) {
     const bool small = n <= 16ll * 32 * sms;
-    if (p->field_model != PIC_FIELD_POISSON) return small ? 32 : 128;
+    if (p->field_model != PIC_FIELD_POISSON) return small && p->precision == 0 ? 32 : 128;
     const int nodes = p->precision == 1 ? 3 : 2;
     return small && p->blocks_per_sm <= 1 && p->n_cells + 1 <= nodes * 31 * (512 >> 6) ? 512 : 1024;
 }

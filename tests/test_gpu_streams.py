@@ -82,3 +82,21 @@ def test_lines_between_the_default_shapes(n, n_cells):
         if precision == 0:
             ref = oracle.etd_step(cfg_of(p), R0, V0)
             assert bit_equal(out[0][0], ref.R) and bit_equal(out[0][1], ref.V)
+
+
+def test_analytic_window_of_the_fp32_form_takes_no_smaller_blocks():
+    # one-warp blocks share out the FP64 pipe; the binary32 window has no FP64 in
+    # its loop, and they only made a step of 5000 particles 16 % longer
+    R0, V0 = inputs.gaussian_beam(5000, seed=1)
+    kw = dict(precision=1, field_model=pic.PIC_FIELD_DUFFING, sort_every=0)
+    hs = [pic.pic_init(pic.pic_default_params(block_size=b, **kw), R0, V0) for b in (0, 128)]
+    t = [[], []]
+    for i in range(400):
+        for k in (i & 1, 1 - (i & 1)):
+            t0 = time.perf_counter()
+            pic.pic_step(hs[k], 1)
+            t[k].append(time.perf_counter() - t0)
+    default, block128 = (sorted(x[40:])[len(x[40:]) // 2] for x in t)
+    for h in hs:
+        pic.pic_destroy(h)
+    assert default < 1.05 * block128, (default, block128)
