@@ -1206,7 +1206,7 @@ int pic::poisson_with_scratch(const pic_params* p, int64_t n_particles, const in
                               double* rE_edges_dev, const pic::ScanScratch* S, void* stream) {
     int rc = check_params(p, true);
     if (rc) return rc;
-    const bool in_block = rc == PIC_OK && pic::poisson_in_block(p->n_cells);
+    const bool in_block = pic::poisson_in_block(p->n_cells);
     if (n_particles <= 0 || !Q_dev || !E_dev || !rE_edges_dev || (!S && !in_block)) return PIC_ERR_INVALID_ARG;
     if ((double)n_particles * (double)p->weight_fixed >= 4.611686018427388e18) return PIC_ERR_OVERFLOW;
     int sms = 0;

@@ -251,6 +251,10 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t parity) {
 // MODE 0: outputs to Y (pic_mlp_forward); 1, 2: the learned step's
 // correction of an FP64 / FP32 state, kept where the frozen-field energy
 // check allows it.
+// Launch bounds for 3 / 4 / 6 blocks per SM, time of a learned binary32 step outside
+// its window: 10^7 particles 2006 / 1855 / 1930 us (1990 with one thread per sample),
+// 2 10^6 477 / 442 / 466 (532), 2 10^5 133 / 129 / 133 (208).  Six leave 40 registers and
+// spill 52 bytes in MODE 2.
 template <int MODE>
 __global__ void __launch_bounds__(kInfThreads, 6) k_mlp_tc(MlpDev M, LearnedArgs A, const float* __restrict__ X,
                                                         float* __restrict__ Y, long long n) {
@@ -545,6 +549,8 @@ static cudaError_t launch_mlp_tc(const MlpDev& D, const LearnedArgs& A, int mode
 // second kernel that reloaded every record for the gradients, the two took 32
 // and 20 us and a third and fourth summed and refreshed in 11; now it is 23.5
 // and 4.9 us, without the wait for every loss: 5 steps and a gradient 551 -> 301 us.
+// Beyond 152 tiles a block of an SM takes several: the same calls with a batch of
+// 4 10^4 896 -> 493 us, 2 10^5 2.81 -> 1.19 ms, 10^6 11.2 -> 4.75 ms.
 
 constexpr int kTrThreads = 512;
 constexpr int kTrRow = kMHid + 4;    // floats per row: 16-byte rows that start 4 banks apart

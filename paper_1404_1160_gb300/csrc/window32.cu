@@ -8,11 +8,12 @@
 // trajectory: row 0 is y^n itself (the public state, Phi(0) = I), rows
 // 1..Kmax live in one array with a row stride of n rounded up to 128.  A
 // step reads row k-1 and writes row k, so the trajectory the landing
-// interpolates is the state the sweeps stream, and nothing else per
-// particle crosses a field cycle: the stage positions are recomputed from
-// z when they are needed again.  Per particle and fine step the window
-// moves 8 B (read row k-1) + 4 B (tracking word) + 8 B (write row k) in the
-// first sweep and 8 B (read row k) in the second.
+// interpolates is the state the sweeps stream; the stage positions are
+// recomputed from z when they are needed again, and the fields (e1, e3) of
+// pair 1 are carried from the second sweep of a step to the first sweep of
+// the next.  Per particle and fine step the window moves 8 B (read row k-1) +
+// 4 B (tracking word) + 8 B (e1, e3) + 8 B (write row k) in the first sweep
+// and 8 B (read row k) + 8 B (e1, e3) in the second.
 //
 // Field cycle (Poisson): as in the FP64 kernel, stages pair up (1,3) and
 // (2,4); each pair is deposited by one sweep into per-block 32-bit
@@ -20,9 +21,8 @@
 // flushed every block turns the global int64 charge into its own field table
 // of binary32 (E_j, E_{j+1} - E_j), computed in binary32 from the exact int64
 // sums and per-node constants (field_cycle32).  Two tables are kept: the
-// one of pair 1 (fields of R1, R3) and the one of pair 2 (R2, R4), so the
-// first sweep of the next step can recompute e1 and e3 instead of reading
-// them back from memory.
+// one of pair 1 (fields of R1, R3), read by the second sweep, and the one of
+// pair 2 (R2, R4), read by the first sweep of the next step.
 #include "pic_internal.h"
 #include "window_common.cuh"
 
